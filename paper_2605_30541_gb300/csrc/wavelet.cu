@@ -12,12 +12,15 @@
 // a conjugate pole pair with two zeros; gain on the first section).
 // Forward-backward filtering follows the usual zero-phase recipe: the signal
 // is extended at both ends by its odd reflection about the end samples
-// (3 (2 S + 1) samples for S sections, fewer zero coefficients aside; the
-// record must be longer than that), each
-// pass starts every section in the steady state of a constant input equal to
-// the first sample it sees, and the extension is dropped at the end. One
-// GPU thread runs the recursion in FP64 (the record is a few thousand
-// samples); the result is written in the requested precision.
+// (3 (2 S + 1) samples for S sections; the record must be longer than that),
+// each pass starts every section in the steady state of a constant input
+// equal to the first sample it sees (a band-pass section passes no constant,
+// so only the first section has a state to start from), and the extension is
+// dropped at the end. The recursion runs in FP64 as a scan over chunks of
+// the record (k_bandpass_ricker); the result is written in the requested
+// precision.
+#include <cooperative_groups.h>
+
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -76,76 +79,314 @@ std::vector<Sos> butter_bandpass(int N, double f_lo, double f_hi, double fs) {
     return s;
 }
 
-// Steady state (transposed direct form II) of each section under a unit
-// constant input to the cascade.
-std::vector<double> sos_steady(const std::vector<Sos> &s) {
-    std::vector<double> zi;
-    double scale = 1.0;  // DC gain of the sections before
-    for (const Sos &q : s) {
-        // y = b0 x + z1, z1' = b1 x - a1 y + z2, z2' = b2 x - a2 y; x = 1 constant, y = dc
-        const double dc = (q.b0 + q.b1 + q.b2) / (1.0 + q.a1 + q.a2);
-        const double z2 = q.b2 - q.a2 * dc, z1 = q.b1 - q.a1 * dc + z2;
-        zi.push_back(scale * z1);
-        zi.push_back(scale * z2);
-        scale *= dc;
-    }
-    return zi;
+constexpr int kMaxSections = 16;
+
+// ---------------------------------------------------------------- scan plan (host)
+//
+// The cascade of N sections with zero input maps its state (two values per
+// section) linearly; P[l] is that map over 2^l chunks of C samples, block
+// lower triangular (section i depends on sections j <= i only), block (i, j)
+// at i (i + 1) / 2 + j, its four values row by row.
+//
+// The poles lie close to z = 1, so an error in the map of one chunk is
+// amplified by the powers: formed in FP64 they put 1.5e-11 of the peak into
+// the wavelet (the serial recursion has 1e-13). They are therefore formed in
+// pairs of doubles (an unevaluated sum hi + lo, Dekker's and Knuth's error-free
+// sum and product) and rounded once: 7e-14 .. 1e-13, the serial recursion's.
+struct Dd {
+    double hi, lo;
+};
+Dd dd_fma(const Dd &a, const Dd &b, const Dd &c) {  // a b + c
+    const volatile double prod = a.hi * b.hi;  // volatile: the compiler may not fuse it into the sum below
+    const double p = prod, pe = std::fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi);
+    const double s = p + c.hi, t = s - p;
+    const double se = ((p - (s - t)) + (c.hi - t)) + (pe + c.lo);
+    const double h = s + se;
+    return {h, se - (h - s)};
+}
+struct Block {
+    Dd v[4];
+};
+using Tri = std::vector<Block>;  // N (N + 1) / 2 blocks
+
+Tri tri_mul(const Tri &a, const Tri &b, int N) {
+    Tri r(a.size());
+    for (int i = 0; i < N; i++)
+        for (int j = 0; j <= i; j++) {
+            Block o{};
+            for (int k = j; k <= i; k++) {
+                const Block &x = a[i * (i + 1) / 2 + k], &y = b[k * (k + 1) / 2 + j];
+                for (int p = 0; p < 2; p++)
+                    for (int q = 0; q < 2; q++)
+                        o.v[2 * p + q] = dd_fma(x.v[2 * p + 1], y.v[2 + q], dd_fma(x.v[2 * p], y.v[q], o.v[2 * p + q]));
+            }
+            r[i * (i + 1) / 2 + j] = o;
+        }
+    return r;
 }
 
-constexpr int kMaxSections = 16;
-struct Filt {
-    int nsec;
-    double b0[kMaxSections], b1[kMaxSections], b2[kMaxSections], a1[kMaxSections], a2[kMaxSections];
-    double z1[kMaxSections], z2[kMaxSections];  // steady state for a unit input
+// NS: sections the plan holds. Four is the production order; the other
+// orders share one instance that loops over its sections.
+template <int NS>
+struct Scan {
+    static constexpr int MAXS = NS ? NS : kMaxSections;
+    static constexpr int CTAS = NS ? 8 : 4;               // one cluster
+    static constexpr int WPC = NS ? 4 : 1;                // warps per CTA
+    static constexpr int WARPS = CTAS * WPC;
+    static constexpr int T = 32 * WARPS;                  // threads = chunks
+    static constexpr int LEV = NS ? 10 : 7;               // (an order-16 plan of 8 would pass 32 KB of parameters)
+    static_assert(T == 1 << LEV, "levels of the scan");
+    int nsec, C;
+    double g;
+    double a1[MAXS], a2[MAXS];
+    double P[LEV][MAXS * (MAXS + 1) / 2 * 4];
 };
 
+// map of one sample: v = 0; per section y = v + z1, z1' = z2 - a1 y, z2' = -v - a2 y, v = y
+template <int NS>
+void plan_scan(Scan<NS> &F, int C) {
+    const int N = F.nsec;
+    F.C = C;
+    Tri one((size_t)N * (N + 1) / 2), m = one;
+    for (int k = 0; k < N; k++) m[k * (k + 1) / 2 + k].v[0].hi = m[k * (k + 1) / 2 + k].v[3].hi = 1.0;
+    for (int j = 0; j < N; j++)
+        for (int q = 0; q < 2; q++) {  // column of state value q of section j
+            Dd v{0.0, 0.0};
+            for (int i = j; i < N; i++) {
+                const Dd z1{i == j && q == 0 ? 1.0 : 0.0, 0.0}, z2{i == j && q == 1 ? 1.0 : 0.0, 0.0};
+                const Dd y = dd_fma({1.0, 0.0}, v, z1);
+                Block &b = one[i * (i + 1) / 2 + j];
+                b.v[q] = dd_fma({-F.a1[i], 0.0}, y, z2);
+                b.v[2 + q] = dd_fma({-F.a2[i], 0.0}, y, {-v.hi, -v.lo});
+                v = y;
+            }
+        }
+    for (int c = C; c; c >>= 1) {
+        if (c & 1) m = tri_mul(one, m, N);
+        if (c > 1) one = tri_mul(one, one, N);
+    }
+    for (int l = 0; l < Scan<NS>::LEV; l++) {
+        for (size_t b = 0; b < m.size(); b++)
+            for (int q = 0; q < 4; q++) F.P[l][4 * b + q] = m[b].v[q].hi;
+        if (l + 1 < Scan<NS>::LEV) m = tri_mul(m, m, N);
+    }
+}
+
+// ---------------------------------------------------------------- kernel
 __device__ double ricker_at(double f0, double t) {
     const double pi = 3.14159265358979323846;
     const double a = (pi * f0 * t) * (pi * f0 * t);
     return (1.0 - 2.0 * a) * exp(-a);
 }
 
-// one pass of the cascade over x[0..n) in place, started in the steady state of x[0]
-__device__ void cascade(const Filt &F, double *x, long long n, int dir) {
-    double z1[kMaxSections], z2[kMaxSections];
-    const double x0 = dir > 0 ? x[0] : x[n - 1];
-    for (int k = 0; k < F.nsec; k++) {
-        z1[k] = F.z1[k] * x0;
-        z2[k] = F.z2[k] * x0;
+// The recursion of 2 N states over n = nt + 2 pad samples is a chain of n
+// dependent steps: one thread walked it in 22.4 ms for the production record
+// (8001 samples, order 4). Here T = 1024 threads own C = ceil(n / T)
+// consecutive samples each: every chunk runs from a zero state, the end
+// states are combined by a scan with the chunk map (within each warp, then
+// over the warps' totals, read through distributed shared memory), and every
+// chunk runs again from its true start, in place. The backward pass is
+// the same with the chunks in reverse order, on the thread's own samples, so
+// a sample never leaves its thread until it is written out. What is left is
+// the latency of the FP64 chains (about C samples four times over, 30 chunk
+// maps, C exponentials), which the four warps of each SM overlap: with one
+// warp per SM (256 chunks) the kernel took 167 us, with four 105 us. 8001
+// samples, launch and host plan included: 22.4 ms before, 0.13 ms after.
+template <int NS>
+__global__ void __launch_bounds__(32 * Scan<NS>::WPC) k_bandpass_ricker(const __grid_constant__ Scan<NS> F, int nt,
+                                                                            double dt, double f0, int pad, double scale,
+                                                                            double *work, void *out, int fp64) {
+    using S = Scan<NS>;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ double chunk[];  // C samples of each thread of the CTA (work: in global memory instead)
+    __shared__ double tot[2][S::WPC][2 * S::MAXS];  // the warps' totals of each pass
+    __shared__ double part[S::WPC];
+    const int N = NS ? NS : F.nsec;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, rank = (int)cl.block_rank(), C = F.C;
+    const int warp = rank * S::WPC + wib, t = warp * 32 + lane;
+    const long long n = nt + 2LL * pad, j0 = (long long)t * C;
+    const int m = (int)max(0LL, min((long long)C, n - j0));  // the thread's samples
+    double *const x = work ? work + t : chunk + threadIdx.x;
+    const int ld = work ? S::T : 32 * S::WPC;
+
+    // the extended record: odd reflections about the end samples
+    for (int i = 0; i < m; i++) {
+        const long long k = j0 + i - pad;
+        double v;
+        if (k < 0) v = 2.0 * ricker_at(f0, -1.0 / f0) - ricker_at(f0, -k * dt - 1.0 / f0);
+        else if (k < nt) v = ricker_at(f0, k * dt - 1.0 / f0);
+        else v = 2.0 * ricker_at(f0, (nt - 1) * dt - 1.0 / f0) - ricker_at(f0, (2LL * (nt - 1) - k) * dt - 1.0 / f0);
+        x[(long long)i * ld] = v;
     }
-    for (long long i = 0; i < n; i++) {
-        const long long j = dir > 0 ? i : n - 1 - i;
-        double v = x[j];
-        for (int k = 0; k < F.nsec; k++) {
-            const double y = F.b0[k] * v + z1[k];
-            z1[k] = F.b1[k] * v - F.a1[k] * y + z2[k];
-            z2[k] = F.b2[k] * v - F.a2[k] * y;
-            v = y;
+
+    for (int dir = 1; dir >= -1; dir -= 2) {
+        const bool first = m > 0 && (dir > 0 ? t == 0 : j0 + C >= n);
+        double z1[S::MAXS], z2[S::MAXS], s1[S::MAXS], s2[S::MAXS];
+        auto start = [&]() {  // the first chunk: the steady state of its first sample
+#pragma unroll
+            for (int k = 0; k < S::MAXS; k++) {
+                if (NS == 0 && k >= N) break;
+                z1[k] = z2[k] = k == 0 && first ? -F.g * x[(long long)(dir > 0 ? 0 : m - 1) * ld] : 0.0;
+            }
+        };
+        auto run = [&](bool store) {
+            for (int i = 0; i < m; i++) {
+                double *p = x + (long long)(dir > 0 ? i : m - 1 - i) * ld;
+                double v = F.g * *p;
+#pragma unroll
+                for (int k = 0; k < S::MAXS; k++) {
+                    if (NS == 0 && k >= N) break;
+                    const double y = v + z1[k];
+                    z1[k] = fma(-F.a1[k], y, z2[k]);
+                    z2[k] = fma(-F.a2[k], y, -v);
+                    v = y;
+                }
+                if (store) *p = v;
+            }
+        };
+        start();
+        run(false);
+        // apply the map over 2^l chunks: (s1, s2) mapped and added to (o1, o2)
+        auto map_add = [&](int l, const double *q1, const double *q2, double *o1, double *o2) {
+#pragma unroll
+            for (int i = 0; i < S::MAXS; i++) {
+                if (NS == 0 && i >= N) break;
+#pragma unroll
+                for (int j = 0; j <= i; j++) {
+                    const double *b = F.P[l] + 4 * (i * (i + 1) / 2 + j);
+                    o1[i] = fma(b[0], q1[j], fma(b[1], q2[j], o1[i]));
+                    o2[i] = fma(b[2], q1[j], fma(b[3], q2[j], o2[i]));
+                }
+            }
+        };
+        auto each = [&](auto f) {
+#pragma unroll
+            for (int k = 0; k < S::MAXS; k++) {
+                if (NS == 0 && k >= N) break;
+                f(k);
+            }
+        };
+        auto back = [&](double v, int d) {  // v of the lane d places earlier in this pass
+            return dir > 0 ? __shfl_up_sync(0xffffffffu, v, d) : __shfl_down_sync(0xffffffffu, v, d);
+        };
+        // inclusive scan of the end states over the warp's chunks, in this pass's order
+        const int place = dir > 0 ? lane : 31 - lane;
+#pragma unroll
+        for (int l = 0; l < 5; l++) {
+            each([&](int k) { s1[k] = back(z1[k], 1 << l), s2[k] = back(z2[k], 1 << l); });
+            if (place >= 1 << l) map_add(l, s1, s2, z1, z2);
         }
-        x[j] = v;
+        // scan of the warps' totals: lane j takes the j-th warp's (the others repeat the last)
+        double(*const mine)[2 * S::MAXS] = tot[dir > 0 ? 0 : 1];
+        if (place == 31) each([&](int k) { mine[wib][2 * k] = z1[k], mine[wib][2 * k + 1] = z2[k]; });
+        cl.sync();
+        const int nth = dir > 0 ? warp : S::WARPS - 1 - warp;  // the warp's place in this pass
+        double t1[S::MAXS], t2[S::MAXS];
+        {
+            const int j = min(lane, S::WARPS - 1), from_w = dir > 0 ? j : S::WARPS - 1 - j;
+            const double *const from = cl.map_shared_rank(&mine[from_w % S::WPC][0], from_w / S::WPC);
+            each([&](int k) { t1[k] = from[2 * k], t2[k] = from[2 * k + 1]; });
+        }
+#pragma unroll
+        for (int l = 5; l < S::LEV; l++) {
+            const int d = 1 << (l - 5);
+            each([&](int k) {
+                s1[k] = __shfl_up_sync(0xffffffffu, t1[k], d);
+                s2[k] = __shfl_up_sync(0xffffffffu, t2[k], d);
+            });
+            if (lane >= d && lane < S::WARPS) map_add(l, s1, s2, t1, t2);
+        }
+        // the state entering the warp's first chunk, carried over the earlier chunks of the warp
+        each([&](int k) {
+            const double v1 = __shfl_sync(0xffffffffu, t1[k], max(nth - 1, 0));
+            const double v2 = __shfl_sync(0xffffffffu, t2[k], max(nth - 1, 0));
+            t1[k] = nth > 0 ? v1 : 0.0;
+            t2[k] = nth > 0 ? v2 : 0.0;
+        });
+#pragma unroll
+        for (int l = 0; l < 5; l++)
+            if (place >> l & 1) {
+                each([&](int k) { s1[k] = s2[k] = 0.0; });
+                map_add(l, t1, t2, s1, s2);
+                each([&](int k) { t1[k] = s1[k], t2[k] = s2[k]; });
+            }
+        // each chunk's true start: the state after the chunk before it
+        each([&](int k) { s1[k] = back(z1[k], 1), s2[k] = back(z2[k], 1); });
+        start();
+        if (!first)
+            each([&](int k) {
+                z1[k] = t1[k] + (place > 0 ? s1[k] : 0.0);
+                z2[k] = t2[k] + (place > 0 ? s2[k] : 0.0);
+            });
+        run(true);
     }
+
+    // l2 norm over the record, in a fixed order
+    double ss = 0.0;
+    for (int i = 0; i < m; i++) {
+        const long long k = j0 + i - pad;
+        const double v = x[(long long)i * ld];
+        if (k >= 0 && k < nt) ss += v * v;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (lane == 0) part[wib] = ss;
+    cl.sync();
+    ss = 0.0;
+    for (int r = 0; r < S::WARPS; r++) ss += *cl.map_shared_rank(&part[r % S::WPC], r / S::WPC);
+    const double c = ss > 0.0 ? scale / sqrt(ss) : 0.0;
+    // the CTA's samples [32 WPC C rank, 32 WPC C (rank + 1)), written in order
+    double *const x0 = x - threadIdx.x;
+    for (int i = threadIdx.x; i < 32 * S::WPC * C; i += 32 * S::WPC) {
+        const long long k = 32LL * S::WPC * C * rank + i - pad;
+        const int h = i / C;
+        if (k < 0 || k >= nt) continue;
+        const double v = c * x0[(long long)(i - h * C) * ld + h];
+        if (fp64) static_cast<double *>(out)[k] = v;
+        else static_cast<float *>(out)[k] = (float)v;
+    }
+    cl.sync();  // no CTA leaves while another reads its shared memory
 }
 
-__global__ void k_bandpass_ricker(const Filt F, int nt, double dt, double f0, int pad, double scale, double *work,
-                                  void *out, int fp64) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+// Most chunk bytes kept in shared memory; longer records (over 200 000
+// samples at order 4) keep their samples in a global workspace.
+constexpr size_t kChunkSmem = 200 * 1024;
+
+template <int NS>
+cudaError_t launch_bandpass(const std::vector<Sos> &s, int nt, double dt, double f0, int pad, double scale, void *out,
+                            int fp64, double **work, cudaStream_t st) {
+    using S = Scan<NS>;
+    S F{};
+    F.nsec = (int)s.size();
+    F.g = s[0].b0;
+    for (int k = 0; k < F.nsec; k++) {
+        F.a1[k] = s[k].a1;
+        F.a2[k] = s[k].a2;
+    }
     const long long n = nt + 2LL * pad;
-    for (int i = 0; i < nt; i++) work[pad + i] = ricker_at(f0, i * dt - 1.0 / f0);
-    const double first = work[pad], last = work[pad + nt - 1];
-    for (int i = 1; i <= pad; i++) {  // odd reflections about the end samples
-        work[pad - i] = 2.0 * first - work[pad + i];
-        work[pad + nt - 1 + i] = 2.0 * last - work[pad + nt - 1 - i];
+    plan_scan<NS>(F, (int)((n + S::T - 1) / S::T));
+    size_t smem = (size_t)F.C * 32 * S::WPC * sizeof(double);
+    cudaError_t e = cudaSuccess;
+    if (smem > kChunkSmem) {
+        smem = 0;
+        e = cudaMalloc(work, (size_t)F.C * S::T * sizeof(double));
+    } else {
+        e = cudaFuncSetAttribute(k_bandpass_ricker<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChunkSmem);
     }
-    cascade(F, work, n, +1);
-    cascade(F, work, n, -1);
-    double ss = 0.0;
-    for (int i = 0; i < nt; i++) ss += work[pad + i] * work[pad + i];
-    const double c = ss > 0.0 ? scale / sqrt(ss) : 0.0;
-    for (int i = 0; i < nt; i++) {
-        const double v = c * work[pad + i];
-        if (fp64) static_cast<double *>(out)[i] = v;
-        else static_cast<float *>(out)[i] = (float)v;
-    }
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(S::CTAS);
+    cfg.blockDim = dim3(32 * S::WPC);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S::CTAS;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_bandpass_ricker<NS>, F, nt, dt, f0, pad, scale, *work, out, fp64);
 }
 
 }  // namespace
@@ -165,26 +406,7 @@ extern "C" sim_status sim_wavelet_bandpass(int nt, double dt, double f0, double 
         set_thread_error("sim_wavelet_bandpass: the band-pass has real poles (band too wide for this design)");
         return SIM_ERR_ARG;
     }
-    const std::vector<double> zi = sos_steady(s);
-    Filt F{};
-    F.nsec = (int)s.size();
-    for (int k = 0; k < F.nsec; k++) {
-        F.b0[k] = s[k].b0;
-        F.b1[k] = s[k].b1;
-        F.b2[k] = s[k].b2;
-        F.a1[k] = s[k].a1;
-        F.a2[k] = s[k].a2;
-        F.z1[k] = zi[2 * k];
-        F.z2[k] = zi[2 * k + 1];
-    }
-    // extension length: 3 (2 S + 1) less the sections with a zero last
-    // coefficient in both numerator and denominator, capped by the record
-    int zb = 0, za = 0;
-    for (const Sos &q : s) {
-        zb += q.b2 == 0.0;
-        za += q.a2 == 0.0;
-    }
-    const int pad = 3 * (2 * F.nsec + 1 - std::min(zb, za));
+    const int pad = 3 * (2 * (int)s.size() + 1);
     if (nt <= pad) {
         set_thread_error("sim_wavelet_bandpass: the record must be longer than the reflection at its ends");
         return SIM_ERR_ARG;
@@ -196,12 +418,13 @@ extern "C" sim_status sim_wavelet_bandpass(int nt, double dt, double f0, double 
     const size_t esz = precision == SIM_FP64 ? 8 : 4;
     double *work = nullptr;
     void *dout = out;
-    cudaError_t e = cudaMalloc(&work, sizeof(double) * (nt + 2 * (size_t)pad));
-    if (e == cudaSuccess && !dev_out) e = cudaMalloc(&dout, esz * nt);
+    cudaError_t e = cudaSuccess;
+    if (!dev_out) e = cudaMalloc(&dout, esz * nt);
     if (e == cudaSuccess) {
-        k_bandpass_ricker<<<1, 1, 0, st>>>(F, nt, dt, f0, pad, std::sqrt((f_hi - f_lo) / 24.0), work, dout,
-                                           precision == SIM_FP64);
-        e = cudaGetLastError();
+        const double scale = std::sqrt((f_hi - f_lo) / 24.0);
+        const int fp64 = precision == SIM_FP64;
+        e = order == 4 ? launch_bandpass<4>(s, nt, dt, f0, pad, scale, dout, fp64, &work, st)
+                       : launch_bandpass<0>(s, nt, dt, f0, pad, scale, dout, fp64, &work, st);
     }
     if (e == cudaSuccess && !dev_out) e = cudaMemcpyAsync(out, dout, esz * nt, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
