@@ -268,6 +268,7 @@ struct sim_s {
     int tuned_nshots = 0;  // shot count the tile shape was tuned for (0: not yet)
     bool use_march = false; // the autotuner's choice: row march rather than the tiled step kernel
     Pt3 *src3 = nullptr, *rec3 = nullptr;  // 3D point tables
+    Add3 add3{};                           // 3D CPML addends of one step
     int *rdone = nullptr;                  // resident path: step counter per (shot, subdomain)
     Inj3 *src3g = nullptr, *res3g = nullptr;  // 3D adjoint: injection groups (sources, residuals)
     InjE3 *src3e = nullptr, *res3e = nullptr;
@@ -281,8 +282,7 @@ struct sim_s {
     int march_nwarps = 0, march_nitems = 0;
     unsigned *mctr = nullptr;              // row march: per-step item counters
     int last_path = 0, last_rows = 0;      // see sim_info
-    int zchunk = 0;                        // z-march chunk of the 3D kernel (planes per CTA)
-    int zvariant = kZMarchTma;             // z-march staging (cp.async or TMA), see autotune3d
+    ZShape zshape;                         // z-march variant, tile and chunk, see autotune3d
     int batch_sched = 0, batch_tile = 0;   // schedule and tile of the last batch forward (as sim_info)
     void *pbuf3 = nullptr;                 // two-step row march: third and fourth pressure fields (max_shots shots each)
     int tuned3d = 0;                       // shot count the 3D launch shape was tuned for
@@ -860,57 +860,54 @@ int zchunk_for(const sim_s *s, int nshots) {
     return (g.NZ + chunks - 1) / chunks;
 }
 
-// One forward-type 3D step without its point work: the CPML passes of the
-// absorbing axes around the z-march (the x axis first, as the march that
-// folds the x strips in adds their term first), skipping the x pass when the
-// march takes it over. slot: the record mode's imaging term (else NULL).
-cudaError_t step3d_core(const sim_s *s, const StepArgs<float> &a, int n, int variant, int zc, int nshots,
-                        cudaStream_t st, bool pdl, int mode, float *slot) {
-    const bool cpml = s->d.bc == SIM_BC_CPML;
-    const bool on[3] = {s->psi[0][0] != nullptr, s->psi[1][0] != nullptr, s->psi[2][0] != nullptr};
-    const bool fx = cpml && zmarch_folds_x(a, variant, mode);
-    const int order[3] = {2, 0, 1};
-    cudaError_t e = cudaSuccess;
-    for (int ax : order)
-        if (e == cudaSuccess && cpml && on[ax] && !(ax == 2 && fx)) e = launch_cpml3d(a, n, ax, 0, nshots, st);
-    if (e == cudaSuccess) e = launch_step3d(a, n, variant, zc, nshots, st, pdl, mode, slot, nullptr);
-    for (int ax : order)
-        if (e == cudaSuccess && cpml && on[ax] && !(ax == 2 && fx)) e = launch_cpml3d(a, n, ax, 1, nshots, st, slot);
+// One forward-type 3D step without its injection and snapshot: the CPML
+// addends (and, with rec, the receivers' samples of p^n), then the z-march
+// that adds them. slot: the record mode's imaging term (else NULL).
+cudaError_t step3d_core(const sim_s *s, const StepArgs<float> &a, int n, const ZShape &zs, int nshots, cudaStream_t st,
+                        bool pdl, int mode, float *slot, const Pt3 *rec = nullptr, int nrec = 0) {
+    cudaError_t e = launch_cpml3d(a, s->add3, n, rec, nrec, nshots, st, pdl);
+    if (e == cudaSuccess) e = launch_step3d(a, n, zs, nshots, st, pdl, mode, s->add3, slot, nullptr);
     return e;
 }
 
-// 3D launch shape: the z-march variant (per-thread cp.async or TMA staging)
-// and the planes per CTA (z chunk: fewer, longer columns re-read less halo;
-// more, shorter ones fill the GPU). The first forward or gradient call for a
-// shot count times a few steps of each candidate on this GPU with CUDA
-// events (on zeroed fields, before the run resets them) and keeps the
-// fastest. GSIM_ZMARCH=async|tma|tma-plain|tma-loop|tma-loop-fold|tma-loop3 fixes the
-// variant, GSIM_ZCHUNK the chunk;
-// GSIM_AUTOTUNE=0 takes the TMA variant with the default chunk untimed.
+// 3D launch shape: the z-march's tile and the planes per CTA (z chunk: fewer,
+// longer columns re-read less halo; more, shorter ones fill the GPU). The
+// first forward or gradient call for a shot count times a few steps of each
+// candidate on this GPU with CUDA events (on zeroed fields, before the run
+// resets them) and keeps the fastest. Candidates are the TMA march unrolled by
+// 3 in its three tiles; the other variants were never more than 1% ahead on
+// the volumes measured and run when asked for:
+// GSIM_ZMARCH=async|tma|tma-plain|tma-loop|tma-loop-fold|tma-loop3 fixes the
+// variant (tma-loop3: 128 columns, tma-loop3-64 and tma-loop3-32), GSIM_ZCHUNK
+// the chunk; GSIM_AUTOTUNE=0 takes the 128-column tile with the default chunk
+// untimed.
 sim_status autotune3d(sim_t s, int nshots) {
     if (s->tuned3d == nshots) return SIM_OK;
     s->tuned3d = nshots;
     const int base = zchunk_for(s, nshots), NZ = s->g.NZ;
-    std::vector<int> variants = {kZMarchTmaLoop3, kZMarchTmaPlain, kZMarchTmaLoop, kZMarchTma, kZMarchTmaFoldLoop,
-                                 kZMarchAsync};
-    if (s->d.bc != SIM_BC_CPML)  // no x strips to fold
-        variants = {kZMarchTmaLoop3, kZMarchTmaPlain, kZMarchTmaLoop, kZMarchAsync};
-    static const char *const names[7] = {"", "async", "tma", "tma-plain", "tma-loop", "tma-loop-fold", "tma-loop3"};
+    struct Shape {
+        int variant, tile;
+        const char *name;
+    };
+    static const Shape all[] = {{kZMarchTmaLoop3, 128, "tma-loop3"}, {kZMarchTmaLoop3, 64, "tma-loop3-64"},
+                                {kZMarchTmaLoop3, 32, "tma-loop3-32"}, {kZMarchAsync, 128, "async"}, {kZMarchTma, 128, "tma"},
+                                {kZMarchTmaPlain, 128, "tma-plain"}, {kZMarchTmaLoop, 128, "tma-loop"},
+                                {kZMarchTmaFoldLoop, 128, "tma-loop-fold"}};
+    std::vector<Shape> shapes(all, all + 3);
     if (const char *f = getenv("GSIM_ZMARCH"))
-        for (int v = 1; v <= 6; v++)
-            if (!strcmp(f, names[v])) variants = {v};
-    s->zvariant = variants[0];
-    s->zchunk = base;
+        for (const Shape &v : all)
+            if (!strcmp(f, v.name)) shapes = {v};
+    s->zshape = ZShape{shapes[0].variant, shapes[0].tile, base};
     const char *at = getenv("GSIM_AUTOTUNE");
     if (at && at[0] == '0') return SIM_OK;
     std::vector<int> chunks = {base};
-    for (int c : {NZ, (NZ + 1) / 2, (NZ + 3) / 4, (NZ + 7) / 8})
-        if (c >= 16 && std::find(chunks.begin(), chunks.end(), c) == chunks.end()) chunks.push_back(c);
+    for (int c : {NZ, (NZ + 1) / 2, (NZ + 3) / 4, (NZ + 7) / 8, (NZ + 15) / 16})
+        if (c >= 8 && std::find(chunks.begin(), chunks.end(), c) == chunks.end()) chunks.push_back(c);
     if (const char *f = getenv("GSIM_ZCHUNK")) {  // a fixed chunk (tests)
         chunks = {std::max(1, std::min(NZ, atoi(f)))};
-        s->zchunk = chunks[0];
+        s->zshape.chunk = chunks[0];
     }
-    if (variants.size() == 1 && chunks.size() == 1) return SIM_OK;
+    if (shapes.size() == 1 && chunks.size() == 1) return SIM_OK;
     if (sim_status r = reset_state(s, nshots)) return r;
     StepArgs<float> a = step_args<float>(s);
     cudaEvent_t e0, e1;
@@ -921,12 +918,13 @@ sim_status autotune3d(sim_t s, int nshots) {
     }
     float best = 1e30f;
     cudaError_t e = cudaSuccess;
-    for (int v : variants)
+    for (const Shape &v : shapes)
         for (int zc : chunks) {
+            const ZShape zs{v.variant, v.tile, zc};
             const int warm = 1, timed = 3;
             for (int n = 0; n < warm + timed && e == cudaSuccess; n++) {
                 if (n == warm) e = cudaEventRecord(e0, s->st);
-                if (e == cudaSuccess) e = step3d_core(s, a, n, v, zc, nshots, s->st, false, kModeForward, nullptr);
+                if (e == cudaSuccess) e = step3d_core(s, a, n, zs, nshots, s->st, false, kModeForward, nullptr);
             }
             if (e == cudaSuccess) e = cudaEventRecord(e1, s->st);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
@@ -935,11 +933,10 @@ sim_status autotune3d(sim_t s, int nshots) {
             if (e != cudaSuccess) break;
             if (getenv("GSIM_TUNE_LOG"))
                 fprintf(stderr, "[gsim autotune] 3D %dx%dx%d shots %d %s chunk %d: %.1f us/step\n", s->g.NZ, s->g.NY,
-                        s->g.NX, nshots, names[v], zc, 1e3 * ms / timed);
+                        s->g.NX, nshots, v.name, zc, 1e3 * ms / timed);
             if (ms < best) {
                 best = ms;
-                s->zvariant = v;
-                s->zchunk = zc;
+                s->zshape = zs;
             }
         }
     cudaEventDestroy(e0);
@@ -1011,14 +1008,16 @@ sim_status forward3d(sim_t s, int nshots, const void *wav, const double *src_pos
     a.sample = nrec > 0 && gdev != nullptr;
     const bool has_src = !src.empty(), has_snap = io.snaps != nullptr;
     const Pt3 *s3 = s->src3, *r3 = s->rec3;
-    return run_graph(s, ((long long)nshots << 8) | (3 << 2) | 2, [&](cudaStream_t st) {
+    const long long key = ((long long)nrec << 32) | ((long long)nshots << 8) | (a.sample << 7) | (has_src << 6) |
+                          (has_snap << 5) | (3 << 2) | 2;
+    return run_graph(s, key, [&](cudaStream_t st) {
         cudaError_t e = cudaSuccess;
         for (int n = 0; n < d.nt && e == cudaSuccess; n++) {
             const StepTime t = step_time(s, a, n, kModeForward, nullptr, nullptr);
             if (has_snap && t.snap_k >= 0) e = launch_snap3d(a, t, d.snap_fp16, nshots, st);
-            if (e == cudaSuccess && a.sample) e = launch_sample3d(a, t, r3, nrec, nshots, st);
             if (e == cudaSuccess)
-                e = step3d_core(s, a, n, s->zvariant, s->zchunk, nshots, st, false, kModeForward, nullptr);
+                e = step3d_core(s, a, n, s->zshape, nshots, st, s->use_graphs, kModeForward, nullptr,
+                                a.sample ? r3 : nullptr, nrec);
             if (e == cudaSuccess && has_src) e = launch_inject3d(a, t, s3, nshots, st);
         }
         return e;
@@ -1924,7 +1923,7 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
 
     if (sim_status r = autotune3d(s, nshots)) return r;
     const AdjPlan &P = s->plan;
-    const int zc = s->zchunk, zv = s->zvariant;
+    const ZShape zs = s->zshape;
     const CkLayout ckl = ck_layout(s, ckpt_fp16);
     StepArgs<float> a = step_args<float>(s);
     a.sample = 1;
@@ -1939,6 +1938,7 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
     float *Gs = static_cast<float *>(s->Gbuf);
     const size_t qstride = q_slot_bytes(s, ckpt_fp16);
     const int nsg = (int)sg.size(), nrg = (int)rg.size();
+    const bool fused = cpml && cpml3d_adjoint_fits(a);
     const Pt3 *r3 = s->rec3;
     const long long gkey = ((long long)nshots << 40) ^ ((long long)nrec << 16) ^ ((long long)ckpt_fp16 << 3) ^
                            ((long long)o.vjp << 5) ^ 6;
@@ -1946,10 +1946,8 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
             cudaError_t e = reset_state_on(s, nshots, st);
             if (e != cudaSuccess) return e;
             auto step = [&](const StepArgs<float> &A, int n, int mode, float *slot, bool sample) {
-                cudaError_t e2 = cudaSuccess;
-                if (sample) e2 = launch_sample3d(A, step_time(s, A, n, kModeForward, nullptr, nullptr), r3, nrec,
-                                                 nshots, st);
-                if (e2 == cudaSuccess) e2 = step3d_core(s, A, n, zv, zc, nshots, st, true, mode, slot);
+                cudaError_t e2 = step3d_core(s, A, n, zs, nshots, st, s->use_graphs, mode, slot,
+                                             sample ? r3 : nullptr, nrec);
                 if (e2 == cudaSuccess)
                     e2 = launch_inj3d(A, n, n, s->src3g, nsg, s->src3e, 0, nshots, mode, slot, nullptr, st);
                 return e2;
@@ -1962,22 +1960,27 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
                 [&](int k, int i) {
                     float *slot = slot_of(i);
                     const int n = d.nt - k;
-                    cudaError_t e2 = launch_step3d(adj, n, zv, zc, nshots, st, true, kModeAdjoint, slot, Gs);
+                    // nu^k, mu^k from u^{k+1} and their bracket, which the march adds as
+                    // c [.] to u^k (strip layouts it does not take: after the march)
+                    const bool terms = cpml && k <= d.nt - 1;
+                    CpmlAdjArgs<float> ca{};
+                    ca.u = adj.pbuf[(d.nt - k) & 1];
+                    for (int ax = 0; ax < 3; ax++) {
+                        ca.nu[ax][0] = static_cast<float *>(s->cnu[ax][0]);
+                        ca.nu[ax][1] = static_cast<float *>(s->cnu[ax][1]);
+                        ca.mu[ax] = static_cast<float *>(s->cmu[ax]);
+                    }
+                    ca.uo = adj.pbuf[(n + 1) & 1];
+                    ca.q = slot;
+                    ca.G = Gs;
+                    cudaError_t e2 = cudaSuccess;
+                    if (terms && fused) e2 = launch_cpml3d_adjoint(a, s->add3, ca, nshots, st, s->use_graphs);
+                    if (e2 == cudaSuccess)
+                        e2 = launch_step3d(adj, n, zs, nshots, st, s->use_graphs, kModeAdjoint,
+                                           terms && fused ? s->add3 : Add3{}, slot, Gs);
                     if (e2 == cudaSuccess)
                         e2 = launch_inj3d(adj, n, k, s->res3g, nrg, s->res3e, 1, nshots, kModeAdjoint, slot, Gs, st);
-                    if (e2 == cudaSuccess && cpml && k <= d.nt - 1) {  // nu^k, mu^k from u^{k+1}; c [.] into u^k
-                        CpmlAdjArgs<float> ca{};
-                        ca.u = adj.pbuf[(d.nt - k) & 1];
-                        for (int ax = 0; ax < 3; ax++) {
-                            ca.nu[ax][0] = static_cast<float *>(s->cnu[ax][0]);
-                            ca.nu[ax][1] = static_cast<float *>(s->cnu[ax][1]);
-                            ca.mu[ax] = static_cast<float *>(s->cmu[ax]);
-                        }
-                        ca.uo = adj.pbuf[(n + 1) & 1];
-                        ca.q = slot;
-                        ca.G = Gs;
-                        e2 = launch_cpml_adjoint<float>(a, ca, k & 1, nshots, st);
-                    }
+                    if (e2 == cudaSuccess && terms && !fused) e2 = launch_cpml_adjoint<float>(a, ca, k & 1, nshots, st);
                     return e2;
                 },
                 [&](int k, int n, bool store) { return checkpoint<float>(s, a, ckl, k, n, store, ckpt_fp16, nshots, st); },
@@ -2881,6 +2884,16 @@ sim_status sim_create(const sim_desc *din, const void *vel, void *cuda_stream, s
     }
     if (rc == SIM_OK && d.ndim == 3) {
         rc = s->cuda(configure_step3d(), "kernel configuration");
+        if (rc == SIM_OK) rc = s->cuda(configure_cpml3d(), "kernel configuration");
+        const bool on[3] = {s->psi[0][0] != nullptr, s->psi[1][0] != nullptr, s->psi[2][0] != nullptr};
+        long long ne[3];
+        s->add3 = add3_layout(g, on, ne);
+        for (int ax = 0; ax < 3; ax++) {
+            if (!on[ax] || ne[ax] == 0) continue;
+            s->add3.a[ax] = static_cast<float *>(A(ne[ax] * ms * sizeof(float)));
+            // rows held at zero and cells past the grid are never written
+            if (rc == SIM_OK) rc = s->cuda(cudaMemsetAsync(s->add3.a[ax], 0, ne[ax] * ms * sizeof(float), s->st), "initial clear");
+        }
         s->src3 = static_cast<Pt3 *>(A(sizeof(Pt3) * ms));
         s->rec3 = static_cast<Pt3 *>(A(sizeof(Pt3) * std::max(1, d.max_rec)));
     }
@@ -3005,8 +3018,8 @@ sim_status sim_get_info(sim_t s, sim_info *out) {
     out->batch_sched = s->batch_sched;
     out->batch_tile = s->batch_tile;
     if (s->g.ndim == 3 && s->tuned3d) {
-        out->z_variant = s->zvariant;
-        out->z_chunk = s->zchunk;
+        out->z_variant = s->zshape.variant;
+        out->z_chunk = s->zshape.chunk;
     }
     if (s->adj_ready) {
         out->adj_levels = s->plan.levels;

@@ -263,28 +263,53 @@ cudaError_t configure_march2x();
 int march2x_warps_per_sm();
 cudaError_t launch_march2x(const TBArgs &b, const TBPass &t, int nwarps, cudaStream_t st);
 
-// 3D launchers (fwd3d.cu). Per step: snapshot, sample, CPML psi, z-march
-// update, CPML zeta + addend, source injection.
+// 3D step (fwd3d.cu, cpml3d.cu). Per step: snapshot, CPML addends and
+// receiver samples, z-march update with the addends, source injection.
 // z-march variants: kZMarchAsync stages each plane by per-thread 16-byte
-// cp.async copies; kZMarchTma by three bulk tensor copies (TMA) per plane
-// issued by one thread, completion on mbarriers, and folds the x-strip CPML
-// in where it can; kZMarchTmaPlain is the TMA march leaving the x strips to
-// their own pass; the two ...Loop variants are the same without unrolling
-// the plane loop (smaller code, the register queue shifted by moves);
-// kZMarchTmaLoop3 unrolls it by 3 (the queue rotated by moves once per three
-// planes). All take z chunks of `zchunk` planes per CTA.
+// cp.async copies; the others by three bulk tensor copies (TMA) per plane
+// issued by one thread, completion on mbarriers, with the plane loop
+// unrolled by 9 (kZMarchTma, kZMarchTmaPlain), not at all (kZMarchTmaLoop,
+// kZMarchTmaFoldLoop) or by 3 (kZMarchTmaLoop3). kZMarchTma and
+// kZMarchTmaFoldLoop are names of earlier variants that formed the x-strip
+// CPML in the march itself; they run the same kernels now. All take z chunks
+// of `zchunk` planes per CTA.
 enum { kZMarchAsync = 1, kZMarchTma = 2, kZMarchTmaPlain = 3, kZMarchTmaLoop = 4, kZMarchTmaFoldLoop = 5, kZMarchTmaLoop3 = 6 };
+// CPML addends of the 3D step: per axis a compact array over the cells of its
+// strips widened by 4 (z: slots of whole (y, x) planes; y: slots of x rows in
+// every plane; x: the float4s from the strip ends of every row), one after
+// another for the shots.
+struct Add3 {
+    float *a[3];        // z, y, x; NULL: axis absent
+    long long st[3];    // elements per shot
+    int zl, zh, nzw;    // planes z < zl (slot z) and z >= zh (slot zl + z - zh)
+    int yl, yh, nyw;    // rows y alike
+    int xl, xs, xe, nxw; // float4s starting in [0, xl) and [xs, xe); nxw floats per row
+};
+Add3 add3_layout(const Geom &g, const bool on[3], long long elems[3]);
+struct Pt3;
+cudaError_t configure_cpml3d();
+// psi^n, zeta^n and the addends of every absorbing axis, and (rec) the
+// receivers' samples of p^n into the gather
+cudaError_t launch_cpml3d(const StepArgs<float> &a, const Add3 &D, int n, const Pt3 *rec, int nrec, int nshots,
+                          cudaStream_t st, bool pdl);
+// the adjoint sweep's multipliers (in place: parity 0 of nu) and brackets, for
+// strip layouts that fit; the z-march of the sweep adds the brackets
+bool cpml3d_adjoint_fits(const StepArgs<float> &a);
+cudaError_t launch_cpml3d_adjoint(const StepArgs<float> &a, const Add3 &D, const CpmlAdjArgs<float> &c, int nshots,
+                                  cudaStream_t st, bool pdl);
 struct Tma3 {
-    CUtensorMap ph;  // p (both parities, all shots): 136 x 16 x 1 boxes, the plane with its x / y halo
-    CUtensorMap po;  // the same buffers: 128 x 8 x 1 boxes, a tile's own cells
-    CUtensorMap c;   // c = (v dt / h)^2: 128 x 8 x 1 boxes
+    CUtensorMap ph;  // p (both parities, all shots): one plane of a tile with its 4-cell x / y halo
+    CUtensorMap po;  // the same buffers: one plane of a tile's own cells
+    CUtensorMap c;   // c = (v dt / h)^2: likewise
 };
 cudaError_t configure_step3d();
-// The TMA march of the forward and record modes takes over the x-strip CPML
-// pass when the widened strips lie inside the first / last x tile.
-bool zmarch_folds_x(const StepArgs<float> &a, int variant, int mode);
-cudaError_t launch_step3d(const StepArgs<float> &a, int n, int variant, int zchunk, int nshots, cudaStream_t st,
-                          bool pdl, int mode = kModeForward, float *qs = nullptr, float *Gs = nullptr);
+struct ZShape {
+    int variant = kZMarchTmaLoop3;
+    int tile = 128;  // columns of a CTA's tile (kZMarchTmaLoop3: 128, 64 or 32 of 1024 cells)
+    int chunk = 0;   // planes per CTA
+};
+cudaError_t launch_step3d(const StepArgs<float> &a, int n, const ZShape &zs, int nshots, cudaStream_t st, bool pdl, int mode,
+                          const Add3 &D, float *qs = nullptr, float *Gs = nullptr);
 // 3D point injection grouped by target cell (the adjoint path): group =
 // cell offset within a field, entry range, shot (-1: the same for every
 // shot, the launch's y index).
@@ -299,10 +324,6 @@ struct InjE3 {
 };
 cudaError_t launch_inj3d(const StepArgs<float> &a, int n, int row, const Inj3 *grp, int ngrp, const InjE3 *ent,
                          int kind, int nshots, int mode, float *qs, float *Gs, cudaStream_t st);
-cudaError_t launch_cpml3d(const StepArgs<float> &a, int n, int ax, int phase, int nshots, cudaStream_t st,
-                          float *qs = nullptr);
-cudaError_t launch_sample3d(const StepArgs<float> &a, const StepTime &t, const void *rec, int nrec, int nshots,
-                            cudaStream_t st);
 cudaError_t launch_inject3d(const StepArgs<float> &a, const StepTime &t, const void *src, int nshots,
                             cudaStream_t st);
 cudaError_t launch_snap3d(const StepArgs<float> &a, const StepTime &t, int fp16, int nshots, cudaStream_t st);
