@@ -6,16 +6,16 @@
 // cells in a register queue, so p^n is read from memory once per cell for the
 // z-derivative. The planes with their radius-4 x/y halo are staged into a
 // shared-memory ring ahead of use: by per-thread cp.async copies (k_step3d)
-// or by tensor-memory-accelerator copies that one thread issues (k_step3d_tma,
-// the autotuner's usual pick). The update is the leapfrog step with the
+// or by tensor-memory-accelerator copies that one thread issues (k_step3d_tma). The update is the leapfrog step with the
 // centred sponge term (Eq. cerjan_pde), the free-surface plane z = 0 held at
 // zero with an odd mirror above it (Eq. free_surface), and no boundary
 // arithmetic outside absorbing tiles.
 //
 // The CPML addends of each axis and the receiver samples come from one launch
-// before the march (cpml3d.cu); point injection of the source and snapshot
-// output are side kernels on small parts of the grid.
+// before the march (cpml3d.cu), the march injects the point sources; snapshot
+// output and the adjoint sweep's injection are side kernels.
 #include <cfloat>
+#include <climits>
 
 #include <cudaTypedefs.h>
 
@@ -76,29 +76,24 @@ __device__ __forceinline__ Cells4 cells4(const float4 &L, const float4 &C, const
     }
     return o;
 }
+__device__ __forceinline__ void cp16(void *smem, const void *gmem) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-// 16-byte copy that writes zeros (reads nothing) when v is false
-__device__ __forceinline__ void cp16z(void *smem, const void *gmem, bool v) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)),
-                 "l"(gmem), "r"(v ? 16 : 0)
-                 : "memory");
-}
-
 // The CPML addends (cpml3d.cu) of one thread's row of four cells (gy, gx0 ..)
 // in a tile at (x0, y0): p^{n+1} += c (addend) axis by axis, in the order x,
 // z, y; the addend is part of the Laplacian in the record mode's imaging
-// term. Tiles and planes away from the strips test two block-uniform flags.
+// term. Tiles and planes away from the strips test block-uniform flags.
 struct AddRows {
-    const Add3 &D;
     const float *x, *y, *z;  // the row's addends at plane 0 (z: at slot 0); NULL: none
-    const float *base;       // some valid address for a copy that reads nothing
     long long px, py, pz;    // plane strides
+    int zl, zh;              // planes < zl and >= zh take z addends (none: every plane lies between)
     bool xy;                 // the tile meets an x or y strip
-    __device__ __forceinline__ AddRows(const Add3 &D_, const Geom &g, int shot, int gy, int gx0, int x0, int tx, int y0,
-                                                       int ty)
-        : D(D_), x(nullptr), y(nullptr), z(nullptr), base(D_.a[0] ? D_.a[0] : D_.a[1] ? D_.a[1] : D_.a[2]) {
+    __device__ __forceinline__ AddRows(const Add3 &D, const Geom &g, int shot, int gy, int gx0, int x0, int tx, int y0, int ty)
+        : x(nullptr), y(nullptr), z(nullptr) {
         const bool row = gy < g.NY && gx0 < g.NX;
         px = (long long)g.NY * D.nxw;
         py = (long long)D.nyw * g.P;
@@ -108,33 +103,42 @@ struct AddRows {
         if (D.a[1] && row && (gy < D.yl || gy >= D.yh))
             y = D.a[1] + shot * D.st[1] + (long long)(gy < D.yl ? gy : D.yl + gy - D.yh) * g.P + gx0;
         if (D.a[0] && row) z = D.a[0] + shot * D.st[0] + (long long)gy * g.P + gx0;
+        zl = D.a[0] ? D.zl : 0;
+        zh = D.a[0] ? D.zh : INT_MAX;
         xy = (D.a[2] && (x0 < D.xl || x0 + tx > D.xs)) || (D.a[1] && (y0 < D.yl || y0 + ty > D.yh));
     }
-    __device__ __forceinline__ bool any(int pl) const { return xy || (z && (pl < D.zl || pl >= D.zh)); }
-    // the row's three addends at plane pl into the thread's slots s, s + step, s + 2 step
-    // (zeros where there is none)
-    __device__ __forceinline__ void fetch(int pl, float4 *s, int step) const {
-        const bool zin = z && (pl < D.zl || pl >= D.zh);
-        cp16z(s, x ? x + pl * px : base, x != nullptr);
-        cp16z(s + step, zin ? z + (pl < D.zl ? pl : D.zl + pl - D.zh) * pz : base, zin);
-        cp16z(s + 2 * step, y ? y + pl * py : base, y != nullptr);
-    }
+    __device__ __forceinline__ bool zin(int pl) const { return pl < zl || pl >= zh; }
+    __device__ __forceinline__ const float *zrow(int pl) const { return z + (pl < zl ? pl : zl + pl - zh) * pz; }
     __device__ __forceinline__ static void add(const float4 v, const float4 &c, float *res, float *qk) {
         res[0] = __fmaf_rn(c.x, v.x, res[0]), qk[0] -= v.x;
         res[1] = __fmaf_rn(c.y, v.y, res[1]), qk[1] -= v.y;
         res[2] = __fmaf_rn(c.z, v.z, res[2]), qk[2] -= v.z;
         res[3] = __fmaf_rn(c.w, v.w, res[3]), qk[3] -= v.w;
     }
+    // straight from memory
     __device__ __forceinline__ void apply(int pl, const float4 &c, float *res, float *qk) const {
-        if (xy && x) add(ld4g(x + pl * px), c, res, qk);
-        if (z && (pl < D.zl || pl >= D.zh)) add(ld4g(z + (pl < D.zl ? pl : D.zl + pl - D.zh) * pz), c, res, qk);
-        if (xy && y) add(ld4g(y + pl * py), c, res, qk);
+        if (x) add(ld4g(x + pl * px), c, res, qk);
+        if (z && zin(pl)) add(ld4g(zrow(pl)), c, res, qk);
+        if (y) add(ld4g(y + pl * py), c, res, qk);
     }
 };
-__device__ __forceinline__ void cp16(void *smem, const void *gmem) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gmem) : "memory");
+// One corner c of a shot's point source into p^{n+1} (already updated); with
+// qs (record mode), its share E d - h^2 s of the imaging term.
+__device__ __noinline__ void inject3(const StepArgs<float> &A, const Pt3 &P, int c, int shot, int n, int row, float *qs) {
+    const Geom &g = A.g;
+    const long long o = P.cell[c], so = (long long)shot * g.fstride + o;
+    float es = 0.f;
+    if (A.bc == SIM_BC_SPONGE) {
+        const long long r = o - g.org, PP = (long long)g.PY * g.P;
+        const int z = (int)(r / PP), y = (int)((r % PP) / g.P), x = (int)(r % g.P);
+        es = A.E[0][z] + A.E[1][y] + A.E[2][x];
+    }
+    const float sum = P.w[c] * static_cast<const float *>(A.io->wavelet)[row], chv = A.ch[o];
+    const float d = chv * A.src_scale * sum / (1.f + chv * es);
+    A.pbuf[(n + 1) & 1][so] += d;
+    if (qs) qs[so] += es * d - A.src_scale * sum;
 }
+
 // Staged planes in flight: while plane z is computed, planes z+1 .. z+4 are
 // ready or arriving and plane z+5 is being requested. A ring slot holds the
 // plane's p^n with its x/y halo, and p^{n-1} and c of the CTA's own cells;
@@ -303,23 +307,24 @@ __global__ void __launch_bounds__(NTH, 2) k_step3d(const StepArgs<float> A, cons
 // A plane is 96 pair-arithmetic instructions per float4, and the march used to
 // spend 250 more on three waits with 64-bit counters, generic addresses, votes
 // and the ring bookkeeping (352 warp instructions per 128 cells, 112 us at
-// 170 x 227 x 273 x 2 shots); one group per plane, offsets instead of
-// pointers and no vote leave 303 and 94 us with the CPML addends
-// read in the march.
+// 170 x 227 x 273 x 2 shots). One group per plane, rings of 8 and 4 slots with
+// the loop unrolled by 4 (slot addresses are constants but for the halves of
+// the halo ring, which swap), offsets instead of pointers and no vote leave 264
+// and 88 us, the CPML addends' read included.
 //
 // A wait that gives up (bounded) marks its thread, which waits no more and
 // goes on with whatever its slots hold; the leader then stages no more, waits
 // (bounded) for the copies in flight, and the kernel sets kFlagTimeout.
 //
-// Tiles of TW x TY cells, TW = 128, 64 or 32 and TW TY = 1024: a warp takes
-// 128 / TW rows. The wide one reads whole 512-byte rows but stages 2.1 cells
-// per cell (136 x 16 for 128 x 8), the others 1.7 and 1.6; on a ragged grid the
-// narrower ones also waste fewer lanes past its edge. The autotuner times them.
+// Tiles of TW x TY cells, TW = 64 or 32 and TW TY = 1024: a warp takes 128 / TW
+// rows. They stage 1.7 and 1.6 cells per cell (a 128 x 8 tile: 2.1; it was
+// slower by 3% at 172 x 152 rows, 5% at 1060 x 1060 and 12% at 273 x 227) and
+// waste few lanes past a ragged edge. The autotuner times both.
+constexpr int AHEAD = 3, NSH = AHEAD + 5, NSO = AHEAD + 1;  // planes z .. z + 4 + AHEAD; z .. z + AHEAD
+static_assert(NSH == 8 && NSO == 4, "the plane loop is unrolled by 4");
 template <int TW>
 struct Tile3 {
     static constexpr int RPW = TX / TW, TY = NW * RPW, SW = TW + 8;
-    static constexpr int AHEAD = TW == 128 ? 2 : 3;
-    static constexpr int NSH = AHEAD + 5, NSO = AHEAD + 1;  // planes z - 0 .. z + 4 + AHEAD; z .. z + AHEAD
     static constexpr int HALO = (TY + 8) * SW * 4, OWN = TY * TW * 4, OSLOT = 2 * OWN;
     static constexpr int ADD = 2 * 3 * NTH * 16;            // CPML addends of two planes, a slot per thread and axis
     static constexpr int OWN0 = NSH * HALO, ADD0 = OWN0 + NSO * OSLOT, BAR0 = ADD0 + ADD;
@@ -365,16 +370,14 @@ __device__ __forceinline__ void tma_load3(unsigned dst, const CUtensorMap *m, in
         : "memory");
 }
 
-// UN = 9: the plane loop unrolled by the queue's length (the queue rotates by
-// renaming); UN = 1: a plain loop that shifts the queue (smaller code); UN =
-// 3: unrolled by three, the queue rotated by three after each block.
-template <int MODE, int UN, int TW>
+// src, row: the shots' point sources and the wavelet row injected (src NULL: none)
+template <int MODE, int TW>
 __global__ void __launch_bounds__(NTH, 2) k_step3d_tma(const StepArgs<float> A, const __grid_constant__ Tma3 M,
                                                        const int n, const int zchunk, const int ms, const Add3 D,
-                                                       float *qs, float *Gs, const int spin) {
+                                                       const Pt3 *src, const int row, float *qs, float *Gs,
+                                                       const int spin) {
     using T3 = Tile3<TW>;
-    constexpr int TY = T3::TY, SW = T3::SW, NSH = T3::NSH, NSO = T3::NSO, AHEAD = T3::AHEAD, HALO = T3::HALO,
-                  OSLOT = T3::OSLOT, OWN = T3::OWN;
+    constexpr int TY = T3::TY, SW = T3::SW, HALO = T3::HALO, OSLOT = T3::OSLOT, OWN = T3::OWN;
     extern __shared__ __align__(128) unsigned char sm_t[];
     const unsigned s0 = smem_u32(sm_t), bar0 = s0 + T3::BAR0;  // barriers: one per own slot, then the first planes'
 
@@ -425,13 +428,30 @@ __global__ void __launch_bounds__(NTH, 2) k_step3d_tma(const StepArgs<float> A, 
         for (int k = 0; k < 4; k++)
             tma_load4(s0 + k * HALO, &M.ph, tx - 4, ty - 4, zb + k + kGhost, wcur, bar0 + 8 * NSO);
         for (int k = 0; k < AHEAD; k++)
-            if (zb + k < ze) stage(zb + k, (k + 4) % NSH, k);
+            if (zb + k < ze) stage(zb + k, k + 4, k);
     }
-    if (add.any(zb)) add.fetch(zb, aslot + (zb & 1) * 3 * NTH, NTH);
-    cp_commit();
+    // CPML addends of the coming plane into the thread's slots (x, y, z of two
+    // planes); slots of an axis the thread has no addend of stay zero
+    const float *ax = add.x + zb * add.px, *ay = add.y + zb * add.py;
+    bool zn = false;  // the coming plane takes z addends
+    auto fetch = [&](int z, int half) {
+        float4 *const v = aslot + half * 3 * NTH;
+        if (add.xy) {
+            if (add.x) cp16(v, ax);
+            if (add.y) cp16(v + NTH, ay);
+            ax += add.px;
+            ay += add.py;
+        }
+        zn = add.zin(z);
+        if (zn && add.z) cp16(v + 2 * NTH, add.zrow(z));
+        cp_commit();
+    };
+    for (int k = 0; k < 6; k++)
+        if (!(k % 3 == 0 ? add.x : k % 3 == 1 ? add.y : add.z)) aslot[k * NTH] = make_float4(0.f, 0.f, 0.f, 0.f);
+    fetch(zb, 0);
 
     // register queue of this thread's cells: plane z + m lives in q[(j + m + 4) % 9]
-    // at unrolled step j of a block of 9 planes
+    // at step j of a block of 4 planes
     const unsigned rowo = ((w + 4) * SW + 4 + lx) * 4;  // the thread's float4 in a halo slot
     float4 q[9];
     {
@@ -453,36 +473,37 @@ __global__ void __launch_bounds__(NTH, 2) k_step3d_tma(const StepArgs<float> A, 
 #pragma unroll
     for (int k = 0; k < 4; k++) q[4 + k] = *reinterpret_cast<const float4 *>(sm_t + k * HALO + rowo);
 
-    // halo slots of planes z - 1, z and z + 4, own slot of planes z - 1 and z, its phase
-    int kp = NSH - 1, kz = 0, k4 = 4 % NSH, op = NSO - 1, ko = 0;
-    unsigned par = 0;
+    unsigned ha = 0, hb = 4;  // first halo slots of planes zz .. zz + 3 and zz + 4 .. zz + 7
+    unsigned par = 0;         // phase of the own slots
     float *out = A.pbuf[(n + 1) & 1] + sh + own0 + (long long)zb * PP;
     long long orow = sh + own0 + (long long)zb * PP;  // record / adjoint: this thread's float4 of plane z
-    for (int zz = zb; zz < ze; zz += UN) {
+    for (int zz = zb; zz < ze; zz += 4) {
+        const unsigned char *const ra = sm_t + ha * HALO + rowo, *const rb = sm_t + hb * HALO + rowo;
 #pragma unroll
-        for (int j = 0; j < UN; j++) {
+        for (int j = 0; j < 4; j++) {
             const int z = zz + j;
             if (z >= ze) break;
-            if (tid == 0 && z + AHEAD < ze && zbad == ze) stage(z + AHEAD, kp, op);  // into the slots plane z - 1 used
+            // into the slots plane z - 1 used
+            if (tid == 0 && z + AHEAD < ze && zbad == ze) stage(z + AHEAD, j == 0 ? hb + 3 : ha + j - 1, (j + 3) % NSO);
             // the next plane's addends, a plane ahead of their use (the tiles at the
             // strips would wait on their latency every plane)
-            if (z + 1 < ze && add.any(z + 1)) add.fetch(z + 1, aslot + ((z + 1) & 1) * 3 * NTH, NTH);
-            cp_commit();
+            const bool zadd = zn;
+            if (z + 1 < ze) fetch(z + 1, (j + 1) & 1);
+            else cp_commit();
             float4 qa = make_float4(0, 0, 0, 0), ga = qa;
             if (MODE == kModeAdjoint && live) {
                 qa = ld4g(qs + orow);
                 ga = ld4g(Gs + orow);
             }
-            if (zbad == ze && !mbar_wait(bar0 + 8 * ko, par, spin)) zbad = z;
-            const unsigned char *const cur = sm_t + kz * HALO + rowo, *const own = sm_t + T3::OWN0 + ko * OSLOT + 16 * tid;
-            q[(j + 8) % 9] = *reinterpret_cast<const float4 *>(sm_t + k4 * HALO + rowo);
+            if (zbad == ze && !mbar_wait(bar0 + 8 * j, par, spin)) zbad = z;
+            const unsigned char *const cur = ra + j * HALO, *const own = sm_t + T3::OWN0 + j * OSLOT + 16 * tid;
+            q[(j + 8) % 9] = *reinterpret_cast<const float4 *>(rb + j * HALO);
             const float ez = spg ? __ldg(A.E[0] + z) : 0.f;
-            const float *row = reinterpret_cast<const float *>(cur);
-            const float4 L = *reinterpret_cast<const float4 *>(row - 4), C = *reinterpret_cast<const float4 *>(row),
-                         R = *reinterpret_cast<const float4 *>(row + 4);
+            const float *pr = reinterpret_cast<const float *>(cur);
+            const float4 L = ld4g(pr - 4), C = ld4g(pr), R = ld4g(pr + 4);
             float4 yv[9];
 #pragma unroll
-            for (int m = 0; m < 9; m++) yv[m] = m == 4 ? C : *reinterpret_cast<const float4 *>(row + (m - 4) * SW);
+            for (int m = 0; m < 9; m++) yv[m] = m == 4 ? C : ld4g(pr + (m - 4) * SW);
             const float4 pp4 = *reinterpret_cast<const float4 *>(own), ch4 = *reinterpret_cast<const float4 *>(own + OWN);
             const Cells4 cu = cells4(L, C, R, yv, q[j % 9], q[(j + 1) % 9], q[(j + 2) % 9], q[(j + 3) % 9], q[(j + 5) % 9],
                                      q[(j + 6) % 9], q[(j + 7) % 9], q[(j + 8) % 9], pp4, ch4, spg, ez + Ey, Ex4);
@@ -493,12 +514,12 @@ __global__ void __launch_bounds__(NTH, 2) k_step3d_tma(const StepArgs<float> A, 
                 const float es = spg ? ez + Ey + lane4(Ex4, k) : 0.f;
                 qk[k] = es * (res[k] - lane4(pp4, k)) - cu.rhs[k];
             }
-            if (add.any(z)) {
+            if (add.xy | zadd) {
                 cp_wait<1>();
-                const float4 *v = aslot + (z & 1) * 3 * NTH;
-                AddRows::add(v[0], ch4, res, qk);
-                AddRows::add(v[NTH], ch4, res, qk);
-                AddRows::add(v[2 * NTH], ch4, res, qk);
+                const float4 *const v = aslot + (j & 1) * 3 * NTH;
+                if (add.xy) AddRows::add(v[0], ch4, res, qk);
+                if (zadd) AddRows::add(v[2 * NTH], ch4, res, qk);
+                if (add.xy) AddRows::add(v[NTH], ch4, res, qk);
             }
             if (xedge) {
 #pragma unroll
@@ -517,26 +538,21 @@ __global__ void __launch_bounds__(NTH, 2) k_step3d_tma(const StepArgs<float> A, 
                     *reinterpret_cast<float4 *>(Gs + orow) = ga;
                 }
             }
-            if (UN == 1) {
-#pragma unroll
-                for (int k = 0; k < 8; k++) q[k] = q[k + 1];
-            }
             out += PP;
             if (MODE != kModeForward) orow += PP;
-            kp = kz;
-            if (++kz == NSH) kz = 0;
-            if (++k4 == NSH) k4 = 0;
-            op = ko;
-            if (++ko == NSO) ko = 0, par ^= 1;
             __syncthreads();  // every thread is done with plane z's slots before they are restaged
         }
-        if (UN == 3) {  // plane zz + 3 + m back to q[(m + 4) % 9] for the next block
-            const float4 t0 = q[0], t1 = q[1];
+        // plane zz + 4 + m back to q[(m + 4) % 9] for the next block
+        const float4 t0 = q[0], t1 = q[1], t2 = q[2];
 #pragma unroll
-            for (int k = 0; k < 6; k++) q[k] = q[k + 3];
-            q[6] = t0;
-            q[7] = t1;
-        }
+        for (int k = 0; k < 5; k++) q[k] = q[k + 4];
+        q[5] = t0;
+        q[6] = t1;
+        q[7] = t2;
+        const unsigned t = ha;
+        ha = hb;
+        hb = t;
+        par ^= 1;
     }
     cp_wait<0>();  // no copy outlives the thread
     // a leader that waited for every group knows that its copies have landed;
@@ -551,51 +567,38 @@ __global__ void __launch_bounds__(NTH, 2) k_step3d_tma(const StepArgs<float> A, 
         }
     }
     __syncthreads();
+    // the source corners among the cells this CTA has written
+    if (MODE != kModeAdjoint && src && tid < 8 && src[shot].cell[tid] >= 0) {
+        const long long o = src[shot].cell[tid], r = o - g.org;
+        const int z = (int)(r / PP), y = (int)(r % PP / g.P), x = (int)(r % g.P);
+        if (x >= x0 && x < x0 + TW && y >= y0 && y < y0 + TY && z >= zb && z < ze)
+            inject3(A, src[shot], tid, shot, n, row, MODE == kModeRecord ? qs : nullptr);
+    }
 }
 
 // ---------------------------------------------------------------- points (3D)
 
-// p^{n+1} += c w[n] weight / h / (1 + a) at each source corner (one thread per shot and corner)
-__global__ void k_inject3d(const StepArgs<float> A, const StepTime t, const Pt3 *src, int nshots) {
+// point sources into p^{n+1} (one thread per shot and corner). The TMA march
+// injects on its own.
+__global__ void k_inject3d(const StepArgs<float> A, const int n, const int row, const Pt3 *src, int nshots, float *qs) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 8 * nshots || t.inj_row < 0) return;
-    const int shot = i >> 3, c = i & 7;
-    const Pt3 P = src[shot];
-    const long long o = P.cell[c];
-    if (o < 0) return;
-    const Geom &g = A.g;
-    float *pn = A.pbuf[(t.n + 1) & 1] + (long long)shot * g.fstride;
-    const float w = static_cast<const float *>(A.io->wavelet)[t.inj_row];
-    float a = 0.f;
-    if (A.bc == SIM_BC_SPONGE) {
-        const long long r = o - g.org;
-        const long long PP = (long long)g.PY * g.P;
-        const int z = (int)(r / PP), y = (int)((r % PP) / g.P), x = (int)(r % g.P);
-        a = A.ch[o] * (A.E[0][z] + A.E[1][y] + A.E[2][x]);
-    }
-    pn[o] += A.ch[o] * A.src_scale * P.w[c] * w / (1.f + a);
+    if (i < 8 * nshots && src[i >> 3].cell[i & 7] >= 0) inject3(A, src[i >> 3], i & 7, i >> 3, n, row, qs);
 }
 
-// Point injection into p^{n+1} by target cell (deterministic order of the
-// entries of a cell): value = wavelet[row] (kind 0) or the residual of
-// receiver pt at row (kind 1). With the record / adjoint modes the cell's
-// imaging term gets the source's share / its G the injected part of u^{n+1}.
+// The adjoint sweep's injection: residuals into u^{n+1} by target cell
+// (deterministic order of the entries of a cell), the cell's G gaining the
+// injected part.
 __global__ void k_inj3d(const StepArgs<float> A, const int n, const int row, const Inj3 *grp, const int ngrp,
-                        const InjE3 *ent, const int kind, const int mode, float *qs, float *Gs) {
+                        const InjE3 *ent, const float *qs, float *Gs) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= ngrp || row < 0 || row >= A.nt) return;
     const Inj3 G = grp[i];
-    if (G.shot >= 0 && blockIdx.y != 0) return;
-    const int shot = G.shot >= 0 ? G.shot : blockIdx.y;
+    const int shot = blockIdx.y;
     const Geom &g = A.g;
     const SimIO *io = A.io;
+    const float *r = static_cast<const float *>(io->resid) + ((long long)shot * A.nt + row) * io->nrec;
     float sum = 0.f;
-    for (int e = G.e0; e < G.e1; e++) {
-        const InjE3 E = ent[e];
-        const float val = kind == 0 ? static_cast<const float *>(io->wavelet)[row]
-                                    : static_cast<const float *>(io->resid)[((long long)shot * A.nt + row) * io->nrec + E.pt];
-        sum += E.w * val;
-    }
+    for (int e = G.e0; e < G.e1; e++) sum += ent[e].w * r[ent[e].pt];
     const long long o = G.cell, so = (long long)shot * g.fstride + o;
     float es = 0.f;
     if (A.bc == SIM_BC_SPONGE) {
@@ -606,8 +609,7 @@ __global__ void k_inj3d(const StepArgs<float> A, const int n, const int row, con
     const float chv = A.ch[o];
     const float d = chv * A.src_scale * sum / (1.f + chv * es);
     A.pbuf[(n + 1) & 1][so] += d;
-    if (mode == kModeRecord) qs[so] += es * d - A.src_scale * sum;
-    if (mode == kModeAdjoint) Gs[so] += d * qs[so];
+    Gs[so] += d * qs[so];
 }
 
 // interior of p^n into the snapshot stack (FP32), or its max |p| (FP16 pass 1)
@@ -685,21 +687,18 @@ cudaError_t make_maps(const StepArgs<float> &a, int tw, Tma3 &m) {
     return q == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int UN, int TW>
+template <int TW>
 cudaError_t configure_tma() {
     cudaError_t e = cudaSuccess;
-    for (auto k : {k_step3d_tma<kModeForward, UN, TW>, k_step3d_tma<kModeRecord, UN, TW>, k_step3d_tma<kModeAdjoint, UN, TW>})
+    for (auto k : {k_step3d_tma<kModeForward, TW>, k_step3d_tma<kModeRecord, TW>, k_step3d_tma<kModeAdjoint, TW>})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile3<TW>::SMEM);
     return e;
 }
 
 cudaError_t configure_step3d() {
-    cudaError_t e = configure_tma<9, 128>();
-    if (e == cudaSuccess) e = configure_tma<1, 128>();
-    if (e == cudaSuccess) e = configure_tma<3, 128>();
-    if (e == cudaSuccess) e = configure_tma<3, 64>();
-    if (e == cudaSuccess) e = configure_tma<3, 32>();
+    cudaError_t e = configure_tma<64>();
+    if (e == cudaSuccess) e = configure_tma<32>();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_step3d<1, kModeForward>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem3d<1>());
@@ -719,9 +718,9 @@ cudaError_t launch_step3d_mode(cudaLaunchConfig_t &cfg, const StepArgs<float> &a
     return cudaLaunchKernelEx(&cfg, k_step3d<RY, MODE>, a, n, zchunk, D, qs, Gs);
 }
 
-template <int UN, int TW>
+template <int TW>
 cudaError_t launch_tma(cudaLaunchConfig_t &cfg, const StepArgs<float> &a, int n, int zchunk, int mode, const Add3 &D,
-                       float *qs, float *Gs) {
+                       const Pt3 *src, int row, float *qs, float *Gs) {
     Tma3 m;
     if (cudaError_t e = make_maps(a, TW, m)) return e;
     cfg.gridDim.x = (a.g.NX + TW - 1) / TW;
@@ -730,15 +729,16 @@ cudaError_t launch_tma(cudaLaunchConfig_t &cfg, const StepArgs<float> &a, int n,
     const int ms = (int)((a.pbuf[1] - a.pbuf[0]) / a.g.fstride);
     const int spin = 1 << 22;
     if (mode == kModeRecord)
-        return cudaLaunchKernelEx(&cfg, k_step3d_tma<kModeRecord, UN, TW>, a, m, n, zchunk, ms, D, qs, Gs, spin);
+        return cudaLaunchKernelEx(&cfg, k_step3d_tma<kModeRecord, TW>, a, m, n, zchunk, ms, D, src, row, qs, Gs, spin);
     if (mode == kModeAdjoint)
-        return cudaLaunchKernelEx(&cfg, k_step3d_tma<kModeAdjoint, UN, TW>, a, m, n, zchunk, ms, D, qs, Gs, spin);
-    return cudaLaunchKernelEx(&cfg, k_step3d_tma<kModeForward, UN, TW>, a, m, n, zchunk, ms, D, qs, Gs, spin);
+        return cudaLaunchKernelEx(&cfg, k_step3d_tma<kModeAdjoint, TW>, a, m, n, zchunk, ms, D, src, row, qs, Gs, spin);
+    return cudaLaunchKernelEx(&cfg, k_step3d_tma<kModeForward, TW>, a, m, n, zchunk, ms, D, src, row, qs, Gs, spin);
 }
 
 cudaError_t launch_step3d(const StepArgs<float> &a, int n, const ZShape &zs, int nshots, cudaStream_t st, bool pdl, int mode,
-                          const Add3 &D, float *qs, float *Gs) {
+                          const Add3 &D, const Pt3 *src, int row, float *qs, float *Gs) {
     const int zchunk = zs.chunk, nchunk = (a.g.NZ + zchunk - 1) / zchunk;
+    if (row < 0 || row >= a.nt) src = nullptr;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.ntx, (a.g.NY + NW - 1) / NW, nchunk * nshots);
     cfg.blockDim = dim3(NTH);
@@ -748,34 +748,21 @@ cudaError_t launch_step3d(const StepArgs<float> &a, int n, const ZShape &zs, int
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    switch (zs.variant) {
-        case kZMarchTma:
-        case kZMarchTmaPlain: return launch_tma<9, 128>(cfg, a, n, zchunk, mode, D, qs, Gs);
-        case kZMarchTmaLoop:
-        case kZMarchTmaFoldLoop: return launch_tma<1, 128>(cfg, a, n, zchunk, mode, D, qs, Gs);
-        case kZMarchTmaLoop3:
-            if (zs.tile == 64) return launch_tma<3, 64>(cfg, a, n, zchunk, mode, D, qs, Gs);
-            if (zs.tile == 32) return launch_tma<3, 32>(cfg, a, n, zchunk, mode, D, qs, Gs);
-            return launch_tma<3, 128>(cfg, a, n, zchunk, mode, D, qs, Gs);
-        default: break;
-    }
-    if (zs.variant != kZMarchAsync) return cudaErrorInvalidValue;
-    if (mode == kModeRecord) return launch_step3d_mode<1, kModeRecord>(cfg, a, n, zchunk, D, qs, Gs);
-    if (mode == kModeAdjoint) return launch_step3d_mode<1, kModeAdjoint>(cfg, a, n, zchunk, D, qs, Gs);
-    return launch_step3d_mode<1, kModeForward>(cfg, a, n, zchunk, D, qs, Gs);
-}
-
-cudaError_t launch_inj3d(const StepArgs<float> &a, int n, int row, const Inj3 *grp, int ngrp, const InjE3 *ent,
-                         int kind, int nshots, int mode, float *qs, float *Gs, cudaStream_t st) {
-    if (ngrp <= 0) return cudaSuccess;
-    k_inj3d<<<dim3((ngrp + 127) / 128, nshots), 128, 0, st>>>(a, n, row, grp, ngrp, ent, kind, mode, qs, Gs);
+    if (zs.variant != kZMarchAsync)
+        return zs.tile == 32 ? launch_tma<32>(cfg, a, n, zchunk, mode, D, src, row, qs, Gs)
+                             : launch_tma<64>(cfg, a, n, zchunk, mode, D, src, row, qs, Gs);
+    cudaError_t e = mode == kModeRecord    ? launch_step3d_mode<1, kModeRecord>(cfg, a, n, zchunk, D, qs, Gs)
+                    : mode == kModeAdjoint ? launch_step3d_mode<1, kModeAdjoint>(cfg, a, n, zchunk, D, qs, Gs)
+                                           : launch_step3d_mode<1, kModeForward>(cfg, a, n, zchunk, D, qs, Gs);
+    if (e != cudaSuccess || !src) return e;
+    k_inject3d<<<(8 * nshots + 63) / 64, 64, 0, st>>>(a, n, row, src, nshots, mode == kModeRecord ? qs : nullptr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_inject3d(const StepArgs<float> &a, const StepTime &t, const void *src, int nshots,
-                            cudaStream_t st) {
-    if (!src || nshots <= 0) return cudaSuccess;
-    k_inject3d<<<(8 * nshots + 63) / 64, 64, 0, st>>>(a, t, static_cast<const Pt3 *>(src), nshots);
+cudaError_t launch_inj3d(const StepArgs<float> &a, int n, int row, const Inj3 *grp, int ngrp, const InjE3 *ent,
+                         int nshots, const float *qs, float *Gs, cudaStream_t st) {
+    if (ngrp <= 0) return cudaSuccess;
+    k_inj3d<<<dim3((ngrp + 127) / 128, nshots), 128, 0, st>>>(a, n, row, grp, ngrp, ent, qs, Gs);
     return cudaGetLastError();
 }
 

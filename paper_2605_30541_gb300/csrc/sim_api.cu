@@ -270,8 +270,8 @@ struct sim_s {
     Pt3 *src3 = nullptr, *rec3 = nullptr;  // 3D point tables
     Add3 add3{};                           // 3D CPML addends of one step
     int *rdone = nullptr;                  // resident path: step counter per (shot, subdomain)
-    Inj3 *src3g = nullptr, *res3g = nullptr;  // 3D adjoint: injection groups (sources, residuals)
-    InjE3 *src3e = nullptr, *res3e = nullptr;
+    Inj3 *res3g = nullptr;                 // 3D adjoint: injection groups of the residuals
+    InjE3 *res3e = nullptr;
     RTile *rtiles = nullptr;               // resident path: subdomain descriptors
     const TileMap *tmap = nullptr;         // set while lists are built for a non-uniform tiling
     std::list<std::pair<int, ResidentPlan>> rplans;  // per shot count
@@ -860,13 +860,14 @@ int zchunk_for(const sim_s *s, int nshots) {
     return (g.NZ + chunks - 1) / chunks;
 }
 
-// One forward-type 3D step without its injection and snapshot: the CPML
-// addends (and, with rec, the receivers' samples of p^n), then the z-march
-// that adds them. slot: the record mode's imaging term (else NULL).
+// One forward-type 3D step without its snapshot: the CPML addends (and, with
+// rec, the receivers' samples of p^n), then the z-march that adds them and
+// injects the sources (src, wavelet row n). slot: the record mode's imaging
+// term (else NULL).
 cudaError_t step3d_core(const sim_s *s, const StepArgs<float> &a, int n, const ZShape &zs, int nshots, cudaStream_t st,
-                        bool pdl, int mode, float *slot, const Pt3 *rec = nullptr, int nrec = 0) {
+                        bool pdl, int mode, float *slot, const Pt3 *src, const Pt3 *rec = nullptr, int nrec = 0) {
     cudaError_t e = launch_cpml3d(a, s->add3, n, rec, nrec, nshots, st, pdl);
-    if (e == cudaSuccess) e = launch_step3d(a, n, zs, nshots, st, pdl, mode, s->add3, slot, nullptr);
+    if (e == cudaSuccess) e = launch_step3d(a, n, zs, nshots, st, pdl, mode, s->add3, src, n, slot, nullptr);
     return e;
 }
 
@@ -874,13 +875,10 @@ cudaError_t step3d_core(const sim_s *s, const StepArgs<float> &a, int n, const Z
 // longer columns re-read less halo; more, shorter ones fill the GPU). The
 // first forward or gradient call for a shot count times a few steps of each
 // candidate on this GPU with CUDA events (on zeroed fields, before the run
-// resets them) and keeps the fastest. Candidates are the TMA march unrolled by
-// 3 in its three tiles; the other variants were never more than 1% ahead on
-// the volumes measured and run when asked for:
-// GSIM_ZMARCH=async|tma|tma-plain|tma-loop|tma-loop-fold|tma-loop3 fixes the
-// variant (tma-loop3: 128 columns, tma-loop3-64 and tma-loop3-32), GSIM_ZCHUNK
-// the chunk; GSIM_AUTOTUNE=0 takes the 128-column tile with the default chunk
-// untimed.
+// resets them) and keeps the fastest. GSIM_ZMARCH fixes the variant (async;
+// tma-64 and tma-32; tma, tma-plain, tma-loop, tma-loop-fold and tma-loop3 are
+// names of earlier forms of the TMA march and mean tma-64), GSIM_ZCHUNK the
+// chunk; GSIM_AUTOTUNE=0 takes the 64-column tile with the default chunk untimed.
 sim_status autotune3d(sim_t s, int nshots) {
     if (s->tuned3d == nshots) return SIM_OK;
     s->tuned3d = nshots;
@@ -889,11 +887,10 @@ sim_status autotune3d(sim_t s, int nshots) {
         int variant, tile;
         const char *name;
     };
-    static const Shape all[] = {{kZMarchTmaLoop3, 128, "tma-loop3"}, {kZMarchTmaLoop3, 64, "tma-loop3-64"},
-                                {kZMarchTmaLoop3, 32, "tma-loop3-32"}, {kZMarchAsync, 128, "async"}, {kZMarchTma, 128, "tma"},
-                                {kZMarchTmaPlain, 128, "tma-plain"}, {kZMarchTmaLoop, 128, "tma-loop"},
-                                {kZMarchTmaFoldLoop, 128, "tma-loop-fold"}};
-    std::vector<Shape> shapes(all, all + 3);
+    static const Shape all[] = {{kZMarchTma, 64, "tma-64"}, {kZMarchTma, 32, "tma-32"}, {kZMarchAsync, 128, "async"},
+                                {kZMarchTma, 64, "tma"}, {kZMarchTma, 64, "tma-plain"}, {kZMarchTma, 64, "tma-loop"},
+                                {kZMarchTma, 64, "tma-loop-fold"}, {kZMarchTma, 64, "tma-loop3"}};
+    std::vector<Shape> shapes(all, all + 2);
     if (const char *f = getenv("GSIM_ZMARCH"))
         for (const Shape &v : all)
             if (!strcmp(f, v.name)) shapes = {v};
@@ -924,7 +921,7 @@ sim_status autotune3d(sim_t s, int nshots) {
             const int warm = 1, timed = 3;
             for (int n = 0; n < warm + timed && e == cudaSuccess; n++) {
                 if (n == warm) e = cudaEventRecord(e0, s->st);
-                if (e == cudaSuccess) e = step3d_core(s, a, n, zs, nshots, s->st, false, kModeForward, nullptr);
+                if (e == cudaSuccess) e = step3d_core(s, a, n, zs, nshots, s->st, false, kModeForward, nullptr, nullptr);
             }
             if (e == cudaSuccess) e = cudaEventRecord(e1, s->st);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
@@ -1017,8 +1014,7 @@ sim_status forward3d(sim_t s, int nshots, const void *wav, const double *src_pos
             if (has_snap && t.snap_k >= 0) e = launch_snap3d(a, t, d.snap_fp16, nshots, st);
             if (e == cudaSuccess)
                 e = step3d_core(s, a, n, s->zshape, nshots, st, s->use_graphs, kModeForward, nullptr,
-                                a.sample ? r3 : nullptr, nrec);
-            if (e == cudaSuccess && has_src) e = launch_inject3d(a, t, s3, nshots, st);
+                                has_src ? s3 : nullptr, a.sample ? r3 : nullptr, nrec);
         }
         return e;
     });
@@ -1613,8 +1609,8 @@ void free_adjoint(sim_t s) {
     s->inj2_start = nullptr;
     s->inj2_grp = nullptr;
     s->inj2_ent = nullptr;
-    s->src3g = s->res3g = nullptr;
-    s->src3e = s->res3e = nullptr;
+    s->res3g = nullptr;
+    s->res3e = nullptr;
 }
 
 // Zero the CPML multipliers (both parities) and the 2D bracket of `nshots`
@@ -1680,8 +1676,6 @@ sim_status ensure_adjoint(sim_t s, int fp16) {
     s->inj2_grp = static_cast<InjGroup *>(A(s->cap_grp * sizeof(InjGroup)));
     s->inj2_ent = A(s->cap_grp * sizeof(InjEntryT<double>));
     if (g.ndim == 3) {
-        s->src3g = static_cast<Inj3 *>(A(8 * (size_t)ms * sizeof(Inj3)));
-        s->src3e = static_cast<InjE3 *>(A(8 * (size_t)ms * sizeof(InjE3)));
         s->res3g = static_cast<Inj3 *>(A(8 * (size_t)std::max(1, d.max_rec) * sizeof(Inj3)));
         s->res3e = static_cast<InjE3 *>(A(8 * (size_t)std::max(1, d.max_rec) * sizeof(InjE3)));
     }
@@ -1762,31 +1756,28 @@ cudaError_t emit_gradient(const AdjPlan &P, int nt, F1 fwd_first, F2 fwd, F3 rec
     return e;
 }
 
-// Injection groups of 3D points (adjoint path): every corner with a non-zero
-// weight off the free surface, grouped by target cell in a fixed order;
-// shot >= 0 gives each point's groups to that shot, -1 shares them.
-void group3d(const std::vector<Pt3> &pts, bool per_shot, std::vector<Inj3> &grp, std::vector<InjE3> &ent) {
+// Injection groups of 3D points (the adjoint sweep's residuals): every corner
+// with a non-zero weight off the free surface, grouped by target cell in a
+// fixed order.
+void group3d(const std::vector<Pt3> &pts, std::vector<Inj3> &grp, std::vector<InjE3> &ent) {
     struct C {
         long long cell;
-        int shot, pt;
+        int pt;
         float w;
     };
     std::vector<C> cs;
     for (size_t q = 0; q < pts.size(); q++)
         for (int k = 0; k < 8; k++)
-            if (pts[q].cell[k] >= 0) cs.push_back({pts[q].cell[k], per_shot ? (int)q : -1, (int)q, pts[q].w[k]});
-    std::stable_sort(cs.begin(), cs.end(), [](const C &a, const C &b) {
-        return a.shot != b.shot ? a.shot < b.shot : a.cell < b.cell;
-    });
+            if (pts[q].cell[k] >= 0) cs.push_back({pts[q].cell[k], (int)q, pts[q].w[k]});
+    std::stable_sort(cs.begin(), cs.end(), [](const C &a, const C &b) { return a.cell < b.cell; });
     grp.clear();
     ent.clear();
     for (size_t i = 0; i < cs.size();) {
         Inj3 G{};
         G.cell = cs[i].cell;
-        G.shot = cs[i].shot;
         G.e0 = (int)ent.size();
         size_t j = i;
-        while (j < cs.size() && cs[j].cell == cs[i].cell && cs[j].shot == cs[i].shot) {
+        while (j < cs.size() && cs[j].cell == cs[i].cell) {
             ent.push_back(InjE3{cs[j].pt, cs[j].w});
             j++;
         }
@@ -1901,15 +1892,15 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
     if (sim_status r = points3d(s, nshots, src_pos, src, true, "source")) return r;
     if (sim_status r = points3d(s, nrec, rec_pos, rsam, false, "receiver")) return r;
     if (sim_status r = points3d(s, nrec, rec_pos, rinj, true, "receiver")) return r;
-    std::vector<Inj3> sg, rg;
-    std::vector<InjE3> se, re;
-    group3d(src, true, sg, se);
-    group3d(rinj, false, rg, re);
+    std::vector<Inj3> rg;
+    std::vector<InjE3> re;
+    group3d(rinj, rg, re);
     if (sim_status r = s->cuda(cudaMemcpyAsync(s->rec3, rsam.data(), rsam.size() * sizeof(Pt3),
                                                cudaMemcpyHostToDevice, s->st), "receiver upload"))
         return r;
-    if (sim_status r = upload(s, s->src3g, sg, 8 * (size_t)ms, "source group")) return r;
-    if (sim_status r = upload(s, s->src3e, se, 8 * (size_t)ms, "source entry")) return r;
+    if (sim_status r = s->cuda(cudaMemcpyAsync(s->src3, src.data(), src.size() * sizeof(Pt3), cudaMemcpyHostToDevice,
+                                               s->st), "source upload"))
+        return r;
     if (sim_status r = upload(s, s->res3g, rg, 8 * (size_t)std::max(1, d.max_rec), "residual group")) return r;
     if (sim_status r = upload(s, s->res3e, re, 8 * (size_t)std::max(1, d.max_rec), "residual entry")) return r;
     SimIO io{};
@@ -1937,20 +1928,16 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
     adj.src_scale = (float)(d.h * d.h);
     float *Gs = static_cast<float *>(s->Gbuf);
     const size_t qstride = q_slot_bytes(s, ckpt_fp16);
-    const int nsg = (int)sg.size(), nrg = (int)rg.size();
+    const int nrg = (int)rg.size();
     const bool fused = cpml && cpml3d_adjoint_fits(a);
-    const Pt3 *r3 = s->rec3;
+    const Pt3 *r3 = s->rec3, *s3 = s->src3;
     const long long gkey = ((long long)nshots << 40) ^ ((long long)nrec << 16) ^ ((long long)ckpt_fp16 << 3) ^
                            ((long long)o.vjp << 5) ^ 6;
     if (sim_status r = run_graph(s, gkey, [&](cudaStream_t st) {
             cudaError_t e = reset_state_on(s, nshots, st);
             if (e != cudaSuccess) return e;
             auto step = [&](const StepArgs<float> &A, int n, int mode, float *slot, bool sample) {
-                cudaError_t e2 = step3d_core(s, A, n, zs, nshots, st, s->use_graphs, mode, slot,
-                                             sample ? r3 : nullptr, nrec);
-                if (e2 == cudaSuccess)
-                    e2 = launch_inj3d(A, n, n, s->src3g, nsg, s->src3e, 0, nshots, mode, slot, nullptr, st);
-                return e2;
+                return step3d_core(s, A, n, zs, nshots, st, s->use_graphs, mode, slot, s3, sample ? r3 : nullptr, nrec);
             };
             auto slot_of = [&](int i) { return reinterpret_cast<float *>(static_cast<char *>(s->qbuf) + (size_t)i * qstride); };
             e = emit_gradient(
@@ -1977,9 +1964,9 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
                     if (terms && fused) e2 = launch_cpml3d_adjoint(a, s->add3, ca, nshots, st, s->use_graphs);
                     if (e2 == cudaSuccess)
                         e2 = launch_step3d(adj, n, zs, nshots, st, s->use_graphs, kModeAdjoint,
-                                           terms && fused ? s->add3 : Add3{}, slot, Gs);
+                                           terms && fused ? s->add3 : Add3{}, nullptr, 0, slot, Gs);
                     if (e2 == cudaSuccess)
-                        e2 = launch_inj3d(adj, n, k, s->res3g, nrg, s->res3e, 1, nshots, kModeAdjoint, slot, Gs, st);
+                        e2 = launch_inj3d(adj, n, k, s->res3g, nrg, s->res3e, nshots, slot, Gs, st);
                     if (e2 == cudaSuccess && terms && !fused) e2 = launch_cpml_adjoint<float>(a, ca, k & 1, nshots, st);
                     return e2;
                 },

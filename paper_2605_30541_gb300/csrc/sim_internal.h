@@ -264,16 +264,11 @@ int march2x_warps_per_sm();
 cudaError_t launch_march2x(const TBArgs &b, const TBPass &t, int nwarps, cudaStream_t st);
 
 // 3D step (fwd3d.cu, cpml3d.cu). Per step: snapshot, CPML addends and
-// receiver samples, z-march update with the addends, source injection.
+// receiver samples, z-march update with the addends and the sources.
 // z-march variants: kZMarchAsync stages each plane by per-thread 16-byte
-// cp.async copies; the others by three bulk tensor copies (TMA) per plane
-// issued by one thread, completion on mbarriers, with the plane loop
-// unrolled by 9 (kZMarchTma, kZMarchTmaPlain), not at all (kZMarchTmaLoop,
-// kZMarchTmaFoldLoop) or by 3 (kZMarchTmaLoop3). kZMarchTma and
-// kZMarchTmaFoldLoop are names of earlier variants that formed the x-strip
-// CPML in the march itself; they run the same kernels now. All take z chunks
-// of `zchunk` planes per CTA.
-enum { kZMarchAsync = 1, kZMarchTma = 2, kZMarchTmaPlain = 3, kZMarchTmaLoop = 4, kZMarchTmaFoldLoop = 5, kZMarchTmaLoop3 = 6 };
+// cp.async copies; kZMarchTma by bulk tensor copies (TMA) issued by one
+// thread, completion on mbarriers.
+enum { kZMarchAsync = 1, kZMarchTma = 6 };
 // CPML addends of the 3D step: per axis a compact array over the cells of its
 // strips widened by 4 (z: slots of whole (y, x) planes; y: slots of x rows in
 // every plane; x: the float4s from the strip ends of every row), one after
@@ -304,28 +299,26 @@ struct Tma3 {
 };
 cudaError_t configure_step3d();
 struct ZShape {
-    int variant = kZMarchTmaLoop3;
-    int tile = 128;  // columns of a CTA's tile (kZMarchTmaLoop3: 128, 64 or 32 of 1024 cells)
+    int variant = kZMarchTma;
+    int tile = 64;   // columns of a CTA's tile (TMA: 64 or 32 of 1024 cells; cp.async: 128 x 8)
     int chunk = 0;   // planes per CTA
 };
+// src, row: the shots' point sources and the wavelet row they inject (NULL, or
+// a row outside the record: none)
 cudaError_t launch_step3d(const StepArgs<float> &a, int n, const ZShape &zs, int nshots, cudaStream_t st, bool pdl, int mode,
-                          const Add3 &D, float *qs = nullptr, float *Gs = nullptr);
-// 3D point injection grouped by target cell (the adjoint path): group =
-// cell offset within a field, entry range, shot (-1: the same for every
-// shot, the launch's y index).
+                          const Add3 &D, const Pt3 *src, int row, float *qs = nullptr, float *Gs = nullptr);
+// 3D residual injection grouped by target cell (the adjoint sweep): group =
+// cell offset within a field and entry range, the same for every shot.
 struct Inj3 {
     long long cell;
     int e0, e1;
-    int shot, pad;
 };
 struct InjE3 {
     int pt;
     float w;
 };
 cudaError_t launch_inj3d(const StepArgs<float> &a, int n, int row, const Inj3 *grp, int ngrp, const InjE3 *ent,
-                         int kind, int nshots, int mode, float *qs, float *Gs, cudaStream_t st);
-cudaError_t launch_inject3d(const StepArgs<float> &a, const StepTime &t, const void *src, int nshots,
-                            cudaStream_t st);
+                         int nshots, const float *qs, float *Gs, cudaStream_t st);
 cudaError_t launch_snap3d(const StepArgs<float> &a, const StepTime &t, int fp16, int nshots, cudaStream_t st);
 
 // Resident execution (resident2d.cu): one cooperative launch runs the whole
