@@ -13,7 +13,7 @@
 // c and reading and writing p^{n+1} once more per axis) cost 0.88 ms of a
 // 3.17 ms step of 649 x 1060 x 1060 cells and, three short launches of 150 to
 // 370 CTAs each, 104 of 225 us at 170 x 227 x 273 x 2 shots. This launch takes
-// 64 us there, and the march pays the addends' read.
+// 62 us there, and the march pays the addends' read.
 // Here a block owns all rows of one strip range for 128 columns at one
 // position of the third axis (z and y axes: k_cpml3d's column blocks), so
 // psi can be updated in place; its warps take runs of rows, with register
@@ -85,11 +85,6 @@ struct Plan3 {
     int nrec, nbs;
 };
 
-// addend of the float4 at x of row (z, y) = row
-__device__ __forceinline__ long long x_slot(const Plan3 &Q, long long row, int x) {
-    return row * Q.D.nxw + (x < Q.D.xl ? x : Q.D.xl + x - Q.D.xs);
-}
-
 // ---------------------------------------------------------------- columns (z and y axes)
 
 // Rows [i0, i1) of the block's L that warp w takes.
@@ -116,61 +111,90 @@ __device__ __forceinline__ void col_block(const StepArgs<float> &A, const Plan3 
     f += o0, m0 += o0, m1 += o0;
     const float *ca = A.ca[ax], *cb = A.cb[ax];
     auto strip = [&](int r) { return (lo > 0 && r >= 0 && r < lo) || (hi > 0 && r >= N - hi && r < N); };
-    // addend row of r
-    const int l1 = ax == 0 ? Q.D.zl : Q.D.yl, h0 = ax == 0 ? Q.D.zh : Q.D.yh;
-    auto out = [&](int r) {
-        const int slot = r < l1 ? r : l1 + r - h0;
-        return add + (ax == 0 ? (long long)slot * g.NY + u : (long long)u * Q.D.nyw + slot) * g.P + x;
-    };
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     constexpr int FH = ADJ ? 4 : 8;       // rows of f beyond the range
     float *F = sm + 4 * lane;             // L + 2 FH rows of f from s0 - FH
     float *S = F + (L + 2 * FH) * CW;     // L + 8 rows of m0 from s0 - 4, zero off the strip
     float *Z = S + (L + 8) * CW;          // forward: L rows of m1 from s0; adjoint: L + 8 from s0 - 4
-    for (int i = w; i < L + 2 * FH; i += NT / 32) cp16z(F + i * CW, f + (long long)(s0 - FH + i) * s, act);
-    for (int i = w; i < L + 8; i += NT / 32) {
-        const int r = s0 - 4 + i;
-        const bool in = act && i >= 4 && i < L + 4 && strip(r);
-        cp16z(S + i * CW, in ? m0 + (long long)r * s : f, in);
-        if (ADJ) cp16z(Z + i * CW, in ? m1 + (long long)r * s : f, in);
-        else if (i >= 4 && i < L + 4) cp16z(Z + (i - 4) * CW, in ? m1 + (long long)r * s : f, in);
+    constexpr int ZH = ADJ ? 4 : 0, NWB = NT / 32;
+    {   // rows w, w + NWB, ...: pointers advance by a stride
+        const float *p = f + (s0 - FH + w) * s;
+        for (int i = w; i < L + 2 * FH; i += NWB, p += NWB * s) cp16z(F + i * CW, p, act);
+        const long long o = (s0 - 4 + w) * s;
+        const float *p0 = m0 + o, *p1 = m1 + o;
+        for (int i = w; i < L + 8; i += NWB, p0 += NWB * s, p1 += NWB * s) {
+            const bool in = i >= 4 && i < L + 4;
+            float *const z = Z + (i - 4 + ZH) * CW;
+            if (in && strip(s0 - 4 + i)) {
+                cp16z(S + i * CW, p0, act);
+                cp16z(z, p1, act);
+            } else {
+                st4(S + i * CW, zero);
+                if (ADJ || in) st4(z, zero);
+            }
+        }
     }
     f32::cp_async_wait_all();
     __syncthreads();
     int i0, i1;
     warp_rows(L, w, i0, i1);
+    // the thread's rows of the memory fields and of the addend (a range's slots are consecutive)
+    float *q0 = m0 + (s0 + i0) * s, *q1 = m1 + (s0 + i0) * s;
+    const int l1 = ax == 0 ? Q.D.zl : Q.D.yl, h0 = ax == 0 ? Q.D.zh : Q.D.yh, r0 = s0 + i0;
+    const int slot = r0 < l1 ? r0 : l1 + r0 - h0;
+    const long long as = ax == 0 ? (long long)g.NY * g.P : g.P;
+    float *out = add + (ax == 0 ? (long long)slot * g.NY + u : (long long)u * Q.D.nyw + slot) * g.P + x;
 
-    if (!ADJ) {
-        float4 W[9], V[9];
+    // Rows i0 .. i1 - 1, blocks of 9 unrolled: the 9-row register windows W (rows
+    // i .. i + 8 of the array at w0) and V (v0; NULL: none) rotate by renaming.
+    // fn(i, place of row i's window) reads W[(k + m) % 9].
+    float4 W[9], V[9];
+    auto windows = [&](const float *w0, const float *v0, auto fn) {
 #pragma unroll
-        for (int m = 0; m < 8; m++) W[m] = ld4(F + (i0 + 4 + m) * CW);
-        for (int i = i0; i < i1; i++) {  // psi^n of row r
+        for (int m = 0; m < 8; m++) {
+            W[m] = ld4(w0 + (i0 + m) * CW);
+            if (v0) V[m] = ld4(v0 + (i0 + m) * CW);
+        }
+        for (int ib = i0; ib < i1; ib += 9) {
+#pragma unroll
+            for (int k = 0; k < 9; k++) {
+                const int i = ib + k;
+                if (i >= i1) break;
+                W[(k + 8) % 9] = ld4(w0 + (i + 8) * CW);
+                if (v0) V[(k + 8) % 9] = ld4(v0 + (i + 8) * CW);
+                fn(i, k);
+            }
+        }
+    };
+    auto d1 = [](const float4 *X, int k, float2 &da, float2 &db) {
+        f32::d1_pairs(X[k % 9], X[(k + 1) % 9], X[(k + 2) % 9], X[(k + 3) % 9], X[(k + 5) % 9], X[(k + 6) % 9],
+                      X[(k + 7) % 9], X[(k + 8) % 9], da, db);
+    };
+    auto d2 = [](const float4 *X, int k, float2 &da, float2 &db) {
+        const float4 &c = X[(k + 4) % 9], &m1 = X[(k + 3) % 9], &p1 = X[(k + 5) % 9], &m2 = X[(k + 2) % 9],
+                     &p2 = X[(k + 6) % 9], &m3 = X[(k + 1) % 9], &p3 = X[(k + 7) % 9], &m4 = X[k % 9], &p4 = X[(k + 8) % 9];
+        da = d2c2(lo2(c), lo2(m1), lo2(p1), lo2(m2), lo2(p2), lo2(m3), lo2(p3), lo2(m4), lo2(p4));
+        db = d2c2(hi2(c), hi2(m1), hi2(p1), hi2(m2), hi2(p2), hi2(m3), hi2(p3), hi2(m4), hi2(p4));
+    };
+    if (!ADJ) {
+        windows(F + 4 * CW, nullptr, [&](int i, int k) {  // psi^n of row r
             const int r = s0 + i;
-            W[8] = ld4(F + (i + 12) * CW);
             if (strip(r)) {
                 const float a = __ldg(ca + r), b = __ldg(cb + r);
                 float2 da, db;
-                f32::d1_pairs(W[0], W[1], W[2], W[3], W[5], W[6], W[7], W[8], da, db);
+                d1(W, k, da, db);
                 const float4 old = ld4(S + (i + 4) * CW);
                 const float2 pa = f32::rec2(splat2(a), da, splat2(b), lo2(old));
                 const float2 pb = f32::rec2(splat2(a), db, splat2(b), hi2(old));
                 const float4 ps = make_float4(pa.x, pa.y, pb.x, pb.y);
                 st4(S + (i + 4) * CW, ps);
-                if (act) st4(m0 + (long long)r * s, ps);
+                if (act) st4(q0, ps);
             }
-#pragma unroll
-            for (int m = 0; m < 8; m++) W[m] = W[m + 1];
-        }
+            q0 += s;
+        });
         __syncthreads();
-#pragma unroll
-        for (int m = 0; m < 8; m++) {
-            W[m] = ld4(F + (i0 + 4 + m) * CW);
-            V[m] = ld4(S + (i0 + m) * CW);
-        }
-        for (int i = i0; i < i1; i++) {  // zeta^n and the addend of row r
+        windows(F + 4 * CW, S, [&](int i, int k) {  // zeta^n and the addend of row r
             const int r = s0 + i;
-            W[8] = ld4(F + (i + 12) * CW);
-            V[8] = ld4(S + (i + 8) * CW);
             float a = 0.f, b = 0.f;
             const bool in = strip(r);
             if (in) {
@@ -178,84 +202,57 @@ __device__ __forceinline__ void col_block(const StepArgs<float> &A, const Plan3 
                 b = __ldg(cb + r);
             }
             const float4 zo = ld4(Z + i * CW);
-            const float2 d2a = d2c2(lo2(W[4]), lo2(W[3]), lo2(W[5]), lo2(W[2]), lo2(W[6]), lo2(W[1]), lo2(W[7]),
-                                    lo2(W[0]), lo2(W[8]));
-            const float2 d2b = d2c2(hi2(W[4]), hi2(W[3]), hi2(W[5]), hi2(W[2]), hi2(W[6]), hi2(W[1]), hi2(W[7]),
-                                    hi2(W[0]), hi2(W[8]));
-            float2 dsa, dsb;
-            f32::d1_pairs(V[0], V[1], V[2], V[3], V[5], V[6], V[7], V[8], dsa, dsb);
+            float2 d2a, d2b, dsa, dsb;
+            d2(W, k, d2a, d2b);
+            d1(V, k, dsa, dsb);
             const float2 za = f32::rec2(splat2(a), add2(d2a, dsa), splat2(b), lo2(zo));
             const float2 zb = f32::rec2(splat2(a), add2(d2b, dsb), splat2(b), hi2(zo));
             if (act) {
-                if (in) st4(m1 + (long long)r * s, make_float4(za.x, za.y, zb.x, zb.y));
+                if (in) st4(q1, make_float4(za.x, za.y, zb.x, zb.y));
                 const float2 aa = add2(dsa, za), ab = add2(dsb, zb);
-                st4(out(r), make_float4(aa.x, aa.y, ab.x, ab.y));
+                st4(out, make_float4(aa.x, aa.y, ab.x, ab.y));
             }
-#pragma unroll
-            for (int m = 0; m < 8; m++) {
-                W[m] = W[m + 1];
-                V[m] = V[m + 1];
-            }
-        }
+            q1 += s;
+            out += as;
+        });
     } else {
         // nu^k = b nu + u of the strip rows (S then holds a nu^k), w = u + a nu^k (F)
-        for (int i = i0; i < i1; i++) {
+        for (int i = i0; i < i1; i++, q0 += s) {
             const int r = s0 + i;
             if (!strip(r)) continue;
             const float a = __ldg(ca + r), b = __ldg(cb + r);
             const float4 uo = ld4(F + (i + 4) * CW), no = ld4(S + (i + 4) * CW);
             const float2 na = fma2(splat2(b), lo2(no), lo2(uo)), nb = fma2(splat2(b), hi2(no), hi2(uo));
-            if (act) st4(m0 + (long long)r * s, make_float4(na.x, na.y, nb.x, nb.y));
+            if (act) st4(q0, make_float4(na.x, na.y, nb.x, nb.y));
             const float2 pa = mul2(splat2(a), na), pb = mul2(splat2(a), nb);
             st4(S + (i + 4) * CW, make_float4(pa.x, pa.y, pb.x, pb.y));
             const float2 wa = add2(lo2(uo), pa), wb = add2(hi2(uo), pb);
             st4(F + (i + 4) * CW, make_float4(wa.x, wa.y, wb.x, wb.y));
         }
         __syncthreads();
-        // mu^k = b mu - D1 w of the strip rows (Z then holds a mu^k)
-        float4 W[9], V[9];
-#pragma unroll
-        for (int m = 0; m < 8; m++) W[m] = ld4(F + (i0 + m) * CW);
-        for (int i = i0; i < i1; i++) {
+        windows(F, nullptr, [&](int i, int k) {  // mu^k = b mu - D1 w of the strip rows (Z then holds a mu^k)
             const int r = s0 + i;
-            W[8] = ld4(F + (i + 8) * CW);
             if (strip(r)) {
                 const float a = __ldg(ca + r), b = __ldg(cb + r);
                 float2 da, db;
-                f32::d1_pairs(W[0], W[1], W[2], W[3], W[5], W[6], W[7], W[8], da, db);
+                d1(W, k, da, db);
                 const float4 mo = ld4(Z + (i + 4) * CW);
                 const float2 ma = fma2(splat2(b), lo2(mo), neg2(da)), mb = fma2(splat2(b), hi2(mo), neg2(db));
-                if (act) st4(m1 + (long long)r * s, make_float4(ma.x, ma.y, mb.x, mb.y));
+                if (act) st4(q1, make_float4(ma.x, ma.y, mb.x, mb.y));
                 const float2 pa = mul2(splat2(a), ma), pb = mul2(splat2(a), mb);
                 st4(Z + (i + 4) * CW, make_float4(pa.x, pa.y, pb.x, pb.y));
             }
-#pragma unroll
-            for (int m = 0; m < 8; m++) W[m] = W[m + 1];
-        }
+            q1 += s;
+        });
         __syncthreads();
-        // the bracket D2 (a nu) - D1 (a mu)
-#pragma unroll
-        for (int m = 0; m < 8; m++) {
-            W[m] = ld4(S + (i0 + m) * CW);
-            V[m] = ld4(Z + (i0 + m) * CW);
-        }
-        for (int i = i0; i < i1; i++) {
-            W[8] = ld4(S + (i + 8) * CW);
-            V[8] = ld4(Z + (i + 8) * CW);
-            const float2 d2a = d2c2(lo2(W[4]), lo2(W[3]), lo2(W[5]), lo2(W[2]), lo2(W[6]), lo2(W[1]), lo2(W[7]),
-                                    lo2(W[0]), lo2(W[8]));
-            const float2 d2b = d2c2(hi2(W[4]), hi2(W[3]), hi2(W[5]), hi2(W[2]), hi2(W[6]), hi2(W[1]), hi2(W[7]),
-                                    hi2(W[0]), hi2(W[8]));
-            float2 dsa, dsb;
-            f32::d1_pairs(V[0], V[1], V[2], V[3], V[5], V[6], V[7], V[8], dsa, dsb);
+        windows(S, Z, [&](int, int k) {  // the bracket D2 (a nu) - D1 (a mu)
+            float2 d2a, d2b, dsa, dsb;
+            d2(W, k, d2a, d2b);
+            d1(V, k, dsa, dsb);
             const float2 ea = add2(d2a, neg2(dsa)), eb = add2(d2b, neg2(dsb));
-            if (act) st4(out(s0 + i), make_float4(ea.x, ea.y, eb.x, eb.y));
-#pragma unroll
-            for (int m = 0; m < 8; m++) {
-                W[m] = W[m + 1];
-                V[m] = V[m + 1];
-            }
-        }
+            if (act) st4(out, make_float4(ea.x, ea.y, eb.x, eb.y));
+            out += as;
+        });
     }
 }
 
@@ -288,26 +285,36 @@ __device__ __forceinline__ void row_ends(const StepArgs<float> &A, const Plan3 &
     for (int j = 1; j < nq + 3; j++)
         if (xstrip4(g, xa + 4 * j)) j0 = min(j0, j), j1 = j + 1;
     const int ns = max(0, j1 - j0);
-    const unsigned n0 = rows * J, n1 = rows * ns, n2 = rows * nq;
-    for (unsigned i = tid; i < n0; i += NT) {
-        const unsigned r = i / J;
-        const int j = (int)(i - r * J);
-        const long long o = base[r] + 4 * j;
-        const bool in = base[r] >= 0, st = in && j >= j0 && j < j1;
-        cp16z(F + 4 * i, in ? f + o : f, in);
-        cp16z(S + 4 * i, st ? m0 + o : f, st);
-        cp16z(Z + 4 * i, st ? m1 + o : f, st);
-    }
+    // fn(row, float4 m of its n) over the block's rows, dealt out to the threads
+    auto deal = [&](int n, auto fn) {
+        if (n <= 0) return;
+        const int dr = NT / n, dm = NT - dr * n;
+        int r = tid / n, m = tid - r * n;
+        while (r < rows) {
+            fn(r, m);
+            r += dr;
+            m += dm;
+            if (m >= n) m -= n, r++;
+        }
+    };
+    deal(J, [&](int r, int j) {
+        const int i = 4 * (r * J + j);
+        const long long o = base[r];
+        const bool in = o >= 0, st = in && j >= j0 && j < j1;
+        const long long p = (in ? o : 0) + 4 * j;
+        cp16z(F + i, f + p, in);
+        cp16z(S + i, m0 + p, st);
+        cp16z(Z + i, m1 + p, st);
+    });
     f32::cp_async_wait_all();
     __syncthreads();
     const float *const ca = A.ca[2] + xa, *const cb = A.cb[2] + xa;
-    const unsigned dq = max(1, ns);
+    float *const ad = add + r0 * Q.D.nxw + (xa + 8 < Q.D.xl ? xa + 8 : Q.D.xl + xa + 8 - Q.D.xs);  // the first row's float4 2
     if (!ADJ) {
-        for (unsigned i = tid; i < n1; i += NT) {  // psi^n
-            const unsigned r = i / dq;
-            const int j = j0 + (int)(i - r * dq);
+        deal(ns, [&](int r, int m) {  // psi^n
+            const int j = j0 + m;
             const long long o = base[r];
-            if (o < 0) continue;
+            if (o < 0) return;
             const float *p = F + 4 * (r * J + j);
             float *s = S + 4 * (r * J + j);
             const float4 a4 = ld4(ca + 4 * j), b4 = ld4(cb + 4 * j), old = ld4(s);
@@ -317,13 +324,12 @@ __device__ __forceinline__ void row_ends(const StepArgs<float> &A, const Plan3 &
             const float4 ps = make_float4(pa.x, pa.y, pb.x, pb.y);
             st4(s, ps);
             st4(m0 + o + 4 * j, ps);
-        }
+        });
         __syncthreads();
-        for (unsigned i = tid; i < n2; i += NT) {  // zeta^n and the addend
-            const unsigned r = i / (unsigned)nq;
-            const int j = 2 + (int)(i - r * nq);
+        deal(nq, [&](int r, int m) {  // zeta^n and the addend
+            const int j = 2 + m;
             const long long o = base[r];
-            if (o < 0) continue;
+            if (o < 0) return;
             const float *p = F + 4 * (r * J + j), *s = S + 4 * (r * J + j);
             const bool in = j >= j0 && j < j1;
             const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -335,14 +341,13 @@ __device__ __forceinline__ void row_ends(const StepArgs<float> &A, const Plan3 &
             const float2 zb = f32::rec2(hi2(a4), add2(yd, db), hi2(b4), hi2(zo));
             if (in) st4(m1 + o + 4 * j, make_float4(za.x, za.y, zb.x, zb.y));
             const float2 aa = add2(da, za), ab = add2(db, zb);
-            st4(add + x_slot(Q, r0 + r, xa + 4 * j), make_float4(aa.x, aa.y, ab.x, ab.y));
-        }
+            st4(ad + r * Q.D.nxw + 4 * m, make_float4(aa.x, aa.y, ab.x, ab.y));
+        });
     } else {
-        for (unsigned i = tid; i < n1; i += NT) {  // nu^k (S then holds a nu^k) and w = u + a nu^k (F)
-            const unsigned r = i / dq;
-            const int j = j0 + (int)(i - r * dq);
+        deal(ns, [&](int r, int m) {  // nu^k (S then holds a nu^k) and w = u + a nu^k (F)
+            const int j = j0 + m;
             const long long o = base[r];
-            if (o < 0) continue;
+            if (o < 0) return;
             float *p = F + 4 * (r * J + j), *s = S + 4 * (r * J + j);
             const float4 a4 = ld4(ca + 4 * j), b4 = ld4(cb + 4 * j), u = ld4(p), old = ld4(s);
             const float2 na = fma2(lo2(b4), lo2(old), lo2(u)), nb = fma2(hi2(b4), hi2(old), hi2(u));
@@ -351,13 +356,12 @@ __device__ __forceinline__ void row_ends(const StepArgs<float> &A, const Plan3 &
             st4(s, make_float4(pa.x, pa.y, pb.x, pb.y));
             const float2 wa = add2(lo2(u), pa), wb = add2(hi2(u), pb);
             st4(p, make_float4(wa.x, wa.y, wb.x, wb.y));
-        }
+        });
         __syncthreads();
-        for (unsigned i = tid; i < n1; i += NT) {  // mu^k (Z then holds a mu^k)
-            const unsigned r = i / dq;
-            const int j = j0 + (int)(i - r * dq);
+        deal(ns, [&](int r, int m) {  // mu^k (Z then holds a mu^k)
+            const int j = j0 + m;
             const long long o = base[r];
-            if (o < 0) continue;
+            if (o < 0) return;
             const float *p = F + 4 * (r * J + j);
             float *t = Z + 4 * (r * J + j);
             const float4 a4 = ld4(ca + 4 * j), b4 = ld4(cb + 4 * j), mo = ld4(t);
@@ -367,19 +371,18 @@ __device__ __forceinline__ void row_ends(const StepArgs<float> &A, const Plan3 &
             st4(m1 + o + 4 * j, make_float4(ma.x, ma.y, mb.x, mb.y));
             const float2 pa = mul2(lo2(a4), ma), pb = mul2(hi2(a4), mb);
             st4(t, make_float4(pa.x, pa.y, pb.x, pb.y));
-        }
+        });
         __syncthreads();
-        for (unsigned i = tid; i < n2; i += NT) {  // the bracket
-            const unsigned r = i / (unsigned)nq;
-            const int j = 2 + (int)(i - r * nq);
-            if (base[r] < 0) continue;
+        deal(nq, [&](int r, int m) {  // the bracket
+            const int j = 2 + m;
+            if (base[r] < 0) return;
             const float *s = S + 4 * (r * J + j), *t = Z + 4 * (r * J + j);
             float2 xd, yd, da, db;
             d2x_pairs(ld4(s - 4), ld4(s), ld4(s + 4), xd, yd);
             f32::d1x_pairs(ld4(t - 4), ld4(t), ld4(t + 4), da, db);
             const float2 ea = add2(xd, neg2(da)), eb = add2(yd, neg2(db));
-            st4(add + x_slot(Q, r0 + r, xa + 4 * j), make_float4(ea.x, ea.y, eb.x, eb.y));
-        }
+            st4(ad + r * Q.D.nxw + 4 * m, make_float4(ea.x, ea.y, eb.x, eb.y));
+        });
     }
 }
 
@@ -402,7 +405,7 @@ struct Mem3 {
 };
 
 template <bool ADJ>
-__global__ void __launch_bounds__(NT) k_cpml3d(const StepArgs<float> A, const Plan3 Q, const Mem3 M, const int n) {
+__global__ void __launch_bounds__(NT, 4) k_cpml3d(const StepArgs<float> A, const Plan3 Q, const Mem3 M, const int n) {
     extern __shared__ float4 sm4[];
     const int shot = blockIdx.y;
     const long long sh = (long long)shot * A.g.fstride;
