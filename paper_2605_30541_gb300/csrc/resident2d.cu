@@ -24,12 +24,21 @@
 //   - sponge subdomains precompute per cell the update weights 2/(1+a),
 //     (1-a)/(1+a) and c/(1+a) (a = c eta dt / 2 is fixed in time), so the
 //     step has no division;
-//   - after each step a CTA publishes the 8 (4 without CPML) border rows and
-//     columns of p^{n+1} to the global pressure buffer and raises its step
-//     counter (release); a CTA starts step n once the counters of the
-//     subdomains above, below and beside it (its descriptor lists them)
-//     reach n (acquire), and copies their borders in as its halo. The
-//     stencil is a cross, so corner neighbours are never needed.
+//   - a CTA writes the 8 (4 without CPML) border rows and columns of p^{n+1} to
+//     its outbox in global memory as 8-byte words (value, step number), as they
+//     are computed; a CTA starts step n by reading its neighbours' words, each
+//     until it carries the number n, and keeping the values as its halo. The
+//     word is one 64-bit access, so a value is never seen without its number
+//     and no fence, counter or second fetch lies on the way: the chain per step
+//     is one store, one read and a block barrier. (With a counter per
+//     subdomain - store, barrier, release, poll, barrier, fetch, barrier - the
+//     exchange alone took 2.55 us: 1000 steps of 241 x 241 cells 3.87 ms, of
+//     669 x 1100 with 100 snapshots 6.35 ms; 2.86 and 4.25 ms with the words.)
+//     The stencil is a cross, so corner
+//     neighbours are never needed.
+//     Two outbox halves alternate by step parity: a CTA that writes p^{n+1}
+//     over p^{n-1} has read p^n from every neighbour that reads it, and each of
+//     them sent p^n only after a barrier behind all its reads of p^{n-1}.
 // The launch is cooperative, so all CTAs are co-resident and the waits
 // always end; each wait is still bounded (spin_limit polls), after which the
 // kernel raises kFlagTimeout and every CTA returns.
@@ -74,6 +83,33 @@ constexpr size_t rsmem_floats(int bc) {
     return 2 * (WZ + 2 * HM) * SW + WZ * TX + rsmem_x<RZ>(bc) + coef + 6 * (size_t)kRecCache;
 }
 
+// Outbox of a subdomain, one half (words): the top border rows, the bottom
+// ones, the left and the right border columns.
+constexpr int XN = 0, XS = HM * TX, XWST = 2 * HM * TX, XEST = XWST + 64 * HM, XHALF = kResidentOutbox / 2;
+static_assert(XEST + 64 * HM == XHALF, "outbox size");
+
+// four words (value, tag) = 32 bytes
+__device__ __forceinline__ void put4(unsigned long long *d, const float4 v, int tag) {
+    const unsigned long long t = (unsigned long long)(unsigned)tag << 32;
+    const unsigned long long a = t | __float_as_uint(v.x), b = t | __float_as_uint(v.y), c = t | __float_as_uint(v.z),
+                             e = t | __float_as_uint(v.w);
+    asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};\nst.relaxed.gpu.global.v2.b64 [%0+16], {%3, %4};\n" ::"l"(d),
+                 "l"(a), "l"(b), "l"(c), "l"(e)
+                 : "memory");
+}
+// reads them; true when all four carry the tag
+__device__ __forceinline__ bool get4(const unsigned long long *d, int tag, float4 &v) {
+    unsigned long long a, b, c, e;
+    asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%4];\nld.relaxed.gpu.global.v2.b64 {%2, %3}, [%4+16];\n"
+                 : "=l"(a), "=l"(b), "=l"(c), "=l"(e)
+                 : "l"(d)
+                 : "memory");
+    v = make_float4(__uint_as_float((unsigned)a), __uint_as_float((unsigned)b), __uint_as_float((unsigned)c),
+                    __uint_as_float((unsigned)e));
+    const unsigned t = (unsigned)tag;
+    return (unsigned)(a >> 32) == t && (unsigned)(b >> 32) == t && (unsigned)(c >> 32) == t && (unsigned)(e >> 32) == t;
+}
+
 // Tile-local hull [lo, hi) of the parts of the absorbing strips [0, nb0) and
 // [N - nb1, N) of one axis that fall in [clip0, clip1) (tile coordinates,
 // origin o); lo >= hi when neither strip reaches the window.
@@ -94,7 +130,6 @@ template <int RZ>
 __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, const ResidentArgs R) {
     constexpr int WZ = NWR * RZ;
     extern __shared__ float4 smem4[];
-    __shared__ int s_abort;
     const bool cpml = A.bc == SIM_BC_CPML;
     float *const S0 = reinterpret_cast<float *>(smem4);
     float *const S1 = S0 + (WZ + 2 * HM) * SW;
@@ -122,12 +157,11 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
     const int shot = blockIdx.x / ntiles, tile = blockIdx.x - shot * ntiles;
     const RTile *const D = R.tiles + tile;
     const int bx = D->bx, x0 = bx * TX, z0 = D->z0, rows = D->rows, rpw = D->rpw, P = g.P;
-    const int my_nbr = lane < D->nnbr ? D->nbr[lane] : -1;  // the subdomain lane polls (warp 0)
     const long long sh = (long long)shot * g.fstride;
     const long long org = cell_off(g, z0, 0, x0);
     float *const gb0 = A.pbuf[0] + sh + org;
     float *const gb1 = A.pbuf[1] + sh + org;
-    int *const done = R.done + shot * ntiles;
+    unsigned long long *const outbox = R.outbox + (long long)blockIdx.x * kResidentOutbox;
 
     const bool cpx = cpml && A.ca[2] &&
                      ((g.nbx0 > 0 && x0 - 4 < g.nbx0) || (g.nbx1 > 0 && x0 + TX + 4 > g.NX - g.nbx1));
@@ -174,7 +208,6 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
         const int n4 = (int)(rsmem_floats<RZ>(A.bc) / 4);
         for (int i = tid; i < n4; i += NTR) smem4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (tid == 0) s_abort = 0;
 
     // run constants of the thread's own cells
     float4 ch4[RZ];
@@ -237,6 +270,58 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
             ROFF[e - r0] = (HM + Rc.lz) * SW + HM + Rc.lx;
             for (int q = 0; q < 4; q++) RW[4 * (e - r0) + q] = Rc.w[q];
         }
+    // The thread's halo float4s (at most two): the words of a neighbour's outbox
+    // and the place in the pressure buffer. Rows -H .. -1 come from the bottom
+    // rows of the subdomain above, rows >= rows from the top rows of the one
+    // below (a last one of fewer than H rows has no more: zeros), columns left
+    // and right from the subdomains of the adjacent columns that hold the row.
+    int xsrc[2] = {-1, -1}, xdst[2] = {0, 0};
+    {
+        const int hq = H / 4, nN = hasN ? 32 * H : 0;
+        int up = -1, down = -1;
+        for (int k = 0; k < D->nnbr; k++) {
+            const RTile &u = R.tiles[D->nbr[k]];
+            if (u.bx == bx && u.z0 < z0) up = D->nbr[k];
+            if (u.bx == bx && u.z0 > z0) down = D->nbr[k];
+        }
+        const int nS = hasS ? 32 * min(H, R.tiles[down].rows) : 0, nW = hasW ? rows * hq : 0, nE = hasE ? rows * hq : 0;
+        auto side = [&](int dx, int gz) {  // word offset of the neighbour column's subdomain that holds row gz, and its row
+            for (int k = 0; k < D->nnbr; k++) {
+                const RTile &u = R.tiles[D->nbr[k]];
+                if (u.bx == bx + dx && gz >= u.z0 && gz < u.z0 + u.rows)
+                    return (shot * ntiles + D->nbr[k]) * kResidentOutbox + (gz - u.z0) * HM;
+            }
+            return -1;
+        };
+        for (int v = 0; v < 2; v++) {
+            int i = tid + v * NTR;
+            if (i < nN) {
+                xsrc[v] = (shot * ntiles + up) * kResidentOutbox + XS + i * 4;
+                xdst[v] = (HM - H + (i >> 5)) * SW + HM + 4 * (i & 31);
+                continue;
+            }
+            i -= nN;
+            if (i < nS) {
+                xsrc[v] = (shot * ntiles + down) * kResidentOutbox + XN + i * 4;
+                xdst[v] = (HM + rows + (i >> 5)) * SW + HM + 4 * (i & 31);
+                continue;
+            }
+            i -= nS;
+            if (i < nW) {
+                const int r = i / hq, q = i - r * hq, o = side(-1, z0 + r);
+                xsrc[v] = o < 0 ? -1 : o + XEST + 4 * q;
+                xdst[v] = (HM + r) * SW + HM - H + 4 * q;
+                continue;
+            }
+            i -= nW;
+            if (i < nE) {
+                const int r = i / hq, q = i - r * hq, o = side(1, z0 + r);
+                xsrc[v] = o < 0 ? -1 : o + XWST + 4 * q;
+                xdst[v] = (HM + r) * SW + HM + TX + 4 * q;
+            }
+        }
+    }
+    static_assert(2 * HM * 32 + 2 * 64 * (HM / 4) <= 2 * NTR, "two halo float4s per thread at most");
     const SimIO *io = A.io;
     const float *const wav = static_cast<const float *>(io->wavelet);
     float *const gout = static_cast<float *>(io->gather);
@@ -248,64 +333,38 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
     for (int n = 0; n < A.nt; n++) {
         float *const cur = (n & 1) ? S1 : S0;
         float *const nxt = (n & 1) ? S0 : S1;
-        const float *const gcur = (n & 1) ? gb1 : gb0;
-        float *const gnxt = (n & 1) ? gb0 : gb1;
-
         // this step's wavelet sample (fetched one step ahead)
         const float wn = wnext;
         if (has_inj && n + 1 < A.nt) wnext = wav[n + 1];
 
-        if (n > 0) {
-            // the subdomains whose borders form the halo must have published p^n
-            if (w == 0) {
-                const int nb = my_nbr;
-                bool need = nb >= 0, quit = false;
-                long long spins = 0;
-                for (;;) {
-                    if (need && ld_acquire(done + nb) >= n) need = false;
-                    if (!__any_sync(0xffffffffu, need)) break;
-                    if (++spins > R.spin_limit) {
-                        quit = true;
-                        if (lane == 0) atomicOr(A.flags, kFlagTimeout);
-                        break;
-                    }
-                    if ((spins & 1023) == 0) {
-                        const unsigned f = lane == 0 ? *reinterpret_cast<volatile unsigned *>(A.flags) : 0u;
-                        if (__shfl_sync(0xffffffffu, f, 0) & kFlagTimeout) {
-                            quit = true;
-                            break;
-                        }
-                    }
+        bool quit = false;
+        if (n > 0) {  // the neighbours' borders of p^n become this step's halo
+            const unsigned long long *const in = R.outbox + (n & 1) * XHALF;
+            bool need0 = xsrc[0] >= 0, need1 = xsrc[1] >= 0;
+            for (long long spins = 0; need0 || need1;) {
+                float4 v0, v1;
+                const bool ok0 = need0 && get4(in + xsrc[0], n, v0), ok1 = need1 && get4(in + xsrc[1], n, v1);
+                if (ok0) {
+                    st4(cur + xdst[0], v0);
+                    need0 = false;
                 }
-                if (lane == 0) s_abort = quit;
+                if (ok1) {
+                    st4(cur + xdst[1], v1);
+                    need1 = false;
+                }
+                if (!(need0 || need1)) break;
+                if (++spins > R.spin_limit) {
+                    quit = true;
+                    atomicOr(A.flags, kFlagTimeout);
+                    break;
+                }
+                if ((spins & 1023) == 0 && (*reinterpret_cast<volatile unsigned *>(A.flags) & kFlagTimeout)) {
+                    quit = true;
+                    break;
+                }
             }
-            __syncthreads();
-            if (s_abort) return;
-            // their borders become this step's halo
-            if (hasN)
-                for (int i = tid; i < H * 32; i += NTR) {
-                    const int r = -H + (i >> 5), c = 4 * (i & 31);
-                    cp_async16(cur + (HM + r) * SW + HM + c, gcur + r * P + c);
-                }
-            if (hasS)
-                for (int i = tid; i < H * 32; i += NTR) {
-                    const int r = rows + (i >> 5), c = 4 * (i & 31);
-                    cp_async16(cur + (HM + r) * SW + HM + c, gcur + r * P + c);
-                }
-            const int hq = H / 4;
-            if (hasW)
-                for (int i = tid; i < rows * hq; i += NTR) {
-                    const int r = i / hq, q = i - r * hq;
-                    cp_async16(cur + (HM + r) * SW + HM - H + 4 * q, gcur + r * P - H + 4 * q);
-                }
-            if (hasE)
-                for (int i = tid; i < rows * hq; i += NTR) {
-                    const int r = i / hq, q = i - r * hq;
-                    cp_async16(cur + (HM + r) * SW + HM + TX + 4 * q, gcur + r * P + TX + 4 * q);
-                }
-            cp_async_wait_all();
         }
-        __syncthreads();
+        if (__syncthreads_or(quit)) return;
         if (top && n > 0) {  // odd mirror above the free surface: p(-k) = -p(k)
             const int nch = (TX + 2 * H) / 4;
             for (int k = 1 + w; k <= H; k += NWR) {
@@ -461,19 +520,16 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
             if (top && lz == 0) res[0] = res[1] = res[2] = res[3] = 0.f;
             const float4 r4 = make_float4(res[0], res[1], res[2], res[3]);
             st4(nxt + (rb + j) * SW + c0, r4);
-            const bool border = (hasN && lz < H) || (hasS && lz >= rows - H) || (hasW && 4 * lane < H) ||
-                                (hasE && 4 * lane >= TX - H);
-            if (border) st4(gnxt + lo + j * P, r4);
+            unsigned long long *const ob = outbox + ((n + 1) & 1) * XHALF;
+            if (hasN && lz < H) put4(ob + XN + lz * TX + 4 * lane, r4, n + 1);
+            if (hasS && lz >= rows - H) put4(ob + XS + (lz - rows + H) * TX + 4 * lane, r4, n + 1);
+            if (hasW && 4 * lane < H) put4(ob + XWST + lz * HM + 4 * lane, r4, n + 1);
+            if (hasE && 4 * lane >= TX - H) put4(ob + XEST + lz * HM + 4 * lane - (TX - H), r4, n + 1);
         }
 
-        // publish p^{n+1}: the release orders every thread's border stores
-        // (ordered before it by the barrier) before the counter
-        __syncthreads();
-        if (tid == 0) st_release(done + tile, n + 1);
-
-        // Off the critical path, while the neighbours proceed: receivers and
-        // the snapshot sample p^n, still held in this buffer until the next
-        // step's update overwrites it.
+        // Off the critical path, while the words travel: receivers and the
+        // snapshot sample p^n, still held in this buffer until the next step's
+        // update (behind the next barrier) overwrites it.
         if (r1 > r0 && gout) {
             const long long rowo = ((long long)shot * A.nt + n) * nrec;
             for (int e = tid; e < r1 - r0; e += NTR) {

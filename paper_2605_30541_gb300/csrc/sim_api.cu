@@ -269,7 +269,8 @@ struct sim_s {
     bool use_march = false; // the autotuner's choice: row march rather than the tiled step kernel
     Pt3 *src3 = nullptr, *rec3 = nullptr;  // 3D point tables
     Add3 add3{};                           // 3D CPML addends of one step
-    int *rdone = nullptr;                  // resident path: step counter per (shot, subdomain)
+    unsigned long long *outbox = nullptr;  // resident path: border words, one outbox per CTA
+    int cap_outbox = 0;                    //   (CTAs it holds)
     Inj3 *res3g = nullptr;                 // 3D adjoint: injection groups of the residuals
     InjE3 *res3e = nullptr;
     RTile *rtiles = nullptr;               // resident path: subdomain descriptors
@@ -1114,11 +1115,11 @@ bool plan_resident_uncached(sim_t s, int nshots, ResidentPlan &plan) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, s->dev);
     if (!coop || sms <= 0) return false;
-    const long long cap_tiles = max_tiles(s);  // step counters and descriptors
+    const long long cap_tiles = max_tiles(s);  // descriptors
     for (int rz = 1; rz <= 4; rz++) {
         const int bps = resident2d_blocks_per_sm(rz, s->d.bc);
         if (bps <= 0) continue;
-        const long long cap = std::min((long long)bps * sms / nshots, cap_tiles);
+        const long long cap = std::min((long long)std::min(bps * sms, s->cap_outbox) / nshots, cap_tiles);
         const int wz = kResidentWarps * rz;
         std::vector<RTile> t;
         // the largest target gives uniform wz-row subdomains (the fewest)
@@ -1148,7 +1149,7 @@ bool plan_resident_uncached(sim_t s, int nshots, ResidentPlan &plan) {
 
 // The plan depends only on the grid and the shot count: kept per handle.
 const ResidentPlan *plan_resident(sim_t s, int nshots) {
-    if (s->g.ndim != 2 || s->d.precision != SIM_FP32 || s->d.snap_fp16 || !s->rdone) return nullptr;
+    if (s->g.ndim != 2 || s->d.precision != SIM_FP32 || s->d.snap_fp16 || !s->outbox) return nullptr;
     const char *f = getenv("GSIM_RESIDENT");
     if (f && f[0] == '0') return nullptr;
     for (const auto &p : s->rplans)
@@ -1159,8 +1160,8 @@ const ResidentPlan *plan_resident(sim_t s, int nshots) {
     return p.rz ? &p : nullptr;
 }
 
-// One cooperative launch for the whole time loop, after zeroing the step
-// counters; ordered on the handle's stream like any other work.
+// One cooperative launch for the whole time loop, after zeroing the border
+// words; ordered on the handle's stream like any other work.
 template <typename T>
 sim_status run_resident(sim_t s, const StepArgs<T> &a, const ResidentPlan &plan, int nshots);
 template <>
@@ -1171,10 +1172,11 @@ template <>
 sim_status run_resident<float>(sim_t s, const StepArgs<float> &a, const ResidentPlan &plan, int nshots) {
     const int nt = (int)plan.tiles.size();
     if (sim_status r = upload(s, s->rtiles, plan.tiles, (size_t)max_tiles(s), "subdomains")) return r;
-    if (sim_status r = s->cuda(cudaMemsetAsync(s->rdone, 0, (size_t)nt * nshots * sizeof(int), s->st),
-                               "step counters"))
+    // no word of an earlier run may carry a step number of this one
+    if (sim_status r = s->cuda(cudaMemsetAsync(s->outbox, 0, (size_t)nt * nshots * kResidentOutbox * sizeof(*s->outbox),
+                                               s->st), "border words"))
         return r;
-    ResidentArgs r{s->rdone, spin_limit(), s->rtiles, nt};
+    ResidentArgs r{s->outbox, spin_limit(), s->rtiles, nt};
     return s->cuda(launch_resident2d(a, r, plan.rz, nshots, s->st), "resident launch");
 }
 
@@ -2861,7 +2863,12 @@ sim_status sim_create(const sim_desc *din, const void *vel, void *cuda_stream, s
         rc = s->cuda(configure_resident2d(), "kernel configuration");
         if (rc == SIM_OK) rc = s->cuda(configure_march2d(), "kernel configuration");
         if (rc == SIM_OK) rc = s->cuda(configure_march2x(), "kernel configuration");
-        s->rdone = static_cast<int *>(A(sizeof(int) * ms * max_tiles(s)));
+        // a grid one of whose runs can be resident: an outbox per CTA (at most one
+        // CTA per SM: 512 threads of over 64 registers)
+        s->cap_outbox = device_sms(s->dev);
+        const long long on_chip = (long long)s->cap_outbox * kResidentWarps * 4 * kTileXF;
+        if ((long long)g.NZ * g.NX <= on_chip)
+            s->outbox = static_cast<unsigned long long *>(A(sizeof(*s->outbox) * kResidentOutbox * s->cap_outbox));
         s->rtiles = static_cast<RTile *>(A(sizeof(RTile) * max_tiles(s)));
         // row march: one item per (shot, strip, 4 rows) at most
         s->cap_mseg = (size_t)ms * ((g.NX + kMarchW - 1) / kMarchW) * ((g.NZ + 3) / 4) + 2;

@@ -325,18 +325,19 @@ cudaError_t launch_snap3d(const StepArgs<float> &a, const StepTime &t, int fp16,
 // forward time loop of a 2D FP32 problem whose state fits on chip; each CTA
 // of kResidentWarps warps owns one subdomain: columns [128 bx, 128 bx + 128),
 // rows [z0, z0 + rows) with rows <= 16 RZ, warps taking rpw rows each.
-// nbr lists the subdomains whose borders form its halo (same shot). done[]
-// holds one step counter per (shot, subdomain), zeroed before the launch.
+// nbr lists the subdomains whose borders form its halo (same shot). outbox:
+// kResidentOutbox 8-byte words per (shot, subdomain), zeroed before the launch.
 constexpr int kResidentWarps = 16;
 constexpr size_t kResidentMaxSmem = 227 * 1024;
 constexpr int kResidentMaxNbr = 11;
+constexpr int kResidentOutbox = 2 * (2 * 8 * 128 + 2 * 64 * 8);  // two step parities of border rows and columns
 struct RTile {
     int bx, z0, rows, rpw;
     int nnbr;
     int nbr[kResidentMaxNbr];
 };
 struct ResidentArgs {
-    int *done;
+    unsigned long long *outbox;
     long long spin_limit;
     const RTile *tiles;  // device array, per shot
     int ntiles;
