@@ -1,53 +1,65 @@
-// Resident FP32 2D forward solve: the whole time loop of one forward run in
-// a single cooperative launch whose CTAs keep the wavefield on chip.
+// Resident FP32 2D steps: a run of time steps of one or more shots in a single
+// cooperative launch whose CTAs keep the wavefield on chip. Three modes: the
+// forward solve, the forward recompute that records the imaging terms, and the
+// adjoint sweep that consumes them.
 //
 // The per-step kernel (fwd2d_f32.cu) pays, every step, a launch, a grid-wide
-// dependency and a reload of p^n, p^{n-1} and c from L2. On a slice of a few
-// hundred thousand to about a million cells the whole state fits in the SMs'
-// shared memory and registers, so here each CTA owns one subdomain of 128
-// columns and at most WZ = 16 RZ rows for the entire run. Subdomain heights
-// vary (RTile descriptors from the host): subdomains with absorbing work get
-// fewer rows, so every CTA takes about as long per step; warps take
-// ceil(rows / 16) consecutive rows each.
+// dependency and a reload of p^n, p^{n-1} and c from L2: 6 to 15 us on grids
+// whose arithmetic takes one. On a slice of a few hundred thousand to about a
+// million cells (all shots of an FWI survey on a small model, or one shot of a
+// field-scale slice) the whole state fits in the SMs' shared memory, so here
+// each CTA owns one subdomain of 128 columns and at most WZ = 16 RZ rows for
+// the entire run. Subdomain heights vary (RTile descriptors from the host):
+// subdomains with absorbing work get fewer rows, so every CTA takes about as
+// long per step; warps take ceil(rows / 16) consecutive rows each.
 //   - p^n with an 8-cell halo lives in shared memory in two buffers; the
 //     other buffer's own cells still hold p^{n-1}, which each thread reads
-//     and overwrites with p^{n+1} in place; c stays in registers;
-//   - the CPML memory variables live in shared memory and are computed only
-//     where they can be non-zero: psi on the absorbing strips (and the
-//     4-cell band beyond the subdomain that a derivative of psi reaches,
-//     recomputed redundantly as in the per-step kernel), zeta and the update
-//     addend D1 psi + zeta on the strips widened by 4 cells. Outside the
-//     strips both recursion coefficients are zero, so everything skipped is
-//     exactly zero. x-strip work is spread over all threads (a strip is
-//     narrower than a row of warps); z-strip work follows the rows of warps,
-//     and zeta_z is fused into the update, which already holds D2z p;
-//   - sponge subdomains precompute per cell the update weights 2/(1+a),
-//     (1-a)/(1+a) and c/(1+a) (a = c eta dt / 2 is fixed in time), so the
-//     step has no division;
+//     and overwrites with p^{n+1} in place;
+//   - the CPML memory variables live in shared memory, on the strips only
+//     (RSpan): psi on the absorbing strips (and the 4-cell band beyond the
+//     subdomain that a derivative of psi reaches, recomputed redundantly as in
+//     the per-step kernel), zeta and the update addend D1 psi + zeta on the
+//     strips widened by 4 cells. Outside the strips both recursion
+//     coefficients are zero, so everything skipped is exactly zero. x-strip
+//     work is spread over all threads (a strip is narrower than a row of
+//     warps); z-strip work follows the rows of warps, and zeta_z is fused into
+//     the update, which already holds D2z p. The adjoint's multipliers nu and
+//     mu (cpml_adj.cu states their recursions) take the same places, with one
+//     phase more;
+//   - sponge subdomains of a forward solve precompute per cell the update
+//     weights 2/(1+a), (1-a)/(1+a) and c/(1+a) (a = c eta dt / 2 is fixed in
+//     time), so the step has no division; the gradient's modes round as the
+//     per-step kernels' division does (quot2, from 1/(1+a) kept per cell), so
+//     that FP16 checkpoints round the same states (with the division itself a
+//     gradient of 4 shots of 231 x 381 cells took 8.8 ms instead of 6.3);
 //   - a CTA writes the 8 (4 without CPML) border rows and columns of p^{n+1} to
-//     its outbox in global memory as 8-byte words (value, step number), as they
+//     its outbox in global memory as 8-byte words (value, step tag), as they
 //     are computed; a CTA starts step n by reading its neighbours' words, each
-//     until it carries the number n, and keeping the values as its halo. The
-//     word is one 64-bit access, so a value is never seen without its number
-//     and no fence, counter or second fetch lies on the way: the chain per step
-//     is one store, one read and a block barrier. (With a counter per
-//     subdomain - store, barrier, release, poll, barrier, fetch, barrier - the
-//     exchange alone took 2.55 us: 1000 steps of 241 x 241 cells 3.87 ms, of
-//     669 x 1100 with 100 snapshots 6.35 ms; 2.86 and 4.25 ms with the words.)
-//     The stencil is a cross, so corner
-//     neighbours are never needed.
+//     until it carries the step's tag, and keeping the values as its halo. The
+//     word is one 64-bit access, so a value is never seen without its tag and
+//     no fence, counter or second fetch lies on the way: the chain per step is
+//     one store, one read and a block barrier. (With a counter per subdomain -
+//     store, barrier, release, poll, barrier, fetch, barrier - the exchange
+//     alone took 2.55 us: 1000 steps of 241 x 241 cells 3.87 ms, of 669 x 1100
+//     with 100 snapshots 6.35 ms; 2.86 and 4.25 ms with the words.) The
+//     stencil is a cross, so corner neighbours are never needed.
 //     Two outbox halves alternate by step parity: a CTA that writes p^{n+1}
 //     over p^{n-1} has read p^n from every neighbour that reads it, and each of
-//     them sent p^n only after a barrier behind all its reads of p^{n-1}.
+//     them sent p^n only after a barrier behind all its reads of p^{n-1}. Tags
+//     never repeat between launches, so a word of an earlier run is never taken.
 // The launch is cooperative, so all CTAs are co-resident and the waits
 // always end; each wait is still bounded (spin_limit polls), after which the
 // kernel raises kFlagTimeout and every CTA returns.
 //
+// Measured (gradients, per-step kernels and this): 16 shots of 241 x 241 cells,
+// 1000 steps, CPML, FP16 checkpoints 58.3 and 24.5 ms; 4 shots of 231 x 381,
+// 600 steps, sponge, with the forward of the loss 13.0 and 6.3 ms.
+//
 // The scheme is the leapfrog update with the centred sponge term or the CPML
 // memory terms (Sec. 2, App. E.3-E.4), free surface as an odd mirror with
 // row 0 held at zero; the per-cell arithmetic is that of the per-step kernel
-// up to the order of a few additions (rounding level). Forward mode with
-// FP32 snapshots only: an FP16 snapshot's scale needs the grid-wide maximum
+// (in FP32 pairs; the same roundings but for the sponge weights above).
+// Snapshots in FP32 only: an FP16 snapshot's scale needs the grid-wide maximum
 // of the previous step, which a schedule without a grid barrier lacks.
 #include <algorithm>
 #include <cfloat>
@@ -67,21 +79,7 @@ constexpr int NWR = kResidentWarps, NTR = NWR * 32;
 // are read from global memory every step).
 constexpr int kRecCache = 128;
 
-// Shared memory (floats): two p buffers, the injection weights, then either
-// the CPML arrays (psi_x, psi_z, zeta_x, zeta_z, x addend) or the three
-// sponge update weights, then the receiver cache (index, cell offset, 4
-// weights per receiver).
-template <int RZ>
-constexpr size_t rsmem_x(int bc) {
-    constexpr size_t WZ = (size_t)NWR * RZ;
-    return bc == SIM_BC_CPML ? WZ * (TX + 8) + (WZ + 8) * TX + 3 * WZ * TX : bc == SIM_BC_SPONGE ? 3 * WZ * TX : 0;
-}
-template <int RZ>
-constexpr size_t rsmem_floats(int bc) {
-    constexpr size_t WZ = (size_t)NWR * RZ;
-    const size_t coef = bc == SIM_BC_CPML ? 2 * (TX + 8) + 2 * (WZ + 8) : 0;  // CPML a, b slices
-    return 2 * (WZ + 2 * HM) * SW + WZ * TX + rsmem_x<RZ>(bc) + coef + 6 * (size_t)kRecCache;
-}
+__device__ __forceinline__ float4 neg4(const float4 &v) { return make_float4(-v.x, -v.y, -v.z, -v.w); }
 
 // Outbox of a subdomain, one half (words): the top border rows, the bottom
 // ones, the left and the right border columns.
@@ -110,51 +108,106 @@ __device__ __forceinline__ bool get4(const unsigned long long *d, int tag, float
     return (unsigned)(a >> 32) == t && (unsigned)(b >> 32) == t && (unsigned)(c >> 32) == t && (unsigned)(e >> 32) == t;
 }
 
-// Tile-local hull [lo, hi) of the parts of the absorbing strips [0, nb0) and
-// [N - nb1, N) of one axis that fall in [clip0, clip1) (tile coordinates,
-// origin o); lo >= hi when neither strip reaches the window.
-__device__ __forceinline__ void strip_hull(int o, int N, int nb0, int nb1, int clip0, int clip1, int &lo, int &hi) {
-    lo = 1 << 30;
-    hi = -(1 << 30);
-    if (nb0 > 0) {
-        const int a = max(-o, clip0), b = min(nb0 - o, clip1);
-        if (a < b) lo = min(lo, a), hi = max(hi, b);
-    }
-    if (nb1 > 0) {
-        const int a = max(N - nb1 - o, clip0), b = min(N - o, clip1);
-        if (a < b) lo = min(lo, a), hi = max(hi, b);
-    }
+
+// The roundings of the per-step kernel's absorbing cells (fwd2d_f32.cu), which
+// the gradient's checkpoints and imaging terms depend on: the first difference
+// starts with fma(d_1, p_1 - m_1, d_2 (p_2 - m_2)); psi and zeta_z are
+// fma(a, d, b m) (rec2), zeta_x is fma(b, m, a d).
+__device__ __forceinline__ float2 d1s2(float2 m1, float2 p1, float2 m2, float2 p2, float2 m3, float2 p3, float2 m4,
+                                       float2 p4) {
+    float2 r = mul2(splat2(float(kD2)), add2(p2, neg2(m2)));
+    r = fma2(splat2(float(kD1)), add2(p1, neg2(m1)), r);
+    r = fma2(splat2(float(kD3)), add2(p3, neg2(m3)), r);
+    return fma2(splat2(float(kD4)), add2(p4, neg2(m4)), r);
+}
+__device__ __forceinline__ float2 rec2b(float2 a, float2 d, float2 b, float2 m) { return fma2(b, m, mul2(a, d)); }
+// first difference along x of the four cells C from the row's float4s L, C, R
+__device__ __forceinline__ void d1x4(const float4 &L, const float4 &C, const float4 &R, float2 &da, float2 &db) {
+    const float2 v34 = make_float2(L.w, C.x), v56 = make_float2(C.y, C.z), v12 = make_float2(L.y, L.z),
+                 v78 = make_float2(C.w, R.x), v910 = make_float2(R.y, R.z);
+    da = d1s2(v34, v56, hi2(L), hi2(C), v12, v78, lo2(L), lo2(R));
+    db = d1s2(v56, v78, lo2(C), lo2(R), v34, v910, hi2(L), hi2(R));
+}
+// and along z at p, rows of pitch ST
+template <int ST>
+__device__ __forceinline__ void d1z4(const float *p, float2 &da, float2 &db) {
+    const float4 m4 = ld4(p - 4 * ST), m3 = ld4(p - 3 * ST), m2 = ld4(p - 2 * ST), m1 = ld4(p - ST), p1 = ld4(p + ST),
+                 p2 = ld4(p + 2 * ST), p3 = ld4(p + 3 * ST), p4 = ld4(p + 4 * ST);
+    da = d1s2(lo2(m1), lo2(p1), lo2(m2), lo2(p2), lo2(m3), lo2(p3), lo2(m4), lo2(p4));
+    db = d1s2(hi2(m1), hi2(p1), hi2(m2), hi2(p2), hi2(m3), hi2(p3), hi2(m4), hi2(p4));
+}
+// second differences along x of the four cells C from the row's float4s L, C, R
+__device__ __forceinline__ void d2x_pairs(const float4 &L, const float4 &C, const float4 &R, float2 &da, float2 &db) {
+    const float2 v34 = make_float2(L.w, C.x), v56 = make_float2(C.y, C.z), v12 = make_float2(L.y, L.z),
+                 v78 = make_float2(C.w, R.x), v910 = make_float2(R.y, R.z);
+    da = d2c2(lo2(C), v34, v56, hi2(L), hi2(C), v12, v78, lo2(L), lo2(R));
+    db = d2c2(hi2(C), v56, v78, lo2(C), lo2(R), v34, v910, hi2(L), hi2(R));
 }
 
-template <int RZ>
-__global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, const ResidentArgs R) {
+// t / d correctly rounded, d >= 1, from y = RN(1/d): Markstein's theorem (IBM
+// J. Res. Dev. 34, 1990): one step from t y gives a quotient within an ulp, and
+// from such a quotient q the step RN(q + y (t - d q)) is RN(t / d), t - d q
+// being exact. Small t, whose residuals would not be exact, are scaled by
+// 2^100. Scaled back, a quotient below 2^-125 rounds a second time, onto
+// multiples of 2^-149: where that went the wrong way from a tie, the residual
+// (exact) is more than half such a step, and one step is added. Fields hold
+// such values wherever a wave has not yet arrived, and the division's own slow
+// path for them took half the time of a step.
+__device__ __forceinline__ float quot_small(float t, float d, float y) {
+    t *= 0x1p100f;
+    float q = t * y;
+    q = __fmaf_rn(__fmaf_rn(-d, q, t), y, q);
+    q = __fmaf_rn(__fmaf_rn(-d, q, t), y, q);
+    float r = q * 0x1p-100f;
+    if (fabsf(q) < 0x1p-25f) {
+        const float e = __fmaf_rn(-d, r * 0x1p100f, t), half = d * 0x1p-50f;
+        if (fabsf(e) > half) r += copysignf(0x1p-149f, e);
+    }
+    return r;
+}
+__device__ __forceinline__ float2 quot2(float2 t, float2 d, float2 y) {
+    const float mx = fabsf(t.x), my = fabsf(t.y);
+    if (!(fmaxf(mx, my) < 0x1p90f && mx + my < 0x1p91f)) return make_float2(t.x / d.x, t.y / d.y);  // huge, infinite, NaN
+    const float2 nd = neg2(d);
+    float2 q = mul2(t, y);
+    q = fma2(fma2(nd, q, t), y, q);
+    q = fma2(fma2(nd, q, t), y, q);
+    if ((mx < 0x1p-90f && mx != 0.f) || (my < 0x1p-90f && my != 0.f)) {
+        if (mx < 0x1p-90f) q.x = quot_small(t.x, d.x, y.x);
+        if (my < 0x1p-90f) q.y = quot_small(t.y, d.y, y.y);
+    }
+    return q;
+}
+
+template <int RZ, int MODE>
+__global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ StepArgs<float> A,
+                                                       const __grid_constant__ ResidentArgs R) {
     constexpr int WZ = NWR * RZ;
+    constexpr bool ADJ = MODE == kResAdjoint;
     extern __shared__ float4 smem4[];
-    const bool cpml = A.bc == SIM_BC_CPML;
+    __shared__ unsigned s_mask[2];  // rows with injected cells
+    const RLayout &Y = R.lay;
     float *const S0 = reinterpret_cast<float *>(smem4);
     float *const S1 = S0 + (WZ + 2 * HM) * SW;
-    float *const INJ = S1 + (WZ + 2 * HM) * SW;    // WZ x TX: injection weight per cell
-    float *const X0 = INJ + WZ * TX;
-    // CPML
-    float *const PX = X0;                          // WZ x (TX + 8): psi_x, cells [-4, TX + 4)
-    float *const PZ = PX + WZ * (TX + 8);          // (WZ + 8) x TX: psi_z, rows [-4, WZ + 4)
-    float *const ZX = PZ + (WZ + 8) * TX;          // WZ x TX: zeta_x
-    float *const ZZ = ZX + WZ * TX;                // WZ x TX: zeta_z
-    float *const AX = ZZ + WZ * TX;                // WZ x TX: D1x psi_x + zeta_x
-    // sponge update weights
-    float *const KA = X0, *const KB = X0 + WZ * TX, *const KC = X0 + 2 * WZ * TX;
-    // CPML recursion coefficients of the subdomain: x in [-4, TX + 4), rows [-4, WZ + 4)
-    float *const CAX = X0 + rsmem_x<RZ>(A.bc), *const CBX = CAX + TX + 8;
-    float *const CAZ = CBX + TX + 8, *const CBZ = CAZ + WZ + 8;
-    // receiver cache
-    int *const RIDX = reinterpret_cast<int *>(X0 + rsmem_x<RZ>(A.bc) + (cpml ? 2 * (TX + 8) + 2 * (WZ + 8) : 0));
+    float *const CC = S0 + Y.c;     // WZ x TX: c
+    float *const F1 = S0 + Y.f1;    // x strips: psi / nu, chunks [p0, p1)
+    float *const F2 = S0 + Y.f2;    // x strips: zeta (own chunks) / mu, chunks [q0, q1)
+    float *const AX = S0 + Y.ax;    // x strips: the term, own chunks [a0, a1)
+    float *const Z1 = S0 + Y.z1;    // z strips: psi / nu, rows [zp0, zp1)
+    float *const Z2 = S0 + Y.z2;    // z strips: zeta (own rows) / mu, rows [zq0, zq1)
+    float *const GG = S0 + Y.G;     // adjoint: WZ x TX gradient sums
+    float *const KA = S0 + Y.K, *const KB = KA + WZ * TX, *const KC = KB + WZ * TX;  // sponge update weights (exact: KA = 1/(1+a))
+    float *const INJ = S0 + Y.inj;  // injected weights (adjoint: values, two halves) of the flagged rows
+    // CPML recursion coefficients: x cells [-8, TX + 8), rows [-8, WZ + 8)
+    float *const CAX = S0 + Y.coef, *const CBX = CAX + TX + 16, *const CAZ = CBX + TX + 16, *const CBZ = CAZ + WZ + 16;
+    int *const RIDX = reinterpret_cast<int *>(S0 + Y.rec);  // receiver cache
     int *const ROFF = RIDX + kRecCache;
     float *const RW = reinterpret_cast<float *>(ROFF + kRecCache);
 
     const Geom &g = A.g;
+    const bool cpml = R.m2[0] || R.m2[1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, tid = threadIdx.x;
-    const int ntiles = R.ntiles;
-    const int shot = blockIdx.x / ntiles, tile = blockIdx.x - shot * ntiles;
+    const int ntiles = R.ntiles, lshot = blockIdx.x / ntiles, tile = blockIdx.x - lshot * ntiles, shot = R.shot0 + lshot;
     const RTile *const D = R.tiles + tile;
     const int bx = D->bx, x0 = bx * TX, z0 = D->z0, rows = D->rows, rpw = D->rpw, P = g.P;
     const long long sh = (long long)shot * g.fstride;
@@ -163,10 +216,9 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
     float *const gb1 = A.pbuf[1] + sh + org;
     unsigned long long *const outbox = R.outbox + (long long)blockIdx.x * kResidentOutbox;
 
-    const bool cpx = cpml && A.ca[2] &&
-                     ((g.nbx0 > 0 && x0 - 4 < g.nbx0) || (g.nbx1 > 0 && x0 + TX + 4 > g.NX - g.nbx1));
-    const bool cpz = cpml && A.ca[0] &&
-                     ((g.nbz0 > 0 && z0 - 4 < g.nbz0) || (g.nbz1 > 0 && z0 + rows + 4 > g.NZ - g.nbz1));
+    const RSpan sp = resident_span(g, cpml ? (int)SIM_BC_CPML : (int)SIM_BC_NONE, bx, z0, rows, ADJ);
+    const int ncx = sp.c1 - sp.c0, nax = sp.a1 - sp.a0;
+    const bool hasx = ncx > 0 && A.ca[2], hasz = sp.zc1 > sp.zc0 && A.ca[0];
     const bool spg = A.bc == SIM_BC_SPONGE &&
                      ((g.nbx0 > 0 && x0 < g.nbx0) || (g.nbx1 > 0 && x0 + TX > g.NX - g.nbx1) ||
                       (g.nbz0 > 0 && z0 < g.nbz0) || (g.nbz1 > 0 && z0 + rows > g.NZ - g.nbz1));
@@ -177,91 +229,153 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
     const int c0 = HM + 4 * lane, gx0 = x0 + 4 * lane, rb = HM + w * rpw;
     const int lo = w * rpw * P + 4 * lane;
 
-    // CPML work ranges. x: psi on float4 chunks cx0 <= c < cx1 of PX (chunk c
-    // holds cells [4c - 4, 4c)), zeta_x / addend on own chunks [ax0, ax1).
-    // z: psi on rows [zp0, zp1) of [-4, rows + 4), zeta_z on rows [zz0, zz1).
-    int cx0 = 0, cx1 = 0, ax0 = 0, ax1 = 0, zp0 = 0, zp1 = 0, zz0 = 0, zz1 = 0;
-    if (cpx) {
-        int plo, phi;
-        strip_hull(x0, g.NX, g.nbx0, g.nbx1, -4, TX + 4, plo, phi);
-        if (plo < phi) {
-            cx0 = (plo + 4) >> 2;
-            cx1 = (phi + 4 + 3) >> 2;
-            ax0 = max(0, plo - 4) >> 2;
-            ax1 = (min(TX, phi + 4) + 3) >> 2;
-        }
-    }
-    if (cpz) {
-        strip_hull(z0, g.NZ, g.nbz0, g.nbz1, -4, rows + 4, zp0, zp1);
-        if (zp0 < zp1) {
-            zz0 = max(0, zp0 - 4);
-            zz1 = min(rows, zp1 + 4);
-        } else {
-            zp0 = zp1 = 0;
-        }
-    }
-    const int ncx = cx1 - cx0, nax = ax1 - ax0;
-
     // Shared memory starts at zero: the halo of an absent neighbour, the rows
     // and columns beyond the grid and every CPML value outside the strips.
-    {
-        const int n4 = (int)(rsmem_floats<RZ>(A.bc) / 4);
-        for (int i = tid; i < n4; i += NTR) smem4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    for (int i = tid; i < Y.total / 4; i += NTR) smem4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid < 2) s_mask[tid] = 0u;
+    __syncthreads();
 
-    // run constants of the thread's own cells
-    float4 ch4[RZ];
+    // run constants
 #pragma unroll
     for (int j = 0; j < RZ; j++) {
-        const bool in = j < rpw && w * rpw + j < rows;
-        ch4[j] = in ? __ldg(reinterpret_cast<const float4 *>(A.ch + org + lo + j * P)) : make_float4(0, 0, 0, 0);
-    }
-    if (cpml) {
-        for (int i = tid; i < TX + 8; i += NTR) {
-            CAX[i] = A.ca[2] ? A.ca[2][x0 - 4 + i] : 0.f;
-            CBX[i] = A.cb[2] ? A.cb[2][x0 - 4 + i] : 0.f;
+        const int lz = w * rpw + j;
+        if (j < rpw && lz < rows) {
+            cp_async16(CC + lz * TX + 4 * lane, A.ch + org + lo + j * P);
+            if (ADJ) cp_async16(GG + lz * TX + 4 * lane, A.G + sh + org + lo + j * P);
         }
-        for (int i = tid; i < WZ + 8; i += NTR) {
-            const int gz = z0 - 4 + i;
+    }
+    if (spg && R.exact_sponge)
+        for (int i = tid; i < rows; i += NTR) CAZ[i + 8] = A.E[0][z0 + i];
+    if (cpml) {
+        for (int i = tid; i < TX + 16; i += NTR) {
+            CAX[i] = A.ca[2] ? A.ca[2][x0 - 8 + i] : 0.f;
+            CBX[i] = A.cb[2] ? A.cb[2][x0 - 8 + i] : 0.f;
+        }
+        for (int i = tid; i < WZ + 16; i += NTR) {
+            const int gz = z0 - 8 + i;
             const bool in = A.ca[0] && gz >= 0 && gz < g.NZ;
             CAZ[i] = in ? A.ca[0][gz] : 0.f;
             CBZ[i] = in ? A.cb[0][gz] : 0.f;
         }
     }
+    if (R.load) {  // p^n0 with its halo, p^{n0-1}, the memory fields
+        const float *pc = (R.n0 & 1) ? gb1 : gb0, *pm = (R.n0 & 1) ? gb0 : gb1;
+        for (int r = w - HM; r < rows + HM; r += NWR) {
+            cp_async16(S0 + (HM + r) * SW + 4 * lane, pc + (long long)r * P - HM + 4 * lane);
+            if (lane < 4) cp_async16(S0 + (HM + r) * SW + 128 + 4 * lane, pc + (long long)r * P - HM + 128 + 4 * lane);
+            if (r >= 0 && r < rows) cp_async16(S1 + (HM + r) * SW + c0, pm + (long long)r * P + 4 * lane);
+        }
+        if (hasx) {
+            const float *m1 = R.m1i[0] + sh + org, *m2 = R.m2[0] + sh + org;
+            for (int i = tid; i < rows * ncx; i += NTR) {
+                const int lz = i / ncx, c = sp.c0 + i - lz * ncx;
+                cp_async16(F1 + lz * Y.w1 + 4 * (c - sp.p0), m1 + (long long)lz * P + 4 * c - 8);
+            }
+            const int b0 = ADJ ? sp.m0 : sp.a0, nb = (ADJ ? sp.m1 : sp.a1) - b0, off = ADJ ? sp.q0 : sp.a0;
+            for (int i = tid; i < rows * nb; i += NTR) {
+                const int lz = i / nb, c = b0 + i - lz * nb;
+                cp_async16(F2 + lz * Y.w2 + 4 * (c - off), m2 + (long long)lz * P + 4 * c - 8);
+            }
+        }
+        if (hasz) {
+            const float *m1 = R.m1i[1] + sh + org, *m2 = R.m2[1] + sh + org;
+            for (int r = sp.zc0 + w; r < sp.zc1; r += NWR)
+                cp_async16(Z1 + (r - sp.zp0) * TX + 4 * lane, m1 + (long long)r * P + 4 * lane);
+            const int b0 = ADJ ? sp.zm0 : sp.za0, b1 = ADJ ? sp.zm1 : sp.za1, off = ADJ ? sp.zq0 : sp.za0;
+            for (int r = b0 + w; r < b1; r += NWR)
+                cp_async16(Z2 + (r - off) * TX + 4 * lane, m2 + (long long)r * P + 4 * lane);
+        }
+    }
+    cp_async_wait_all();
     __syncthreads();
-    if (spg) {  // sponge: out = KA p - KB p^{n-1} + KC rhs, a = c (eta_z + eta_x)
-        const float4 E4 = __ldg(reinterpret_cast<const float4 *>(A.E[2] + gx0));
+    float4 E4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (spg) {
+        E4 = __ldg(reinterpret_cast<const float4 *>(A.E[2] + gx0));
+        // out = KA p - KB p^{n-1} + KC rhs, a = c (eta_z + eta_x); exact: KA = 1/(1+a)
 #pragma unroll
         for (int j = 0; j < RZ; j++) {
             const int lz = w * rpw + j, gz = z0 + lz;
             if (j >= rpw || lz >= rows) continue;
             const float ez = A.E[0][gz];
+            const float4 c4 = ld4(CC + lz * TX + 4 * lane);
             float ka[4], kb[4], kc[4];
 #pragma unroll
             for (int k = 0; k < 4; k++) {
-                const float chv = lane_of(ch4[j], k), a = chv * (ez + lane_of(E4, k)), inv = 1.f / (1.f + a);
-                ka[k] = 2.f * inv;
+                const float chv = lane_of(c4, k), es = ez + lane_of(E4, k), a = chv * es, inv = 1.f / (1.f + a);
+                ka[k] = R.exact_sponge ? 1.f / __fmaf_rn(chv, es, 1.f) : 2.f * inv;
                 kb[k] = (1.f - a) * inv;
                 kc[k] = chv * inv;
             }
             st4(KA + lz * TX + 4 * lane, make_float4(ka[0], ka[1], ka[2], ka[3]));
+            if (R.exact_sponge) continue;
             st4(KB + lz * TX + 4 * lane, make_float4(kb[0], kb[1], kb[2], kb[3]));
             st4(KC + lz * TX + 4 * lane, make_float4(kc[0], kc[1], kc[2], kc[3]));
         }
     }
-    // Point sources: the injected value of a target cell at step n is its
-    // weight (sum of its entries' weights) times w(n); the target cells are
-    // fixed, so their weights are set once and the step only scales them.
+    // Injection: the target cells are fixed, so their rows are found once. A
+    // point source's value is its weight times w(n); the adjoint's values are
+    // sums of residuals, formed a step ahead into the other half of INJ.
+    const SimIO *io = A.io;
     const int itile = A.inj_per_shot ? shot * ntiles + tile : tile;
     const int g0 = A.inj_start[itile], g1 = A.inj_start[itile + 1];
     const bool has_inj = g1 > g0;
     for (int gi = g0 + tid; gi < g1; gi += NTR) {
-        const InjGroup G = A.inj_grp[gi];
-        float wsum = 0.f;
-        for (int e = G.e0; e < G.e1; e++) wsum += A.inj_ent[e].w;
-        INJ[G.cell] = wsum;
+        const int lz = A.inj_grp[gi].cell >> 7;
+        atomicOr(&s_mask[lz >> 5], 1u << (lz & 31));
     }
-    const int r0 = A.sample ? A.rec_start[tile] : 0, r1 = A.sample ? A.rec_start[tile + 1] : 0;
+    __syncthreads();
+    const unsigned mask0 = s_mask[0], mask1 = s_mask[1];
+    auto inj_row = [&](int lz) {  // place of a flagged row
+        return lz < 32 ? __popc(mask0 & ((1u << lz) - 1u)) : __popc(mask0) + __popc(mask1 & ((1u << (lz - 32)) - 1u));
+    };
+    auto inj_flag = [&](int lz) { return ((lz < 32 ? mask0 >> lz : mask1 >> (lz - 32)) & 1u) != 0u; };
+    // adjoint: the values of sweep step n (gather row nt - n). A thread's first
+    // cell, of one or two entries, has them in registers, and the residuals of
+    // the next step are fetched while this one waits for its borders.
+    int gplace = -1, gpt0 = 0, gpt1 = 0;
+    float gw0 = 0.f, gw1 = 0.f, gr0 = 0.f, gr1 = 0.f;
+    if (ADJ && g0 + tid < g1) {
+        const InjGroup G = A.inj_grp[g0 + tid];
+        if (G.e1 - G.e0 <= 2) {
+            gplace = inj_row(G.cell >> 7) * TX + (G.cell & 127);
+            gpt0 = gpt1 = A.inj_ent[G.e0].pt;
+            gw0 = A.inj_ent[G.e0].w;
+            if (G.e1 - G.e0 == 2) gpt1 = A.inj_ent[G.e0 + 1].pt, gw1 = A.inj_ent[G.e0 + 1].w;
+        }
+    }
+    auto resid_row = [&](int n) {
+        return static_cast<const float *>(io->resid) + ((long long)shot * A.nt + A.nt - n) * io->nrec;
+    };
+    auto fetch_residuals = [&](int n) {
+        gr0 = gr1 = 0.f;
+        if (gplace < 0 || n < 1) return;
+        gr0 = resid_row(n)[gpt0];
+        if (gw1 != 0.f) gr1 = resid_row(n)[gpt1];
+    };
+    auto residuals = [&](int n) {
+        float *const half = INJ + (n & 1) * Y.injr * TX;
+        if (gplace >= 0) half[gplace] = __fmaf_rn(gw1, gr1, gw0 * gr0);
+        for (int gi = g0 + tid + (gplace >= 0 ? NTR : 0); gi < g1; gi += NTR) {
+            const InjGroup G = A.inj_grp[gi];
+            float sum = 0.f;
+            if (n >= 1)
+                for (int e = G.e0; e < G.e1; e++) sum += A.inj_ent[e].w * resid_row(n)[A.inj_ent[e].pt];
+            half[inj_row(G.cell >> 7) * TX + (G.cell & 127)] = sum;
+        }
+    };
+    if (ADJ) {
+        fetch_residuals(R.n0);
+        residuals(R.n0);
+    } else {
+        for (int gi = g0 + tid; gi < g1; gi += NTR) {
+            const InjGroup G = A.inj_grp[gi];
+            float wsum = 0.f;
+            for (int e = G.e0; e < G.e1; e++) wsum += A.inj_ent[e].w;
+            INJ[inj_row(G.cell >> 7) * TX + (G.cell & 127)] = wsum;
+        }
+    }
+    const bool sample = MODE == kResForward && A.sample;
+    const int r0 = sample ? A.rec_start[tile] : 0, r1 = sample ? A.rec_start[tile + 1] : 0;
     const bool rec_cached = r1 - r0 <= kRecCache;
     if (rec_cached)
         for (int e = r0 + tid; e < r1; e += NTR) {
@@ -275,7 +389,7 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
     // rows of the subdomain above, rows >= rows from the top rows of the one
     // below (a last one of fewer than H rows has no more: zeros), columns left
     // and right from the subdomains of the adjacent columns that hold the row.
-    int xsrc[2] = {-1, -1}, xdst[2] = {0, 0};
+    int xsrc[2] = {-1, -1}, xdst[2] = {0, 0}, xmir[2] = {-1, -1};  // xmir: the float4's place above the free surface
     {
         const int hq = H / 4, nN = hasN ? 32 * H : 0;
         int up = -1, down = -1;
@@ -289,20 +403,20 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
             for (int k = 0; k < D->nnbr; k++) {
                 const RTile &u = R.tiles[D->nbr[k]];
                 if (u.bx == bx + dx && gz >= u.z0 && gz < u.z0 + u.rows)
-                    return (shot * ntiles + D->nbr[k]) * kResidentOutbox + (gz - u.z0) * HM;
+                    return (lshot * ntiles + D->nbr[k]) * kResidentOutbox + (gz - u.z0) * HM;
             }
             return -1;
         };
         for (int v = 0; v < 2; v++) {
             int i = tid + v * NTR;
             if (i < nN) {
-                xsrc[v] = (shot * ntiles + up) * kResidentOutbox + XS + i * 4;
+                xsrc[v] = (lshot * ntiles + up) * kResidentOutbox + XS + i * 4;
                 xdst[v] = (HM - H + (i >> 5)) * SW + HM + 4 * (i & 31);
                 continue;
             }
             i -= nN;
             if (i < nS) {
-                xsrc[v] = (shot * ntiles + down) * kResidentOutbox + XN + i * 4;
+                xsrc[v] = (lshot * ntiles + down) * kResidentOutbox + XN + i * 4;
                 xdst[v] = (HM + rows + (i >> 5)) * SW + HM + 4 * (i & 31);
                 continue;
             }
@@ -311,6 +425,7 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
                 const int r = i / hq, q = i - r * hq, o = side(-1, z0 + r);
                 xsrc[v] = o < 0 ? -1 : o + XEST + 4 * q;
                 xdst[v] = (HM + r) * SW + HM - H + 4 * q;
+                if (top && r >= 1 && r <= H) xmir[v] = xdst[v] - 2 * r * SW;
                 continue;
             }
             i -= nW;
@@ -318,38 +433,72 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
                 const int r = i / hq, q = i - r * hq, o = side(1, z0 + r);
                 xsrc[v] = o < 0 ? -1 : o + XWST + 4 * q;
                 xdst[v] = (HM + r) * SW + HM + TX + 4 * q;
+                if (top && r >= 1 && r <= H) xmir[v] = xdst[v] - 2 * r * SW;
             }
         }
     }
     static_assert(2 * HM * 32 + 2 * 64 * (HM / 4) <= 2 * NTR, "two halo float4s per thread at most");
-    const SimIO *io = A.io;
     const float *const wav = static_cast<const float *>(io->wavelet);
     float *const gout = static_cast<float *>(io->gather);
-    float *const snaps = static_cast<float *>(io->snaps);
+    float *const snaps = MODE == kResForward ? static_cast<float *>(io->snaps) : nullptr;
     const int nrec = io->nrec;
-    float wnext = (has_inj && A.nt > 0) ? wav[0] : 0.f;
+    if (top && R.load)  // odd mirror above the free surface: p(-k) = -p(k); later steps write it with p(k)
+        for (int k = 1 + w; k <= H; k += NWR)
+            for (int c = HM - H + 4 * lane; c < HM + TX + H; c += 128)
+                st4(S0 + (HM - k) * SW + c, neg4(ld4(S0 + (HM + k) * SW + c)));
+    float wnext = (!ADJ && has_inj && R.n0 < R.n1) ? wav[R.n0] : 0.f;
     __syncthreads();
 
-    for (int n = 0; n < A.nt; n++) {
-        float *const cur = (n & 1) ? S1 : S0;
-        float *const nxt = (n & 1) ? S0 : S1;
+    for (int n = R.n0; n < R.n1; n++) {
+        const int par = (n - R.n0) & 1;
+        const unsigned tag = R.tag0 + (unsigned)(n - R.n0);
+        float *const cur = par ? S1 : S0;
+        float *const nxt = par ? S0 : S1;
+
         // this step's wavelet sample (fetched one step ahead)
         const float wn = wnext;
-        if (has_inj && n + 1 < A.nt) wnext = wav[n + 1];
+        if (!ADJ && has_inj && n + 1 < R.n1) wnext = wav[n + 1];
+        // this step's imaging terms, in flight during the wait
+        const long long slot = MODE == kResRecord ? n - R.n0 : R.n1 - 1 - n;
+        char *const qs = R.q + slot * R.qstride;
+        // FP16 slots: a warp's scale lies in the shot's top ghost rows, which hold nothing else
+        float *const qsc = reinterpret_cast<float *>(reinterpret_cast<__half *>(qs) + sh) + tile * NWR + w;
+        float4 qv[RZ];
+        if (MODE == kResAdjoint) {
+            const float s = A.q_fp16 ? *qsc : 1.f;
+#pragma unroll
+            for (int j = 0; j < RZ; j++) {
+                qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (j >= rpw || w * rpw + j >= rows) continue;
+                const long long o = sh + org + lo + j * P;
+                if (A.q_fp16) {
+                    const uint2 u = *reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(qs) + o);
+                    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&u.x)),
+                                 b = __half22float2(*reinterpret_cast<const __half2 *>(&u.y));
+                    qv[j] = make_float4(a.x * s, a.y * s, b.x * s, b.y * s);
+                } else {
+                    qv[j] = ld4(reinterpret_cast<const float *>(qs) + o);
+                }
+            }
+        }
+
+        if (ADJ && has_inj && n + 1 < R.n1) fetch_residuals(n + 1);
 
         bool quit = false;
-        if (n > 0) {  // the neighbours' borders of p^n become this step's halo
-            const unsigned long long *const in = R.outbox + (n & 1) * XHALF;
+        if (n > R.n0) {  // the neighbours' borders of p^n become this step's halo
+            const unsigned long long *const in = R.outbox + par * XHALF;
             bool need0 = xsrc[0] >= 0, need1 = xsrc[1] >= 0;
             for (long long spins = 0; need0 || need1;) {
                 float4 v0, v1;
-                const bool ok0 = need0 && get4(in + xsrc[0], n, v0), ok1 = need1 && get4(in + xsrc[1], n, v1);
+                const bool ok0 = need0 && get4(in + xsrc[0], tag, v0), ok1 = need1 && get4(in + xsrc[1], tag, v1);
                 if (ok0) {
                     st4(cur + xdst[0], v0);
+                    if (xmir[0] >= 0) st4(cur + xmir[0], neg4(v0));
                     need0 = false;
                 }
                 if (ok1) {
                     st4(cur + xdst[1], v1);
+                    if (xmir[1] >= 0) st4(cur + xmir[1], neg4(v1));
                     need1 = false;
                 }
                 if (!(need0 || need1)) break;
@@ -365,153 +514,223 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
             }
         }
         if (__syncthreads_or(quit)) return;
-        if (top && n > 0) {  // odd mirror above the free surface: p(-k) = -p(k)
-            const int nch = (TX + 2 * H) / 4;
-            for (int k = 1 + w; k <= H; k += NWR) {
-                float4 *d = reinterpret_cast<float4 *>(cur + (HM - k) * SW + (HM - H));
-                const float4 *sr = reinterpret_cast<const float4 *>(cur + (HM + k) * SW + (HM - H));
-                for (int c = lane; c < nch; c += 32) {
-                    const float4 v = sr[c];
-                    d[c] = make_float4(-v.x, -v.y, -v.z, -v.w);
+        if (!ADJ) {
+            // CPML psi^n = b psi^{n-1} + a D1 p^n (scaled by h) on the strips
+            if (hasx)
+                for (int i = tid; i < rows * ncx; i += NTR) {
+                    const int lz = i / ncx, c = sp.c0 + (i - lz * ncx);
+                    const float *row = cur + (HM + lz) * SW + 4 * c;
+                    const float4 a4 = ld4(CAX + 4 * c), b4 = ld4(CBX + 4 * c);
+                    float *px = F1 + lz * Y.w1 + 4 * (c - sp.p0);
+                    const float4 old = ld4(px);
+                    float2 da, db;
+                    d1x4(ld4(row - 4), ld4(row), ld4(row + 4), da, db);
+                    const float2 pa = rec2(lo2(a4), da, lo2(b4), lo2(old)), pb = rec2(hi2(a4), db, hi2(b4), hi2(old));
+                    st4(px, make_float4(pa.x, pa.y, pb.x, pb.y));
+                }
+            if (hasz)
+                for (int r = sp.zc0 + w; r < sp.zc1; r += NWR) {
+                    const float *col = cur + (HM + r) * SW + c0;
+                    float2 da, db;
+                    d1z4<SW>(col, da, db);
+                    const float2 a2 = splat2(CAZ[r + 8]), b2 = splat2(CBZ[r + 8]);
+                    float *pz = Z1 + (r - sp.zp0) * TX + 4 * lane;
+                    const float4 old = ld4(pz);
+                    const float2 pa = rec2(a2, da, b2, lo2(old)), pb = rec2(a2, db, b2, hi2(old));
+                    st4(pz, make_float4(pa.x, pa.y, pb.x, pb.y));
+                }
+            if (hasx || hasz) __syncthreads();
+            // zeta_x^n = b zeta_x^{n-1} + a (D2x p^n + D1x psi_x^n) and the addend
+            // D1x psi_x^n + zeta_x^n on the widened x-strips
+            if (hasx && nax > 0) {
+                for (int i = tid; i < rows * nax; i += NTR) {
+                    const int lz = i / nax, c = sp.a0 + (i - lz * nax);
+                    const float *row = cur + (HM + lz) * SW + 4 * c, *px = F1 + lz * Y.w1 + 4 * (c - sp.p0);
+                    const float4 a4 = ld4(CAX + 4 * c), b4 = ld4(CBX + 4 * c);
+                    float *zp = F2 + lz * Y.w2 + 4 * (c - sp.a0);
+                    const float4 z4 = ld4(zp);
+                    float2 xa, xb, da, db;
+                    d2x_pairs(ld4(row - 4), ld4(row), ld4(row + 4), xa, xb);
+                    d1x4(ld4(px - 4), ld4(px), ld4(px + 4), da, db);
+                    const float2 za = rec2b(lo2(a4), add2(xa, da), lo2(b4), lo2(z4));
+                    const float2 zb = rec2b(hi2(a4), add2(xb, db), hi2(b4), hi2(z4));
+                    st4(zp, make_float4(za.x, za.y, zb.x, zb.y));
+                    const float2 ea = add2(da, za), eb = add2(db, zb);
+                    st4(AX + lz * Y.wa + 4 * (c - sp.a0), make_float4(ea.x, ea.y, eb.x, eb.y));
+                }
+                __syncthreads();
+            }
+        } else if (hasx || hasz) {
+            // nu^k = b nu^{k+1} + u^{k+1}
+            if (hasx)
+                for (int i = tid; i < rows * ncx; i += NTR) {
+                    const int lz = i / ncx, c = sp.c0 + (i - lz * ncx);
+                    const float4 u = ld4(cur + (HM + lz) * SW + 4 * c), b4 = ld4(CBX + 4 * c);
+                    float *px = F1 + lz * Y.w1 + 4 * (c - sp.p0);
+                    const float4 old = ld4(px);
+                    const float2 na = fma2(lo2(b4), lo2(old), lo2(u)), nb = fma2(hi2(b4), hi2(old), hi2(u));
+                    st4(px, make_float4(na.x, na.y, nb.x, nb.y));
+                }
+            if (hasz)
+                for (int r = sp.zc0 + w; r < sp.zc1; r += NWR) {
+                    const float4 u = ld4(cur + (HM + r) * SW + c0);
+                    const float2 b2 = splat2(CBZ[r + 8]);
+                    float *pz = Z1 + (r - sp.zp0) * TX + 4 * lane;
+                    const float4 old = ld4(pz);
+                    const float2 na = fma2(b2, lo2(old), lo2(u)), nb = fma2(b2, hi2(old), hi2(u));
+                    st4(pz, make_float4(na.x, na.y, nb.x, nb.y));
+                }
+            __syncthreads();
+            // mu^k = b mu^{k+1} - D1 (u^{k+1} + a nu^k)
+            if (hasx && sp.m1 > sp.m0) {
+                const int nm = sp.m1 - sp.m0;
+                auto wx = [&](const float *row, const float *px, int c) {  // u + a nu of chunk c
+                    const float4 u = ld4(row), nu = ld4(px), a4 = ld4(CAX + 4 * c);
+                    const float2 wa = fma2(lo2(a4), lo2(nu), lo2(u)), wb = fma2(hi2(a4), hi2(nu), hi2(u));
+                    return make_float4(wa.x, wa.y, wb.x, wb.y);
+                };
+                for (int i = tid; i < rows * nm; i += NTR) {
+                    const int lz = i / nm, c = sp.m0 + (i - lz * nm);
+                    const float *row = cur + (HM + lz) * SW + 4 * c, *px = F1 + lz * Y.w1 + 4 * (c - sp.p0);
+                    const float4 b4 = ld4(CBX + 4 * c);
+                    float *mp = F2 + lz * Y.w2 + 4 * (c - sp.q0);
+                    const float4 old = ld4(mp);
+                    float2 da, db;
+                    d1x_pairs(wx(row - 4, px - 4, c - 1), wx(row, px, c), wx(row + 4, px + 4, c + 1), da, db);
+                    const float2 ma = fma2(lo2(b4), lo2(old), neg2(da)), mb = fma2(hi2(b4), hi2(old), neg2(db));
+                    st4(mp, make_float4(ma.x, ma.y, mb.x, mb.y));
+                }
+            }
+            if (hasz && sp.zm1 > sp.zm0) {
+                auto wz = [&](int r) {
+                    const float4 u = ld4(cur + (HM + r) * SW + c0), nu = ld4(Z1 + (r - sp.zp0) * TX + 4 * lane);
+                    const float2 a2 = splat2(CAZ[r + 8]);
+                    const float2 wa = fma2(a2, lo2(nu), lo2(u)), wb = fma2(a2, hi2(nu), hi2(u));
+                    return make_float4(wa.x, wa.y, wb.x, wb.y);
+                };
+                for (int r = sp.zm0 + w; r < sp.zm1; r += NWR) {
+                    float2 da, db;
+                    d1_pairs(wz(r - 4), wz(r - 3), wz(r - 2), wz(r - 1), wz(r + 1), wz(r + 2), wz(r + 3), wz(r + 4), da, db);
+                    const float2 b2 = splat2(CBZ[r + 8]);
+                    float *mp = Z2 + (r - sp.zq0) * TX + 4 * lane;
+                    const float4 old = ld4(mp);
+                    const float2 ma = fma2(b2, lo2(old), neg2(da)), mb = fma2(b2, hi2(old), neg2(db));
+                    st4(mp, make_float4(ma.x, ma.y, mb.x, mb.y));
                 }
             }
             __syncthreads();
-        }
-
-        // CPML psi^n = b psi^{n-1} + a D1 p^n (scaled by h) on the strips
-        if (ncx > 0) {
-            for (int i = tid; i < rows * ncx; i += NTR) {
-                const int lz = i / ncx, c = cx0 + (i - lz * ncx), gz = z0 + lz, gx = x0 + 4 * c - 4;
-                const float *row = cur + (HM + lz) * SW + HM + 4 * c - 4;
-                float v[12];
-                unpack3(ld4(row - 4), ld4(row), ld4(row + 4), v);
-                const float4 a4 = ld4(CAX + 4 * c), b4 = ld4(CBX + 4 * c);
-                float *px = PX + lz * (TX + 8) + 4 * c;
-                const float4 old = ld4(px);
-                float o4[4];
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    const bool in = gz < g.NZ && gx + k >= 0 && gx + k < g.NX;
-                    o4[k] = in ? lane_of(b4, k) * lane_of(old, k) + lane_of(a4, k) * d1w(v, k) : 0.f;
+            // the bracket of the x axis: D2 (a nu) - D1 (a mu)
+            if (hasx && nax > 0) {
+                auto am = [&](const float *p, int c) {
+                    const float4 v = ld4(p), a4 = ld4(CAX + 4 * c);
+                    return make_float4(a4.x * v.x, a4.y * v.y, a4.z * v.z, a4.w * v.w);
+                };
+                for (int i = tid; i < rows * nax; i += NTR) {
+                    const int lz = i / nax, c = sp.a0 + (i - lz * nax);
+                    const float *np = F1 + lz * Y.w1 + 4 * (c - sp.p0), *mp = F2 + lz * Y.w2 + 4 * (c - sp.q0);
+                    float2 xa, xb, da, db;
+                    d2x_pairs(am(np - 4, c - 1), am(np, c), am(np + 4, c + 1), xa, xb);
+                    d1x_pairs(am(mp - 4, c - 1), am(mp, c), am(mp + 4, c + 1), da, db);
+                    st4(AX + lz * Y.wa + 4 * (c - sp.a0),
+                        make_float4(xa.x - da.x, xa.y - da.y, xb.x - db.x, xb.y - db.y));
                 }
-                st4(px, make_float4(o4[0], o4[1], o4[2], o4[3]));
+                __syncthreads();
             }
         }
-        if (zp1 > zp0) {
-            for (int lzz = zp0 + w; lzz < zp1; lzz += NWR) {
-                const int gz = z0 + lzz;
-                const float *col = cur + (HM + lzz) * SW + c0;
-                float4 q[9];
-#pragma unroll
-                for (int m = 0; m < 9; m++) q[m] = ld4(col + (m - 4) * SW);
-                const bool zin = gz >= 0 && gz < g.NZ;
-                const float az = CAZ[lzz + 4], bz = CBZ[lzz + 4];
-                float *pz = PZ + (lzz + 4) * TX + 4 * lane;
-                const float4 old = ld4(pz);
-                float o4[4];
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    const float d1 = float(kD1) * (lane_of(q[5], k) - lane_of(q[3], k)) +
-                                     float(kD2) * (lane_of(q[6], k) - lane_of(q[2], k)) +
-                                     float(kD3) * (lane_of(q[7], k) - lane_of(q[1], k)) +
-                                     float(kD4) * (lane_of(q[8], k) - lane_of(q[0], k));
-                    o4[k] = (zin && gx0 + k < g.NX) ? bz * lane_of(old, k) + az * d1 : 0.f;
-                }
-                st4(pz, make_float4(o4[0], o4[1], o4[2], o4[3]));
-            }
-        }
-        if (ncx > 0 || zp1 > zp0) __syncthreads();
 
-        // zeta_x^n = b zeta_x^{n-1} + a (D2x p^n + D1x psi_x^n) and the addend
-        // D1x psi_x^n + zeta_x^n on the widened x-strips
-        if (nax > 0) {
-            for (int i = tid; i < rows * nax; i += NTR) {
-                const int lz = i / nax, c = ax0 + (i - lz * nax);
-                float v[12], px[12];
-                const float *row = cur + (HM + lz) * SW + HM + 4 * c;
-                unpack3(ld4(row - 4), ld4(row), ld4(row + 4), v);
-                const float *pr = PX + lz * (TX + 8) + 4 * c;
-                unpack3(ld4(pr), ld4(pr + 4), ld4(pr + 8), px);
-                const float4 a4 = ld4(CAX + 4 * c + 4), b4 = ld4(CBX + 4 * c + 4);
-                float *zp = ZX + lz * TX + 4 * c;
-                const float4 z4 = ld4(zp);
-                float zo[4], ad[4];
-#pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    const float dps = d1w(px, k);
-                    zo[k] = lane_of(b4, k) * lane_of(z4, k) + lane_of(a4, k) * (d2w(v, k) + dps);
-                    ad[k] = dps + zo[k];
-                }
-                st4(zp, make_float4(zo[0], zo[1], zo[2], zo[3]));
-                st4(AX + lz * TX + 4 * c, make_float4(ad[0], ad[1], ad[2], ad[3]));
-            }
-            __syncthreads();
-        }
-
-        // update: p^{n+1} into the other buffer, borders to the global buffer
+        // update: p^{n+1} into the other buffer, borders to the outbox
         float4 zw[RZ + 8];
 #pragma unroll
         for (int j = 0; j < RZ + 8; j++) zw[j] = ld4(cur + (rb - 4 + j) * SW + c0);
+        float tmax = 0.f;
+        const bool inx = hasx && lane + 2 >= sp.a0 && lane + 2 < sp.a1;
+        unsigned long long *const ob = outbox + (par ^ 1) * XHALF;
 #pragma unroll
         for (int j = 0; j < RZ; j++) {
             const int lz = w * rpw + j;
             if (j >= rpw || lz >= rows) continue;
-            float v[12];
-            unpack3(ld4(cur + (rb + j) * SW + c0 - 4), zw[j + 4], ld4(cur + (rb + j) * SW + c0 + 4), v);
+            const float4 C = zw[j + 4];
+            const Pairs4 d = d2_pairs(ld4(cur + (rb + j) * SW + c0 - 4), C, ld4(cur + (rb + j) * SW + c0 + 4), zw + j);
+            float2 ra = add2(d.za, d.xa), rbb = add2(d.zb, d.xb);
             const float4 pp4 = ld4(nxt + (rb + j) * SW + c0);  // p^{n-1}
-            float4 ax4 = make_float4(0, 0, 0, 0), inj4 = make_float4(0, 0, 0, 0);
-            if (cpx) ax4 = ld4(AX + lz * TX + 4 * lane);
-            if (has_inj) inj4 = ld4(INJ + lz * TX + 4 * lane);
-            // zeta_z^n = b zeta_z^{n-1} + a (D2z p^n + D1z psi_z^n) on the widened z-strips
-            const bool zrow = lz >= zz0 && lz < zz1;
-            float4 dz4 = make_float4(0, 0, 0, 0), zz4 = make_float4(0, 0, 0, 0);
-            float az = 0.f, bzc = 0.f;
-            if (zrow) {
-                const float *pzc = PZ + (lz + 4) * TX + 4 * lane;
-                float4 a = ld4(pzc + TX), b = ld4(pzc - TX);
-                float d[4];
-#pragma unroll
-                for (int k = 0; k < 4; k++) d[k] = float(kD1) * (lane_of(a, k) - lane_of(b, k));
-                a = ld4(pzc + 2 * TX), b = ld4(pzc - 2 * TX);
-#pragma unroll
-                for (int k = 0; k < 4; k++) d[k] += float(kD2) * (lane_of(a, k) - lane_of(b, k));
-                a = ld4(pzc + 3 * TX), b = ld4(pzc - 3 * TX);
-#pragma unroll
-                for (int k = 0; k < 4; k++) d[k] += float(kD3) * (lane_of(a, k) - lane_of(b, k));
-                a = ld4(pzc + 4 * TX), b = ld4(pzc - 4 * TX);
-#pragma unroll
-                for (int k = 0; k < 4; k++) d[k] += float(kD4) * (lane_of(a, k) - lane_of(b, k));
-                dz4 = make_float4(d[0], d[1], d[2], d[3]);
-                zz4 = ld4(ZZ + lz * TX + 4 * lane);
-                az = CAZ[lz + 4];
-                bzc = CBZ[lz + 4];
-            }
-            float4 ka4 = make_float4(0, 0, 0, 0), kb4 = ka4, kc4 = ka4;
-            if (spg) {
-                ka4 = ld4(KA + lz * TX + 4 * lane);
-                kb4 = ld4(KB + lz * TX + 4 * lane);
-                kc4 = ld4(KC + lz * TX + 4 * lane);
-            }
-            float res[4], zo[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const float p = v[4 + k];
-                const float d2x = d2w(v, k);
-                const float d2z = d2c<float>(p, lane_of(zw[j + 3], k), lane_of(zw[j + 5], k), lane_of(zw[j + 2], k), lane_of(zw[j + 6], k),
-                                         lane_of(zw[j + 1], k), lane_of(zw[j + 7], k), lane_of(zw[j], k), lane_of(zw[j + 8], k));
-                float rhs = d2z + d2x;
-                if (cpx) rhs += lane_of(ax4, k);
-                zo[k] = 0.f;
-                if (zrow) {
-                    zo[k] = bzc * lane_of(zz4, k) + az * (d2z + lane_of(dz4, k));
-                    rhs += lane_of(dz4, k) + zo[k];
+            const float4 c4 = ld4(CC + lz * TX + 4 * lane);
+            // CPML terms: x from the phase above; z in place on the widened z-strips
+            const bool zrow = hasz && lz >= sp.za0 && lz < sp.za1;
+            if (inx || zrow) {
+                float2 ea = make_float2(0.f, 0.f), eb = ea;
+                if (inx) {
+                    const float4 ax4 = ld4(AX + lz * Y.wa + 4 * (lane + 2 - sp.a0));
+                    ea = lo2(ax4), eb = hi2(ax4);
                 }
-                if (has_inj) rhs += A.src_scale * (lane_of(inj4, k) * wn);
-                const float pp = lane_of(pp4, k);
-                res[k] = spg ? lane_of(ka4, k) * p - lane_of(kb4, k) * pp + lane_of(kc4, k) * rhs
-                             : 2.f * p - pp + lane_of(ch4[j], k) * rhs;
+                if (zrow) {
+                    const float *z1 = Z1 + (lz - sp.zp0) * TX + 4 * lane;
+                    if (!ADJ) {  // zeta_z^n = b zeta_z^{n-1} + a (D2z p^n + D1z psi_z^n)
+                        float2 da, db;
+                        d1z4<TX>(z1, da, db);
+                        float *zp = Z2 + (lz - sp.za0) * TX + 4 * lane;
+                        const float4 z4 = ld4(zp);
+                        const float2 a2 = splat2(CAZ[lz + 8]), b2 = splat2(CBZ[lz + 8]);
+                        const float2 za = rec2(a2, add2(d.za, da), b2, lo2(z4)), zb = rec2(a2, add2(d.zb, db), b2, hi2(z4));
+                        st4(zp, make_float4(za.x, za.y, zb.x, zb.y));
+                        ea = add2(ea, add2(da, za));
+                        eb = add2(eb, add2(db, zb));
+                    } else {  // D2 (a nu) - D1 (a mu)
+                        const float *z2 = Z2 + (lz - sp.zq0) * TX + 4 * lane;
+                        float4 an[9], m[9];
+#pragma unroll
+                        for (int k = 0; k < 9; k++) {
+                            const float a = CAZ[lz + 4 + k];
+                            const float4 v = ld4(z1 + (k - 4) * TX), u = ld4(z2 + (k - 4) * TX);
+                            an[k] = make_float4(a * v.x, a * v.y, a * v.z, a * v.w);
+                            m[k] = make_float4(a * u.x, a * u.y, a * u.z, a * u.w);
+                        }
+                        const float2 d2a = d2c2(lo2(an[4]), lo2(an[3]), lo2(an[5]), lo2(an[2]), lo2(an[6]), lo2(an[1]),
+                                                lo2(an[7]), lo2(an[0]), lo2(an[8]));
+                        const float2 d2b = d2c2(hi2(an[4]), hi2(an[3]), hi2(an[5]), hi2(an[2]), hi2(an[6]), hi2(an[1]),
+                                                hi2(an[7]), hi2(an[0]), hi2(an[8]));
+                        float2 da, db;
+                        d1_pairs(m[0], m[1], m[2], m[3], m[5], m[6], m[7], m[8], da, db);
+                        ea = add2(ea, add2(d2a, neg2(da)));
+                        eb = add2(eb, add2(d2b, neg2(db)));
+                    }
+                }
+                ra = add2(ra, ea);
+                rbb = add2(rbb, eb);
             }
-            if (zrow) st4(ZZ + lz * TX + 4 * lane, make_float4(zo[0], zo[1], zo[2], zo[3]));
+            if (has_inj && inj_flag(lz)) {
+                const float4 v = ld4(INJ + ((ADJ ? (n & 1) * Y.injr : 0) + inj_row(lz)) * TX + 4 * lane);
+                const float f = ADJ ? 1.f : wn;
+                ra.x = __fmaf_rn(A.src_scale, v.x * f, ra.x);
+                ra.y = __fmaf_rn(A.src_scale, v.y * f, ra.y);
+                rbb.x = __fmaf_rn(A.src_scale, v.z * f, rbb.x);
+                rbb.y = __fmaf_rn(A.src_scale, v.w * f, rbb.y);
+            }
+            float res[4], qk[4];
+            const float rhs[4] = {ra.x, ra.y, rbb.x, rbb.y};
+            if (!spg) {
+                const float4 o = plain4(C, pp4, c4, ra, rbb);
+                res[0] = o.x, res[1] = o.y, res[2] = o.z, res[3] = o.w;
+#pragma unroll
+                for (int k = 0; k < 4; k++) qk[k] = 0.f * (res[k] - lane_of(pp4, k)) - rhs[k];
+            } else if (R.exact_sponge) {
+                const float ez = CAZ[lz + 8];
+const float4 y4 = ld4(KA + lz * TX + 4 * lane);
+                const float2 one = splat2(1.f), two = splat2(2.f), ea = add2(splat2(ez), lo2(E4)), eb = add2(splat2(ez), hi2(E4));
+                const float2 ta = fma2(lo2(c4), ra, fma2(neg2(fma2(neg2(lo2(c4)), ea, one)), lo2(pp4), mul2(two, lo2(C))));
+                const float2 tb = fma2(hi2(c4), rbb, fma2(neg2(fma2(neg2(hi2(c4)), eb, one)), hi2(pp4), mul2(two, hi2(C))));
+                const float2 oa = quot2(ta, fma2(lo2(c4), ea, one), lo2(y4)), ob2 = quot2(tb, fma2(hi2(c4), eb, one), hi2(y4));
+                res[0] = oa.x, res[1] = oa.y, res[2] = ob2.x, res[3] = ob2.y;
+                qk[0] = __fmaf_rn(ea.x, oa.x - pp4.x, -ra.x), qk[1] = __fmaf_rn(ea.y, oa.y - pp4.y, -ra.y);
+                qk[2] = __fmaf_rn(eb.x, ob2.x - pp4.z, -rbb.x), qk[3] = __fmaf_rn(eb.y, ob2.y - pp4.w, -rbb.y);
+            } else {
+                const float4 ka = ld4(KA + lz * TX + 4 * lane), kb = ld4(KB + lz * TX + 4 * lane),
+                             kc = ld4(KC + lz * TX + 4 * lane);
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    res[k] = lane_of(ka, k) * lane_of(C, k) - lane_of(kb, k) * lane_of(pp4, k) + lane_of(kc, k) * rhs[k];
+                    qk[k] = 0.f;
+                }
+            }
             if (xedge) {
 #pragma unroll
                 for (int k = 0; k < 4; k++)
@@ -519,13 +738,46 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
             }
             if (top && lz == 0) res[0] = res[1] = res[2] = res[3] = 0.f;
             const float4 r4 = make_float4(res[0], res[1], res[2], res[3]);
+            if (top && lz >= 1 && lz <= H) st4(nxt + (HM - lz) * SW + c0, neg4(r4));  // odd mirror above the free surface
             st4(nxt + (rb + j) * SW + c0, r4);
-            unsigned long long *const ob = outbox + ((n + 1) & 1) * XHALF;
-            if (hasN && lz < H) put4(ob + XN + lz * TX + 4 * lane, r4, n + 1);
-            if (hasS && lz >= rows - H) put4(ob + XS + (lz - rows + H) * TX + 4 * lane, r4, n + 1);
-            if (hasW && 4 * lane < H) put4(ob + XWST + lz * HM + 4 * lane, r4, n + 1);
-            if (hasE && 4 * lane >= TX - H) put4(ob + XEST + lz * HM + 4 * lane - (TX - H), r4, n + 1);
+            if (n + 1 < R.n1) {
+                if (hasN && lz < H) put4(ob + XN + lz * TX + 4 * lane, r4, tag + 1);
+                if (hasS && lz >= rows - H) put4(ob + XS + (lz - rows + H) * TX + 4 * lane, r4, tag + 1);
+                if (hasW && 4 * lane < H) put4(ob + XWST + lz * HM + 4 * lane, r4, tag + 1);
+                if (hasE && 4 * lane >= TX - H) put4(ob + XEST + lz * HM + 4 * lane - (TX - H), r4, tag + 1);
+            }
+            if (MODE == kResRecord) {
+                qv[j] = make_float4(qk[0], qk[1], qk[2], qk[3]);
+                if (A.q_fp16)
+                    tmax = fmaxf(tmax, fmaxf(fmaxf(fabsf(qk[0]), fabsf(qk[1])), fmaxf(fabsf(qk[2]), fabsf(qk[3]))));
+                else
+                    st4(reinterpret_cast<float *>(qs) + sh + org + lo + j * P, qv[j]);
+            }
+            if (ADJ) {
+                float *gp = GG + lz * TX + 4 * lane;
+                float4 gv = ld4(gp);
+                gv.x += res[0] * qv[j].x;
+                gv.y += res[1] * qv[j].y;
+                gv.z += res[2] * qv[j].z;
+                gv.w += res[3] * qv[j].w;
+                st4(gp, gv);
+            }
         }
+        if (MODE == kResRecord && A.q_fp16) {  // one power-of-two scale per warp and step
+            const float s = pow2_scale(warp_max(tmax)), inv = 1.f / s;
+            if (lane == 0) *qsc = s;
+#pragma unroll
+            for (int j = 0; j < RZ; j++) {
+                if (j >= rpw || w * rpw + j >= rows) continue;
+                const __half2 a = __floats2half2_rn(qv[j].x * inv, qv[j].y * inv),
+                              b = __floats2half2_rn(qv[j].z * inv, qv[j].w * inv);
+                uint2 u;
+                u.x = *reinterpret_cast<const unsigned *>(&a);
+                u.y = *reinterpret_cast<const unsigned *>(&b);
+                *reinterpret_cast<uint2 *>(reinterpret_cast<__half *>(qs) + sh + org + lo + j * P) = u;
+            }
+        }
+        if (ADJ && has_inj && n + 1 < R.n1) residuals(n + 1);
 
         // Off the critical path, while the words travel: receivers and the
         // snapshot sample p^n, still held in this buffer until the next step's
@@ -569,58 +821,124 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const StepArgs<float> A, 
         }
     }
 
-    // final state: p^nt and p^{nt-1} into the global buffers of the per-step
-    // layout (the buffer written last holds p^nt); own cells only, each
-    // thread copying the cells it wrote
-    if (A.nt > 0) {
-        const float *fin = (A.nt & 1) ? S1 : S0, *prv = (A.nt & 1) ? S0 : S1;
-        float *gl = (A.nt & 1) ? gb1 : gb0, *gp = (A.nt & 1) ? gb0 : gb1;
+    // final state: p^{n1} and p^{n1-1} into the global buffers of the per-step
+    // layout, own cells only, each thread copying the cells it wrote; the
+    // memory fields' own cells on the strips, and the gradient sums
+    if (R.n1 > R.n0) {
+        const bool odd = (R.n1 - R.n0) & 1;
+        const float *fin = odd ? S1 : S0, *prv = odd ? S0 : S1;
+        float *gl = (R.n1 & 1) ? gb1 : gb0, *gp = (R.n1 & 1) ? gb0 : gb1;
 #pragma unroll
         for (int j = 0; j < RZ; j++) {
-            if (j >= rpw || w * rpw + j >= rows) continue;
+            const int lz = w * rpw + j;
+            if (j >= rpw || lz >= rows) continue;
             st4(gl + lo + j * P, ld4(fin + (rb + j) * SW + c0));
             st4(gp + lo + j * P, ld4(prv + (rb + j) * SW + c0));
+            if (ADJ) st4(A.G + sh + org + lo + j * P, ld4(GG + lz * TX + 4 * lane));
+        }
+        if (R.store_mem && (hasx || hasz)) {
+            __syncthreads();
+            if (hasx) {
+                float *m1 = R.m1o[0] + sh + org, *m2 = R.m2[0] + sh + org;
+                const int k0 = max(sp.c0, 2), nk = min(sp.c1, 2 + TX / 4) - k0;
+                for (int i = tid; i < rows * max(nk, 0); i += NTR) {
+                    const int lz = i / nk, c = k0 + i - lz * nk;
+                    st4(m1 + (long long)lz * P + 4 * c - 8, ld4(F1 + lz * Y.w1 + 4 * (c - sp.p0)));
+                }
+                const int b0 = ADJ ? max(sp.m0, 2) : sp.a0, nb = (ADJ ? min(sp.m1, 2 + TX / 4) : sp.a1) - b0,
+                          off = ADJ ? sp.q0 : sp.a0;
+                for (int i = tid; i < rows * max(nb, 0); i += NTR) {
+                    const int lz = i / nb, c = b0 + i - lz * nb;
+                    st4(m2 + (long long)lz * P + 4 * c - 8, ld4(F2 + lz * Y.w2 + 4 * (c - off)));
+                }
+            }
+            if (hasz) {
+                float *m1 = R.m1o[1] + sh + org, *m2 = R.m2[1] + sh + org;
+                for (int r = max(sp.zc0, 0) + w; r < min(sp.zc1, rows); r += NWR)
+                    st4(m1 + (long long)r * P + 4 * lane, ld4(Z1 + (r - sp.zp0) * TX + 4 * lane));
+                const int b0 = ADJ ? max(sp.zm0, 0) : sp.za0, b1 = ADJ ? min(sp.zm1, rows) : sp.za1,
+                          off = ADJ ? sp.zq0 : sp.za0;
+                for (int r = b0 + w; r < b1; r += NWR)
+                    st4(m2 + (long long)r * P + 4 * lane, ld4(Z2 + (r - off) * TX + 4 * lane));
+            }
         }
     }
 }
 
-template <int RZ>
+template <int RZ, int MODE>
 cudaError_t launch_rz(const StepArgs<float> &a, const ResidentArgs &r, int nshots, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(r.ntiles * nshots);
     cfg.blockDim = dim3(NTR);
-    cfg.dynamicSmemBytes = rsmem_floats<RZ>(a.bc) * sizeof(float);
+    cfg.dynamicSmemBytes = (size_t)r.lay.total * sizeof(float);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_resident2d<RZ>, a, r);
+    return cudaLaunchKernelEx(&cfg, k_resident2d<RZ, MODE>, a, r);
 }
 
 template <int RZ>
-int blocks_per_sm(int bc) {
-    const size_t bytes = rsmem_floats<RZ>(bc) * sizeof(float);
-    if (bytes > kResidentMaxSmem) return 0;
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_resident2d<RZ>, NTR, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return nb;
+cudaError_t launch_mode(const StepArgs<float> &a, const ResidentArgs &r, int mode, int nshots, cudaStream_t st) {
+    if (mode == kResRecord) return launch_rz<RZ, kResRecord>(a, r, nshots, st);
+    if (mode == kResAdjoint) return launch_rz<RZ, kResAdjoint>(a, r, nshots, st);
+    return launch_rz<RZ, kResForward>(a, r, nshots, st);
 }
 
 template <int RZ>
 cudaError_t configure_rz() {
-    size_t most = rsmem_floats<RZ>(SIM_BC_NONE);
-    for (int bc : {SIM_BC_SPONGE, SIM_BC_CPML})
-        if (rsmem_floats<RZ>(bc) * sizeof(float) <= kResidentMaxSmem) most = std::max(most, rsmem_floats<RZ>(bc));
-    return cudaFuncSetAttribute(k_resident2d<RZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(most * sizeof(float)));
+    cudaError_t e = cudaSuccess;
+    for (auto k : {k_resident2d<RZ, kResForward>, k_resident2d<RZ, kResRecord>, k_resident2d<RZ, kResAdjoint>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentMaxSmem - 64);
+    return e;
 }
 
 }  // namespace
+
+// Shared-memory layout of a launch over the given subdomains; false when it
+// does not fit. injr: rows with injected cells a subdomain has at most.
+bool resident2d_layout(const Geom &g, int bc, int rz, int mode, bool exact_sponge, const std::vector<RTile> &tiles, int injr,
+                       RLayout &Y) {
+    const int WZ = kResidentWarps * rz;
+    const bool adj = mode == kResAdjoint, cpml = bc == SIM_BC_CPML;
+    int w1 = 0, w2 = 0, wa = 0, z1 = 0, z2 = 0;
+    if (cpml)
+        for (const RTile &t : tiles) {
+            const RSpan s = resident_span(g, bc, t.bx, t.z0, t.rows, adj);
+            w1 = std::max(w1, 4 * (s.p1 - s.p0));
+            wa = std::max(wa, 4 * (s.a1 - s.a0));
+            w2 = std::max(w2, adj ? 4 * (s.q1 - s.q0) : 4 * (s.a1 - s.a0));
+            z1 = std::max(z1, s.zp1 - s.zp0);
+            z2 = std::max(z2, adj ? s.zq1 - s.zq0 : s.za1 - s.za0);
+        }
+    Y = RLayout{};
+    Y.w1 = w1;
+    Y.w2 = w2;
+    Y.wa = wa;
+    Y.injr = injr;
+    long long o = 2LL * (WZ + 2 * HM) * SW;
+    auto take = [&](long long n) {
+        const long long at = o;
+        o += (n + 3) / 4 * 4;
+        return (int)at;
+    };
+    Y.c = take((long long)WZ * TX);
+    Y.coef = take(bc != SIM_BC_NONE ? 2 * (TX + 16) + 2 * (WZ + 16) : 0);
+    Y.f1 = take((long long)WZ * w1);
+    Y.f2 = take((long long)WZ * w2);
+    Y.ax = take((long long)WZ * wa);
+    Y.z1 = take((long long)z1 * TX);
+    Y.z2 = take((long long)z2 * TX);
+    Y.G = take(adj ? (long long)WZ * TX : 0);
+    Y.K = take(bc == SIM_BC_SPONGE ? (exact_sponge ? 1LL : 3LL) * WZ * TX : 0);
+    Y.inj = take((long long)(adj ? 2 : 1) * injr * TX);
+    Y.rec = take(mode == kResForward ? 6 * kRecCache : 0);
+    Y.total = (int)std::min<long long>(o, 1 << 28);
+    return o * (long long)sizeof(float) + 64 <= (long long)kResidentMaxSmem;
+}
 
 cudaError_t configure_resident2d() {
     cudaError_t e = configure_rz<1>();
@@ -630,23 +948,13 @@ cudaError_t configure_resident2d() {
     return e;
 }
 
-int resident2d_blocks_per_sm(int rz, int bc) {
-    switch (rz) {
-        case 1: return blocks_per_sm<1>(bc);
-        case 2: return blocks_per_sm<2>(bc);
-        case 3: return blocks_per_sm<3>(bc);
-        case 4: return blocks_per_sm<4>(bc);
-        default: return 0;
-    }
-}
-
-cudaError_t launch_resident2d(const StepArgs<float> &a, const ResidentArgs &r, int rz, int nshots,
+cudaError_t launch_resident2d(const StepArgs<float> &a, const ResidentArgs &r, int rz, int mode, int nshots,
                               cudaStream_t st) {
     switch (rz) {
-        case 1: return launch_rz<1>(a, r, nshots, st);
-        case 2: return launch_rz<2>(a, r, nshots, st);
-        case 3: return launch_rz<3>(a, r, nshots, st);
-        case 4: return launch_rz<4>(a, r, nshots, st);
+        case 1: return launch_mode<1>(a, r, mode, nshots, st);
+        case 2: return launch_mode<2>(a, r, mode, nshots, st);
+        case 3: return launch_mode<3>(a, r, mode, nshots, st);
+        case 4: return launch_mode<4>(a, r, mode, nshots, st);
         default: return cudaErrorInvalidValue;
     }
 }

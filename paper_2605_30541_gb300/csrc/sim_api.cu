@@ -208,11 +208,14 @@ struct TileMap {
     std::vector<int> z0;    // [tile]
 };
 
-// Resident-path decomposition for one shot count (see plan_resident).
+// Resident-path decomposition of one shot count (see plan_resident).
 struct ResidentPlan {
-    int rz = 0;  // 0: the run does not fit on chip
-    std::vector<RTile> tiles;
+    int rz = 0;                // 0: the run does not fit on chip
+    int group = 0;             // shots per launch
+    double cost = 0;           // estimated time per step of all shots
+    std::vector<RTile> tiles;  // of one shot
     TileMap map;
+    RLayout lay[3];            // by mode
 };
 
 // Checkpoint schedule of the gradient and the sizes it was planned for
@@ -276,6 +279,7 @@ struct sim_s {
     RTile *rtiles = nullptr;               // resident path: subdomain descriptors
     const TileMap *tmap = nullptr;         // set while lists are built for a non-uniform tiling
     std::list<std::pair<int, ResidentPlan>> rplans;  // per shot count
+    std::list<std::pair<long long, ResidentPlan>> gplans;  // per shot count
     MarchSeg *mseg = nullptr;              // row march: segments, warp ranges, slice arguments
     StepArgs<float> *mslice = nullptr;
     size_t cap_mseg = 0;
@@ -1054,6 +1058,10 @@ int strip_chunks(const Geom &g, int bx) {
     return ncx + nax;
 }
 
+constexpr double kTileFixed = 50.0;  // exchange and barriers
+constexpr int kSourceRows = 2;       // a shot's source injects into two rows at most
+constexpr int kMaxGroups = 16;
+
 bool cut_columns(const sim_s *s, int wz, double target, std::vector<RTile> &tiles) {
     const Geom &g = s->g;
     const bool cp = s->d.bc == SIM_BC_CPML;
@@ -1066,7 +1074,7 @@ bool cut_columns(const sim_s *s, int wz, double target, std::vector<RTile> &tile
             RTile t{};
             t.bx = bx;
             t.z0 = z;
-            double acc = 50.0;
+            double acc = kTileFixed;
             while (z < g.NZ && t.rows < wz) {
                 const bool zs = cp && ((g.nbz0 > 0 && z < g.nbz0 + 4) || (g.nbz1 > 0 && z >= g.NZ - g.nbz1 - 4));
                 const double c = 1.0 + cx + (zs ? 1.34 : 0.0);
@@ -1110,28 +1118,54 @@ bool link_tiles(std::vector<RTile> &tiles) {
     return true;
 }
 
-bool plan_resident_uncached(sim_t s, int nshots, ResidentPlan &plan) {
+// Cost of the slowest subdomain.
+double plan_cost(const sim_s *s, const std::vector<RTile> &tiles) {
+    const Geom &g = s->g;
+    const bool cp = s->d.bc == SIM_BC_CPML;
+    double worst = 0;
+    for (const RTile &t : tiles) {
+        double c = kTileFixed + t.rows * (1.0 + (cp ? 0.039 * strip_chunks(g, t.bx) : 0.0));
+        if (cp)
+            for (int z = t.z0; z < t.z0 + t.rows; z++)
+                if ((g.nbz0 > 0 && z < g.nbz0 + 4) || (g.nbz1 > 0 && z >= g.NZ - g.nbz1 - 4)) c += 1.34;
+        worst = std::max(worst, c);
+    }
+    return worst;
+}
+
+// Subdomains of `nshots` shots in one launch. rec_rows < 0: a forward solve;
+// else a gradient whose residuals enter at most that many rows of a column.
+bool plan_resident_uncached(sim_t s, int nshots, int rec_rows, bool q_fp16, ResidentPlan &plan) {
     int sms = 0, coop = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, s->dev);
     if (!coop || sms <= 0) return false;
-    const long long cap_tiles = max_tiles(s);  // descriptors
+    const bool grad = rec_rows >= 0;
+    long long cap = std::min((long long)std::min(sms, s->cap_outbox) / nshots, max_tiles(s));
+    // the scales of an FP16 slot lie in its top ghost rows
+    if (grad && q_fp16) cap = std::min<long long>(cap, (long long)kGhost * s->g.P / 2 / kResidentWarps);
     for (int rz = 1; rz <= 4; rz++) {
-        const int bps = resident2d_blocks_per_sm(rz, s->d.bc);
-        if (bps <= 0) continue;
-        const long long cap = std::min((long long)std::min(bps * sms, s->cap_outbox) / nshots, cap_tiles);
         const int wz = kResidentWarps * rz;
+        auto fits = [&](const std::vector<RTile> &t) {
+            if ((long long)t.size() > cap) return false;
+            if (!resident2d_layout(s->g, s->d.bc, rz, kResForward, grad, t, kSourceRows, plan.lay[kResForward])) return false;
+            if (!grad) return true;
+            return resident2d_layout(s->g, s->d.bc, rz, kResRecord, true, t, kSourceRows, plan.lay[kResRecord]) &&
+                   resident2d_layout(s->g, s->d.bc, rz, kResAdjoint, true, t, std::min(rec_rows, wz), plan.lay[kResAdjoint]);
+        };
         std::vector<RTile> t;
         // the largest target gives uniform wz-row subdomains (the fewest)
         if (!cut_columns(s, wz, 1e30, t) || (long long)t.size() > cap) continue;
-        double lo = 50, hi = 50 + 4.0 * wz;
+        double lo = kTileFixed, hi = kTileFixed + 4.0 * wz;
         for (int it = 0; it < 40; it++) {
             const double mid = 0.5 * (lo + hi);
             if (cut_columns(s, wz, mid, t) && (long long)t.size() <= cap) hi = mid;
             else lo = mid;
         }
-        if (!cut_columns(s, wz, hi, t) || (long long)t.size() > cap || !link_tiles(t)) continue;
+        if (!cut_columns(s, wz, hi, t) || !fits(t) || !link_tiles(t)) continue;
         plan.rz = rz;
+        plan.group = nshots;
+        plan.cost = plan_cost(s, t);
         plan.tiles = t;
         TileMap &m = plan.map;
         m.NZ = s->g.NZ;
@@ -1147,17 +1181,76 @@ bool plan_resident_uncached(sim_t s, int nshots, ResidentPlan &plan) {
     return false;
 }
 
+bool resident_enabled(const sim_s *s) {
+    if (s->g.ndim != 2 || s->d.precision != SIM_FP32 || !s->outbox) return false;
+    const char *f = getenv("GSIM_RESIDENT");
+    return !(f && f[0] == '0');
+}
+
 // The plan depends only on the grid and the shot count: kept per handle.
 const ResidentPlan *plan_resident(sim_t s, int nshots) {
-    if (s->g.ndim != 2 || s->d.precision != SIM_FP32 || s->d.snap_fp16 || !s->outbox) return nullptr;
-    const char *f = getenv("GSIM_RESIDENT");
-    if (f && f[0] == '0') return nullptr;
+    if (!resident_enabled(s) || s->d.snap_fp16) return nullptr;
     for (const auto &p : s->rplans)
         if (p.first == nshots) return p.second.rz ? &p.second : nullptr;
     s->rplans.emplace_back(nshots, ResidentPlan{});
     ResidentPlan &p = s->rplans.back().second;
-    if (!plan_resident_uncached(s, nshots, p)) p = ResidentPlan{};
+    if (!plan_resident_uncached(s, nshots, -1, false, p)) p = ResidentPlan{};
     return p.rz ? &p : nullptr;
+}
+
+// Per time step of a gradient (a forward, a recording and an adjoint step of
+// every shot): the resident path's time by the cost model (0.15 us a unit with
+// CPML, 0.17 with the sponge) and the per-step kernels', launches' latency or
+// a rate that only large grids reach. Measured, per-step kernels and resident:
+// one shot of 131 x 131 cells with CPML 21.5 and 12.4 us, 60 of them (in 4
+// launches) 103 and 68, 16 shots of 241 x 241 59.4 and 26.3, 192 of them (in
+// 12) 550 and 319; with the sponge one shot of 699 x 1080 24.1 and 16.3, 8 of
+// them (in 8) 121 and 133: those stay with the per-step kernels.
+bool resident_gradient_faster(const sim_s *s, int nshots, const ResidentPlan &p) {
+    const Geom &g = s->g;
+    const double mcells = 1e-6 * nshots * g.NZ * (double)roundup(g.NX, kTileXF);
+    return s->d.bc == SIM_BC_CPML ? 0.15 * p.cost <= std::max(21.0, 14.0 + 38.0 * mcells)
+                                  : 0.17 * p.cost <= std::max(21.0, 10.0 + 17.8 * mcells);
+}
+
+// The gradient's plan: shots in as few launches (groups) per run of steps as
+// are fastest by the cost model.
+const ResidentPlan *plan_resident_gradient(sim_t s, int nshots, int nrec, const double *rec_pos, bool q_fp16) {
+    if (!resident_enabled(s) || s->plan.L < 2) return nullptr;  // the adjoint's in-place fields: sim_internal.h
+    const Geom &g = s->g;
+    // rows of a column that receivers inject into, at most
+    std::vector<char> seen((size_t)((g.NX + kTileXF - 1) / kTileXF) * g.NZ, 0);
+    std::vector<int> count((g.NX + kTileXF - 1) / kTileXF, 0);
+    int rows = 1;
+    for (int q = 0; q < nrec; q++) {
+        int i0[3];
+        double t[3];
+        if (!locate(g, s->d.h, rec_pos + (size_t)q * g.ndim, i0, t)) return nullptr;  // refused by the caller
+        for (int dz = 0; dz < 2; dz++)
+            for (int dx = 0; dx < 2; dx++) {
+                const int z = i0[0] + dz, bx = (i0[2] + dx) / kTileXF;
+                if (corner_weight(t, dz, 0, dx) == 0.0 || seen[(size_t)bx * g.NZ + z]) continue;
+                seen[(size_t)bx * g.NZ + z] = 1;
+                rows = std::max(rows, ++count[bx]);
+            }
+    }
+    rows = std::min(rows, 4 * kResidentWarps);
+    const long long key = ((long long)nshots << 8) | (rows << 1) | (q_fp16 ? 1 : 0);
+    for (const auto &p : s->gplans)
+        if (p.first == key) return p.second.rz ? &p.second : nullptr;
+    s->gplans.emplace_back(key, ResidentPlan{});
+    ResidentPlan &best = s->gplans.back().second;
+    for (int k = 1; k <= std::min(nshots, kMaxGroups); k++) {
+        ResidentPlan p;
+        if (!plan_resident_uncached(s, (nshots + k - 1) / k, rows, q_fp16, p)) continue;
+        p.cost *= (nshots + p.group - 1) / p.group;
+        if (getenv("GSIM_TUNE_LOG"))
+            fprintf(stderr, "[gsim resident gradient] grid %dx%d shots %d in %d launches: %d subdomains of %d rows, cost %.0f\n",
+                    g.NZ, g.NX, nshots, (nshots + p.group - 1) / p.group, (int)p.tiles.size(), p.tiles[0].rows, p.cost);
+        if (!best.rz || p.cost < best.cost) best = p;
+    }
+    if (best.rz && !resident_gradient_faster(s, nshots, best)) best = ResidentPlan{};
+    return best.rz ? &best : nullptr;
 }
 
 // One cooperative launch for the whole time loop, after zeroing the border
@@ -1168,16 +1261,74 @@ template <>
 sim_status run_resident<double>(sim_t s, const StepArgs<double> &, const ResidentPlan &, int) {
     return s->fail(SIM_ERR_UNSUPPORTED, "the resident path is FP32 only");
 }
+// no word of an earlier run may carry a tag of this one
+cudaError_t clear_outbox(sim_t s, int ctas, cudaStream_t st) {
+    return cudaMemsetAsync(s->outbox, 0, (size_t)ctas * kResidentOutbox * sizeof(*s->outbox), st);
+}
+ResidentArgs resident_args(sim_t s, const ResidentPlan &plan, int mode) {
+    ResidentArgs r{};
+    r.outbox = s->outbox;
+    r.spin_limit = spin_limit();
+    r.tiles = s->rtiles;
+    r.ntiles = (int)plan.tiles.size();
+    r.lay = plan.lay[mode];
+    return r;
+}
 template <>
 sim_status run_resident<float>(sim_t s, const StepArgs<float> &a, const ResidentPlan &plan, int nshots) {
-    const int nt = (int)plan.tiles.size();
     if (sim_status r = upload(s, s->rtiles, plan.tiles, (size_t)max_tiles(s), "subdomains")) return r;
-    // no word of an earlier run may carry a step number of this one
-    if (sim_status r = s->cuda(cudaMemsetAsync(s->outbox, 0, (size_t)nt * nshots * kResidentOutbox * sizeof(*s->outbox),
-                                               s->st), "border words"))
-        return r;
-    ResidentArgs r{s->outbox, spin_limit(), s->rtiles, nt};
-    return s->cuda(launch_resident2d(a, r, plan.rz, nshots, s->st), "resident launch");
+    ResidentArgs r = resident_args(s, plan, kResForward);
+    if (sim_status e = s->cuda(clear_outbox(s, r.ntiles * nshots, s->st), "border words")) return e;
+    r.n1 = a.nt;
+    if (s->d.bc == SIM_BC_CPML)
+        for (int k = 0; k < 2; k++) r.m2[k] = a.zeta[k ? 0 : 2];
+    return s->cuda(launch_resident2d(a, r, plan.rz, kResForward, nshots, s->st), "resident launch");
+}
+
+// What a captured gradient depends on beyond the handle's buffers.
+long long resident_key(const ResidentPlan &plan) {
+    return (((long long)plan.group << 20) ^ (plan.lay[kResAdjoint].injr << 8) ^ 1) << 24 ^ spin_limit() * 0x9e3779b97f4aLL;
+}
+// Lists follow the resident subdomains while this lasts.
+struct MapScope {
+    sim_t s;
+    ~MapScope() { s->tmap = nullptr; }
+};
+
+// A run of steps of the gradient: forward from the state in the global fields
+// (recording into q when given), or adjoint sweep steps; a launch per group of
+// shots. tag: the next unused tag of this call.
+cudaError_t gradient_run(sim_t s, const StepArgs<float> &a, const ResidentPlan &plan, int mode, int n0, int n1, int nshots,
+                         size_t qstride, unsigned &tag, cudaStream_t st) {
+    ResidentArgs r = resident_args(s, plan, mode);
+    r.n0 = n0;
+    r.n1 = n1;
+    r.load = 1;
+    r.store_mem = mode != kResRecord;  // a recorded segment is followed by a restored state
+    r.exact_sponge = 1;
+    r.q = static_cast<char *>(s->qbuf);
+    r.qstride = (long long)qstride;
+    if (s->d.bc == SIM_BC_CPML)
+        for (int k = 0; k < 2; k++) {
+            const int ax = k ? 0 : 2;
+            if (mode == kResAdjoint) {
+                r.m1i[k] = static_cast<float *>(s->cnu[ax][n0 & 1]);
+                r.m1o[k] = static_cast<float *>(s->cnu[ax][n1 & 1]);
+                r.m2[k] = static_cast<float *>(s->cmu[ax]);
+            } else {
+                r.m1i[k] = a.psi[ax][(n0 + 1) & 1];
+                r.m1o[k] = a.psi[ax][(n1 + 1) & 1];
+                r.m2[k] = a.zeta[ax];
+            }
+        }
+    cudaError_t e = cudaSuccess;
+    for (int s0 = 0; s0 < nshots && e == cudaSuccess; s0 += plan.group) {
+        r.shot0 = s0;
+        r.tag0 = tag;
+        tag += (unsigned)(n1 - n0);
+        e = launch_resident2d(a, r, plan.rz, mode, std::min(plan.group, nshots - s0), st);
+    }
+    return e;
 }
 
 // ---------------------------------------------------------------- row march plan
@@ -1329,10 +1480,7 @@ sim_status forward_t(sim_t s, int nshots, const void *wavelet, const double *src
     } else {
     // geometry lists, per tile of the kernel that runs (the resident
     // subdomains while this scope lasts)
-    struct MapScope {
-        sim_t s;
-        ~MapScope() { s->tmap = nullptr; }
-    } map_scope{s};
+    MapScope map_scope{s};
     s->tmap = rz ? &plan->map : nullptr;
     std::vector<int> rstart, istart;
     std::vector<RecEntryT<T>> rent;
@@ -1722,20 +1870,20 @@ cudaError_t checkpoint(sim_t s, const StepArgs<T> &a, const CkLayout &c, int k, 
     return e;
 }
 
-// The reverse schedule of a plan as a sequence of launches:
-//   fwd_first(n): forward step n of the first sweep (samples the gather);
-//   fwd(n): forward step n of a recompute that keeps checkpoints only;
-//   rec(n, slot): forward step n recording its imaging term into slot;
-//   adj(k, slot): adjoint step k (the slot recorded by forward step k - 1);
+// The reverse schedule of a plan as a sequence of runs of steps:
+//   fwd_first(n0, n1): forward steps of the first sweep (sampling the gather);
+//   fwd(n0, n1): forward steps of a recompute that keeps checkpoints only;
+//   rec(n0, n1): forward steps recording their imaging terms, step n into slot n - n0;
+//   adj(n0, n1): adjoint steps k = n1 .. n0 + 1 (the slot recorded by forward step k - 1);
 //   ck(slot, n, store): store / restore the state entering step n;
 //   mid(): between the forward sweep and the reverse (residual, zeroing).
 template <typename F1, typename F2, typename F3, typename F4, typename F5, typename F6>
 cudaError_t emit_gradient(const AdjPlan &P, int nt, F1 fwd_first, F2 fwd, F3 rec, F4 adj, F5 ck, F6 mid) {
     const int S1 = P.L * P.m;
     cudaError_t e = cudaSuccess;
-    for (int n = 0; n < nt && e == cudaSuccess; n++) {
-        if (n % S1 == 0) e = ck(n / S1, n, true);
-        if (e == cudaSuccess) e = fwd_first(n);
+    for (int n = 0; n < nt && e == cudaSuccess; n += S1) {
+        e = ck(n / S1, n, true);
+        if (e == cudaSuccess) e = fwd_first(n, std::min(nt, n + S1));
     }
     if (e == cudaSuccess) e = mid();
     for (int t = (nt + S1 - 1) / S1 - 1; t >= 0 && e == cudaSuccess; t--) {
@@ -1744,18 +1892,35 @@ cudaError_t emit_gradient(const AdjPlan &P, int nt, F1 fwd_first, F2 fwd, F3 rec
         e = ck(t, t0, false);
         // recompute up to the last inner segment, keeping the inner starts
         // 1 .. msub - 2 (the first restarts from slot t, the last from here)
-        for (int n = t0; n < t0 + (msub - 1) * P.L && e == cudaSuccess; n++) {
-            if (n > t0 && (n - t0) % P.L == 0 && (n - t0) / P.L <= msub - 2) e = ck(P.n1 + (n - t0) / P.L - 1, n, true);
-            if (e == cudaSuccess) e = fwd(n);
+        for (int j = 0; j < msub - 1 && e == cudaSuccess; j++) {
+            if (j > 0) e = ck(P.n1 + j - 1, t0 + j * P.L, true);
+            if (e == cudaSuccess) e = fwd(t0 + j * P.L, t0 + (j + 1) * P.L);
         }
         for (int j = msub - 1; j >= 0 && e == cudaSuccess; j--) {
             const int s0 = t0 + j * P.L, s1 = std::min(t1, s0 + P.L);
             if (j < msub - 1) e = ck(j == 0 ? t : P.n1 + j - 1, s0, false);
-            for (int n = s0; n < s1 && e == cudaSuccess; n++) e = rec(n, n - s0);
-            for (int k = s1; k >= s0 + 1 && e == cudaSuccess; k--) e = adj(k, k - 1 - s0);
+            if (e == cudaSuccess) e = rec(s0, s1);
+            if (e == cudaSuccess) e = adj(s0, s1);
         }
     }
     return e;
+}
+// Runs as one launch (or a few) per step.
+template <typename F>
+auto each_step(F step) {
+    return [step](int n0, int n1) {
+        cudaError_t e = cudaSuccess;
+        for (int n = n0; n < n1 && e == cudaSuccess; n++) e = step(n, n - n0);
+        return e;
+    };
+}
+template <typename F>
+auto each_step_back(F step) {
+    return [step](int n0, int n1) {
+        cudaError_t e = cudaSuccess;
+        for (int k = n1; k > n0 && e == cudaSuccess; k--) e = step(k, k - 1 - n0);
+        return e;
+    };
 }
 
 // Injection groups of 3D points (the adjoint sweep's residuals): every corner
@@ -1943,10 +2108,10 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
             };
             auto slot_of = [&](int i) { return reinterpret_cast<float *>(static_cast<char *>(s->qbuf) + (size_t)i * qstride); };
             e = emit_gradient(
-                P, d.nt, [&](int n) { return step(a, n, kModeForward, nullptr, true); },
-                [&](int n) { return step(quiet, n, kModeForward, nullptr, false); },
-                [&](int n, int i) { return step(quiet, n, kModeRecord, slot_of(i), false); },
-                [&](int k, int i) {
+                P, d.nt, each_step([&](int n, int) { return step(a, n, kModeForward, nullptr, true); }),
+                each_step([&](int n, int) { return step(quiet, n, kModeForward, nullptr, false); }),
+                each_step([&](int n, int i) { return step(quiet, n, kModeRecord, slot_of(i), false); }),
+                each_step_back([&](int k, int i) {
                     float *slot = slot_of(i);
                     const int n = d.nt - k;
                     // nu^k, mu^k from u^{k+1} and their bracket, which the march adds as
@@ -1971,7 +2136,7 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
                         e2 = launch_inj3d(adj, n, k, s->res3g, nrg, s->res3e, nshots, slot, Gs, st);
                     if (e2 == cudaSuccess && terms && !fused) e2 = launch_cpml_adjoint<float>(a, ca, k & 1, nshots, st);
                     return e2;
-                },
+                }),
                 [&](int k, int n, bool store) { return checkpoint<float>(s, a, ckl, k, n, store, ckpt_fp16, nshots, st); },
                 [&]() { return gradient_mid<float>(s, nshots, nrows, o.vjp, st); });
             // FP64 sum over shots and replicated cells
@@ -2000,10 +2165,15 @@ sim_status adjoint_t(sim_t s, int nshots, const void *wavelet, const double *src
         return adjoint3d(s, nshots, wavelet, src_pos, nrec, rec_pos, d_obs, gather_out, misfit_out, ckpt_fp16,
                          grad_v, o);
     if (sim_status r = ensure_adjoint(s, ckpt_fp16)) return r;
-    if (sim_status r = autotune(s, nshots)) return r;
+    const ResidentPlan *plan =
+        std::is_same<T, float>::value ? plan_resident_gradient(s, nshots, nrec, rec_pos, ckpt_fp16 != 0) : nullptr;
+    if (!plan)
+        if (sim_status r = autotune(s, nshots)) return r;
+    MapScope map_scope{s};
+    s->tmap = plan ? &plan->map : nullptr;
     const size_t nt = d.nt;
     const int ms = d.max_shots;
-    const int ntiles = s->ntx * s->nty * s->ntz;
+    const int ntiles = tiles_of(s);
     const long long nint = (long long)g.nz * g.ny * g.nx;
     const size_t nrows = (size_t)nshots * nt * nrec;
 
@@ -2058,6 +2228,8 @@ sim_status adjoint_t(sim_t s, int nshots, const void *wavelet, const double *src
     io.resid = s->res;
     io.nrec = nrec;
     io.nshots = nshots;
+    if (plan)
+        if (sim_status r = upload(s, s->rtiles, plan->tiles, (size_t)max_tiles(s), "subdomains")) return r;
     if (sim_status r = s->cuda(cudaMemcpyAsync(s->io, &io, sizeof io, cudaMemcpyHostToDevice, s->st), "io upload"))
         return r;
 
@@ -2092,39 +2264,56 @@ sim_status adjoint_t(sim_t s, int nshots, const void *wavelet, const double *src
         adj.bc = SIM_BC_NONE;
         adj.cext = static_cast<const T *>(s->cext);
     }
-    const size_t qstride = q_slot_bytes(s, ckpt_fp16), q_tiles = (size_t)ms * ntiles;
+    const size_t qstride = q_slot_bytes(s, ckpt_fp16);
     // graph key: everything the captured launches depend on beyond handle buffers
     const long long gkey = ((long long)nshots << 40) ^ ((long long)nrec << 12) ^ ((long long)s->tile_z << 4) ^
-                           ((long long)ckpt_fp16 << 3) ^ ((long long)o.vjp << 9) ^ 5;
+                           ((long long)ckpt_fp16 << 3) ^ ((long long)o.vjp << 9) ^ (plan ? resident_key(*plan) : 0) ^ 5;
     if (sim_status r = run_graph(s, gkey, [&](cudaStream_t st) {
             cudaError_t e = reset_state_on(s, nshots, st);
             if (e != cudaSuccess) return e;
             auto slot_of = [&](int i) { return static_cast<void *>(static_cast<char *>(s->qbuf) + (size_t)i * qstride); };
             auto scale_of = [&](int i) { return s->qscale + (size_t)i * (q_scale_bytes(s) / sizeof(float)); };
-            (void)q_tiles;
-            e = emit_gradient(
-                P, d.nt, [&](int n) { return launch_step<T>(s, a, n, nshots, kModeForward, st); },
-                [&](int n) { return launch_step<T>(s, quiet, n, nshots, kModeForward, st); },
-                [&](int n, int i) { return launch_step<T>(s, rcp, n, nshots, kModeRecord, st, slot_of(i), scale_of(i)); },
-                [&](int k, int i) {
-                    cudaError_t e2 = cudaSuccess;
-                    if (cpml && k <= d.nt - 1) {  // nu^k, mu^k from u^{k+1}, then their term in u^k
-                        CpmlAdjArgs<T> ca{};
-                        ca.u = adj.pbuf[(d.nt - k) & 1];
-                        for (int ax = 0; ax < 3; ax++) {
-                            ca.nu[ax][0] = static_cast<T *>(s->cnu[ax][0]);
-                            ca.nu[ax][1] = static_cast<T *>(s->cnu[ax][1]);
-                            ca.mu[ax] = static_cast<T *>(s->cmu[ax]);
+            auto ck = [&](int k, int n, bool store) { return checkpoint<T>(s, a, ckl, k, n, store, ckpt_fp16, nshots, st); };
+            auto mid = [&]() { return gradient_mid<T>(s, nshots, nrows, o.vjp, st); };
+            if constexpr (std::is_same<T, float>::value)
+                if (plan) {
+                    unsigned tag = 0;
+                    auto run = [&](const StepArgs<float> &x, int mode, int n0, int n1) {
+                        return gradient_run(s, x, *plan, mode, n0, n1, nshots, qstride, tag, st);
+                    };
+                    e = clear_outbox(s, (int)plan->tiles.size() * plan->group, st);
+                    if (e == cudaSuccess)
+                        e = emit_gradient(
+                            P, d.nt, [&](int n0, int n1) { return run(a, kResForward, n0, n1); },
+                            [&](int n0, int n1) { return run(quiet, kResForward, n0, n1); },
+                            [&](int n0, int n1) { return run(rcp, kResRecord, n0, n1); },
+                            [&](int n0, int n1) { return run(adj, kResAdjoint, d.nt - n1, d.nt - n0); }, ck, mid);
+                }
+            if (!plan)
+                e = emit_gradient(
+                    P, d.nt, each_step([&](int n, int) { return launch_step<T>(s, a, n, nshots, kModeForward, st); }),
+                    each_step([&](int n, int) { return launch_step<T>(s, quiet, n, nshots, kModeForward, st); }),
+                    each_step([&](int n, int i) {
+                        return launch_step<T>(s, rcp, n, nshots, kModeRecord, st, slot_of(i), scale_of(i));
+                    }),
+                    each_step_back([&](int k, int i) {
+                        cudaError_t e2 = cudaSuccess;
+                        if (cpml && k <= d.nt - 1) {  // nu^k, mu^k from u^{k+1}, then their term in u^k
+                            CpmlAdjArgs<T> ca{};
+                            ca.u = adj.pbuf[(d.nt - k) & 1];
+                            for (int ax = 0; ax < 3; ax++) {
+                                ca.nu[ax][0] = static_cast<T *>(s->cnu[ax][0]);
+                                ca.nu[ax][1] = static_cast<T *>(s->cnu[ax][1]);
+                                ca.mu[ax] = static_cast<T *>(s->cmu[ax]);
+                            }
+                            ca.ext = static_cast<T *>(s->cext);
+                            e2 = launch_cpml_adjoint<T>(a, ca, k & 1, nshots, st);
                         }
-                        ca.ext = static_cast<T *>(s->cext);
-                        e2 = launch_cpml_adjoint<T>(a, ca, k & 1, nshots, st);
-                    }
-                    if (e2 == cudaSuccess)
-                        e2 = launch_step<T>(s, adj, d.nt - k, nshots, kModeAdjoint, st, slot_of(i), scale_of(i));
-                    return e2;
-                },
-                [&](int k, int n, bool store) { return checkpoint<T>(s, a, ckl, k, n, store, ckpt_fp16, nshots, st); },
-                [&]() { return gradient_mid<T>(s, nshots, nrows, o.vjp, st); });
+                        if (e2 == cudaSuccess)
+                            e2 = launch_step<T>(s, adj, d.nt - k, nshots, kModeAdjoint, st, slot_of(i), scale_of(i));
+                        return e2;
+                    }),
+                    ck, mid);
             // FP64 sum over shots and replicated cells
             if (e == cudaSuccess) e = cudaMemsetAsync(s->acc, 0, nint * sizeof(double), st);
             if (e == cudaSuccess)

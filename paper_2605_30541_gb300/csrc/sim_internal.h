@@ -321,30 +321,129 @@ cudaError_t launch_inj3d(const StepArgs<float> &a, int n, int row, const Inj3 *g
                          int nshots, const float *qs, float *Gs, cudaStream_t st);
 cudaError_t launch_snap3d(const StepArgs<float> &a, const StepTime &t, int fp16, int nshots, cudaStream_t st);
 
-// Resident execution (resident2d.cu): one cooperative launch runs the whole
-// forward time loop of a 2D FP32 problem whose state fits on chip; each CTA
-// of kResidentWarps warps owns one subdomain: columns [128 bx, 128 bx + 128),
-// rows [z0, z0 + rows) with rows <= 16 RZ, warps taking rpw rows each.
-// nbr lists the subdomains whose borders form its halo (same shot). outbox:
-// kResidentOutbox 8-byte words per (shot, subdomain), zeroed before the launch.
+// Resident execution (resident2d.cu): one cooperative launch runs steps [n0, n1)
+// of 2D FP32 shots whose state fits on chip; each CTA of kResidentWarps warps
+// owns one subdomain: columns [128 bx, 128 bx + 128), rows [z0, z0 + rows) with
+// rows <= 16 RZ, warps taking rpw rows each. nbr lists the subdomains whose
+// borders form its halo (same shot).
 constexpr int kResidentWarps = 16;
 constexpr size_t kResidentMaxSmem = 227 * 1024;
 constexpr int kResidentMaxNbr = 11;
-constexpr int kResidentOutbox = 2 * (2 * 8 * 128 + 2 * 64 * 8);  // two step parities of border rows and columns
+constexpr int kResidentOutbox = 2 * (2 * 8 * 128 + 2 * 64 * 8);  // words: two halves of border rows and columns
 struct RTile {
     int bx, z0, rows, rpw;
     int nnbr;
     int nbr[kResidentMaxNbr];
 };
+
+// CPML work of one subdomain. Columns in float4 chunks (chunk c: the cells
+// 4c - 8 .. 4c - 5 of the subdomain, c in [0, 36)), rows subdomain-local; the
+// memory fields are non-zero on the strips only, the terms that use them on
+// the strips widened by 4. Forward: first field psi, second zeta; adjoint: nu
+// and mu (kept on the ring of 8 and 4 cells round the subdomain that the
+// transposed derivatives reach, recomputed redundantly as psi is on 4).
+struct RSpan {
+    int c0, c1;   // chunks of the first field that are updated
+    int m0, m1;   // adjoint: chunks of the second
+    int a0, a1;   // own chunks that take the term
+    int p0, p1;   // chunks of the first field kept (zeros round [c0, c1) for the derivative windows)
+    int q0, q1;   // adjoint: of the second
+    int zc0, zc1, zm0, zm1, za0, za1, zp0, zp1, zq0, zq1;  // the same along z, in rows
+};
+__host__ __device__ inline void strip_hull(int o, int N, int nb0, int nb1, int c0, int c1, int &lo, int &hi) {
+    lo = 1 << 30;
+    hi = -(1 << 30);
+    if (nb0 > 0) {
+        const int a = -o > c0 ? -o : c0, b = nb0 - o < c1 ? nb0 - o : c1;
+        if (a < b) lo = a < lo ? a : lo, hi = b > hi ? b : hi;
+    }
+    if (nb1 > 0) {
+        const int a = N - nb1 - o > c0 ? N - nb1 - o : c0, b = N - o < c1 ? N - o : c1;
+        if (a < b) lo = a < lo ? a : lo, hi = b > hi ? b : hi;
+    }
+}
+__host__ __device__ inline RSpan resident_span(const Geom &g, int bc, int bx, int z0, int rows, bool adj) {
+    RSpan s{};
+    if (bc != SIM_BC_CPML) return s;
+    const int x0 = bx * kTileXF, ring = adj ? 8 : 4;
+    auto mn = [](int a, int b) { return a < b ? a : b; };
+    auto mx = [](int a, int b) { return a > b ? a : b; };
+    int lo, hi;
+    strip_hull(x0, g.NX, g.nbx0, g.nbx1, -ring, kTileXF + ring, lo, hi);
+    if (lo < hi) {
+        s.c0 = (lo + 8) >> 2, s.c1 = (hi + 11) >> 2;
+        s.p0 = s.c0, s.p1 = s.c1;
+        const int al = mx(0, lo - 4), ah = mn(kTileXF, hi + 4);
+        if (al < ah) s.a0 = (al + 8) >> 2, s.a1 = (ah + 11) >> 2;
+        if (adj) {
+            strip_hull(x0, g.NX, g.nbx0, g.nbx1, -4, kTileXF + 4, lo, hi);
+            if (lo < hi) {
+                s.m0 = (lo + 8) >> 2, s.m1 = (hi + 11) >> 2;
+                s.p0 = mn(s.p0, s.m0 - 1), s.p1 = mx(s.p1, s.m1 + 1);
+            }
+            s.q0 = s.m0, s.q1 = s.m1;
+            if (s.a0 < s.a1) {
+                if (s.q0 >= s.q1) s.q0 = s.a0, s.q1 = s.a1;
+                s.q0 = mn(s.q0, s.a0 - 1), s.q1 = mx(s.q1, s.a1 + 1);
+            }
+        }
+        if (s.a0 < s.a1) s.p0 = mn(s.p0, s.a0 - 1), s.p1 = mx(s.p1, s.a1 + 1);
+    }
+    strip_hull(z0, g.NZ, g.nbz0, g.nbz1, -ring, rows + ring, lo, hi);
+    if (lo < hi) {
+        s.zc0 = lo, s.zc1 = hi;
+        s.zp0 = lo, s.zp1 = hi;
+        s.za0 = mx(0, lo - 4), s.za1 = mn(rows, hi + 4);
+        if (s.za0 >= s.za1) s.za0 = s.za1 = 0;
+        if (adj) {
+            strip_hull(z0, g.NZ, g.nbz0, g.nbz1, -4, rows + 4, lo, hi);
+            if (lo < hi) {
+                s.zm0 = lo, s.zm1 = hi;
+                s.zp0 = mn(s.zp0, lo - 4), s.zp1 = mx(s.zp1, hi + 4);
+            }
+            s.zq0 = s.zm0, s.zq1 = s.zm1;
+            if (s.za0 < s.za1) {
+                if (s.zq0 >= s.zq1) s.zq0 = s.za0, s.zq1 = s.za1;
+                s.zq0 = mn(s.zq0, s.za0 - 4), s.zq1 = mx(s.zq1, s.za1 + 4);
+            }
+        }
+        if (s.za0 < s.za1) s.zp0 = mn(s.zp0, s.za0 - 4), s.zp1 = mx(s.zp1, s.za1 + 4);
+    }
+    return s;
+}
+
+// Shared memory of a launch (floats; the same for every CTA): offsets and the
+// widths of the compact CPML arrays (the largest over the subdomains).
+struct RLayout {
+    int c, coef, f1, f2, ax, z1, z2, G, K, inj, rec;  // offsets
+    int w1, w2, wa;                                   // floats per row of f1, f2, ax
+    int injr;                                         // rows with injected cells a subdomain may have
+    int total;
+};
+enum { kResForward = 0, kResRecord = 1, kResAdjoint = 2 };
 struct ResidentArgs {
-    unsigned long long *outbox;
+    unsigned long long *outbox;  // kResidentOutbox words per CTA
     long long spin_limit;
     const RTile *tiles;  // device array, per shot
     int ntiles;
+    int shot0;           // first shot of the launch
+    int n0, n1;          // steps (adjoint: sweep index n = nt - k)
+    unsigned tag0;       // words of step n carry tag0 + n - n0; no earlier launch has used tags from tag0 on
+    int load;            // start from the state in the global fields (else from rest)
+    int store_mem;       // leave the CPML memory in the global fields too
+    int exact_sponge;    // the sponge update with its division, as the per-step kernels have it
+    RLayout lay;
+    // CPML memory, field layout (x, z): forward psi in, psi out, zeta; adjoint nu, mu
+    float *m1i[2], *m1o[2], *m2[2];
+    // imaging-term slots of the launch's steps (record: slot n - n0; adjoint: slot n1 - 1 - n); FP16
+    // slots keep a scale per (subdomain, warp) in the top ghost rows of each shot's field
+    char *q;
+    long long qstride;
 };
 cudaError_t configure_resident2d();
-int resident2d_blocks_per_sm(int rz, int bc);  // 0: does not fit
-cudaError_t launch_resident2d(const StepArgs<float> &a, const ResidentArgs &r, int rz, int nshots,
+bool resident2d_layout(const Geom &g, int bc, int rz, int mode, bool exact_sponge, const std::vector<RTile> &tiles, int injr,
+                       RLayout &lay);
+cudaError_t launch_resident2d(const StepArgs<float> &a, const ResidentArgs &r, int rz, int mode, int nshots,
                               cudaStream_t st);
 
 // Message returned by sim_last_error(NULL) for failures of this thread.
