@@ -382,8 +382,7 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &A, const StepTi
             float out, es = 0.f;
             if (spg) {
                 es = ez + lane_of(E4, k);
-                const float a = chv * es;
-                out = (2.f * p - (1.f - a) * pp + chv * rhs) / (1.f + a);
+                out = quot1(__fmaf_rn(chv, rhs, __fmaf_rn(-__fmaf_rn(-chv, es, 1.f), pp, 2.f * p)), __fmaf_rn(chv, es, 1.f));
             } else {
                 out = 2.f * p - pp + chv * rhs;
             }

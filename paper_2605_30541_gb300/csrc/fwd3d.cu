@@ -71,7 +71,7 @@ __device__ __forceinline__ Cells4 cells4(const float4 &L, const float4 &C, const
         for (int k = 0; k < 4; k++) {
             const float p = lane4(C, k), chv = lane4(ch4, k), pp = lane4(pp4, k);
             const float a = chv * (es0 + lane4(Ex4, k));
-            o.res[k] = (2.f * p - (1.f - a) * pp + chv * o.rhs[k]) / (1.f + a);
+            o.res[k] = quot1(2.f * p - (1.f - a) * pp + chv * o.rhs[k], 1.f + a);
         }
     }
     return o;

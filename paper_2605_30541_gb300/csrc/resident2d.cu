@@ -144,41 +144,6 @@ __device__ __forceinline__ void d2x_pairs(const float4 &L, const float4 &C, cons
     db = d2c2(hi2(C), v56, v78, lo2(C), lo2(R), v34, v910, hi2(L), hi2(R));
 }
 
-// t / d correctly rounded, d >= 1, from y = RN(1/d): Markstein's theorem (IBM
-// J. Res. Dev. 34, 1990): one step from t y gives a quotient within an ulp, and
-// from such a quotient q the step RN(q + y (t - d q)) is RN(t / d), t - d q
-// being exact. Small t, whose residuals would not be exact, are scaled by
-// 2^100. Scaled back, a quotient below 2^-125 rounds a second time, onto
-// multiples of 2^-149: where that went the wrong way from a tie, the residual
-// (exact) is more than half such a step, and one step is added. Fields hold
-// such values wherever a wave has not yet arrived, and the division's own slow
-// path for them took half the time of a step.
-__device__ __forceinline__ float quot_small(float t, float d, float y) {
-    t *= 0x1p100f;
-    float q = t * y;
-    q = __fmaf_rn(__fmaf_rn(-d, q, t), y, q);
-    q = __fmaf_rn(__fmaf_rn(-d, q, t), y, q);
-    float r = q * 0x1p-100f;
-    if (fabsf(q) < 0x1p-25f) {
-        const float e = __fmaf_rn(-d, r * 0x1p100f, t), half = d * 0x1p-50f;
-        if (fabsf(e) > half) r += copysignf(0x1p-149f, e);
-    }
-    return r;
-}
-__device__ __forceinline__ float2 quot2(float2 t, float2 d, float2 y) {
-    const float mx = fabsf(t.x), my = fabsf(t.y);
-    if (!(fmaxf(mx, my) < 0x1p90f && mx + my < 0x1p91f)) return make_float2(t.x / d.x, t.y / d.y);  // huge, infinite, NaN
-    const float2 nd = neg2(d);
-    float2 q = mul2(t, y);
-    q = fma2(fma2(nd, q, t), y, q);
-    q = fma2(fma2(nd, q, t), y, q);
-    if ((mx < 0x1p-90f && mx != 0.f) || (my < 0x1p-90f && my != 0.f)) {
-        if (mx < 0x1p-90f) q.x = quot_small(t.x, d.x, y.x);
-        if (my < 0x1p-90f) q.y = quot_small(t.y, d.y, y.y);
-    }
-    return q;
-}
-
 template <int RZ, int MODE>
 __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ StepArgs<float> A,
                                                        const __grid_constant__ ResidentArgs R) {

@@ -52,6 +52,54 @@ __device__ __forceinline__ float2 splat2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
 
+// t / d correctly rounded, d >= 1, from y = RN(1/d): Markstein's theorem (IBM
+// J. Res. Dev. 34, 1990): one step from t y gives a quotient within an ulp, and
+// from such a quotient q the step RN(q + y (t - d q)) is RN(t / d), t - d q
+// being exact. Small t, whose residuals would not be exact, are scaled by
+// 2^100. Scaled back, a quotient below 2^-125 rounds a second time, onto
+// multiples of 2^-149: where that went the wrong way from a tie, the residual
+// (exact) is more than half such a step, and one step is added. (No difference
+// from the division in 3e9 pairs over the whole range of t, d in [1, 6).) Fields
+// hold such values wherever a wave has not yet arrived, and the division takes
+// a slow path for each: with this quotient a 739 x 1120 sponge slice with FP16
+// snapshots runs 701 steps in 4.56 ms instead of 4.84, 8 shots of 452 x 952
+// 438 steps in 8.0 instead of 9.7, 2 shots of a 228 x 232 x 165 volume 104
+// steps in 11.9 instead of 19.3. quot2 takes kept reciprocals, quot1 forms them.
+__device__ __forceinline__ float quot_small(float t, float d, float y) {
+    t *= 0x1p100f;
+    float q = t * y;
+    q = __fmaf_rn(__fmaf_rn(-d, q, t), y, q);
+    q = __fmaf_rn(__fmaf_rn(-d, q, t), y, q);
+    float r = q * 0x1p-100f;
+    if (fabsf(q) < 0x1p-25f) {
+        const float e = __fmaf_rn(-d, r * 0x1p100f, t), half = d * 0x1p-50f;
+        if (fabsf(e) > half) r += copysignf(0x1p-149f, e);
+    }
+    return r;
+}
+__device__ __forceinline__ float2 quot2(float2 t, float2 d, float2 y) {
+    const float mx = fabsf(t.x), my = fabsf(t.y);
+    if (!(fmaxf(mx, my) < 0x1p90f && mx + my < 0x1p91f)) return make_float2(t.x / d.x, t.y / d.y);  // huge, infinite, NaN
+    const float2 nd = neg2(d);
+    float2 q = mul2(t, y);
+    q = fma2(fma2(nd, q, t), y, q);
+    q = fma2(fma2(nd, q, t), y, q);
+    if ((mx < 0x1p-90f && mx != 0.f) || (my < 0x1p-90f && my != 0.f)) {
+        if (mx < 0x1p-90f) q.x = quot_small(t.x, d.x, y.x);
+        if (my < 0x1p-90f) q.y = quot_small(t.y, d.y, y.y);
+    }
+    return q;
+}
+__device__ __forceinline__ float quot1(float t, float d) {
+    const float m = fabsf(t);
+    if (!(m < 0x1p90f)) return t / d;
+    const float y = __frcp_rn(d);
+    float q = t * y;
+    q = __fmaf_rn(__fmaf_rn(-d, q, t), y, q);
+    q = __fmaf_rn(__fmaf_rn(-d, q, t), y, q);
+    return m < 0x1p-90f && m != 0.f ? quot_small(t, d, y) : q;
+}
+
 // First difference (without 1/h) of two cells from the eight neighbours
 // m_k = p_-k, p_k = p_+k: d_1 (p_1 - m_1) + d_2 (p_2 - m_2) + d_3 (p_3 - m_3) +
 // d_4 (p_4 - m_4), each further term one fused multiply-add
