@@ -423,14 +423,15 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ S
         // this step's wavelet sample (fetched one step ahead)
         const float wn = wnext;
         if (!ADJ && has_inj && n + 1 < R.n1) wnext = wav[n + 1];
-        // this step's imaging terms, in flight during the wait
+        // this step's imaging terms, in flight during the wait (FP16: as they lie, two words)
         const long long slot = MODE == kResRecord ? n - R.n0 : R.n1 - 1 - n;
         char *const qs = R.q + slot * R.qstride;
         // FP16 slots: a warp's scale lies in the shot's top ghost rows, which hold nothing else
         float *const qsc = reinterpret_cast<float *>(reinterpret_cast<__half *>(qs) + sh) + tile * NWR + w;
         float4 qv[RZ];
+        float qs1 = 1.f;
         if (MODE == kResAdjoint) {
-            const float s = A.q_fp16 ? *qsc : 1.f;
+            qs1 = A.q_fp16 ? *qsc : 1.f;
 #pragma unroll
             for (int j = 0; j < RZ; j++) {
                 qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -438,9 +439,8 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ S
                 const long long o = sh + org + lo + j * P;
                 if (A.q_fp16) {
                     const uint2 u = *reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(qs) + o);
-                    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&u.x)),
-                                 b = __half22float2(*reinterpret_cast<const __half2 *>(&u.y));
-                    qv[j] = make_float4(a.x * s, a.y * s, b.x * s, b.y * s);
+                    qv[j].x = __uint_as_float(u.x);
+                    qv[j].y = __uint_as_float(u.y);
                 } else {
                     qv[j] = ld4(reinterpret_cast<const float *>(qs) + o);
                 }
@@ -721,6 +721,12 @@ const float4 y4 = ld4(KA + lz * TX + 4 * lane);
             if (ADJ) {
                 float *gp = GG + lz * TX + 4 * lane;
                 float4 gv = ld4(gp);
+                if (A.q_fp16) {
+                    const unsigned u0 = __float_as_uint(qv[j].x), u1 = __float_as_uint(qv[j].y);
+                    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&u0)),
+                                 b = __half22float2(*reinterpret_cast<const __half2 *>(&u1));
+                    qv[j] = make_float4(a.x * qs1, a.y * qs1, b.x * qs1, b.y * qs1);
+                }
                 gv.x += res[0] * qv[j].x;
                 gv.y += res[1] * qv[j].y;
                 gv.z += res[2] * qv[j].z;
