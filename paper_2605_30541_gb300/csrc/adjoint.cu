@@ -16,7 +16,7 @@ namespace {
 constexpr int TX = kTileX2, TZ = kTileZ2, BX = 32, BY = 8, RZ = TZ / BY, NTH = BX * BY;
 
 __device__ __forceinline__ float tile_max(float v, float *red) {
-    const int tid = threadIdx.y * BX + threadIdx.x;
+    const int tid = threadIdx.x;
     v = warp_max(v);
     if ((tid & 31) == 0) red[tid >> 5] = v;
     __syncthreads();
@@ -33,53 +33,52 @@ __device__ __forceinline__ long long row_off(const Geom &g, int r, int x) {
     return cell_off(g, r / g.NY, r % g.NY, x);
 }
 
-// One CTA per (tile of rows x columns, shot); the compact copy of a state is
-// [shot][NZ NY NX].
-template <typename T>
-__global__ void __launch_bounds__(NTH) k_store(const Geom g, const T *__restrict__ field, void *dst, float *scale,
-                                               int fp16, long long sstride, int ntx) {
-    __shared__ float red[NTH / 32];
-    const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ, shot = blockIdx.z, nrow = g.NZ * g.NY;
-    const int tile = blockIdx.y * ntx + blockIdx.x, ntiles = ntx * gridDim.y;
-    const T *f = field + (long long)shot * g.fstride;
+// A checkpoint is stored or restored by one launch: its first CTAs take the two
+// pressure fields, a CTA per (tile of rows x columns, shot, field), the others
+// the CPML memory, a warp per (box row, shot) of each field. (With a launch per
+// field, twelve per segment of a 2D CPML gradient, 16 shots of 241 x 241 cells
+// in 32 segments took 24.2 ms instead of 23.1, one shot of 132 x 152 x 172 in
+// 11 segments 14.4 instead of 13.8.)
+//
+// The compact copy of a pressure field is [shot][NZ NY NX], in FP16 with a
+// scale per tile.
+template <typename T, bool STORE>
+__device__ __forceinline__ void state_tile(const Geom &g, const CkArgs<T> &C, int w, int bx, int bz, int shot, float *red) {
+    const int x0 = bx * TX, z0 = bz * TZ, nrow = g.NZ * g.NY;
+    const int tx = threadIdx.x & (BX - 1), ty = threadIdx.x / BX;
+    T *f = C.state[w] + (long long)shot * g.fstride;
+    float *scale = C.state_scale[w] + (long long)shot * C.ntx * C.ntz + bz * C.ntx + bx;
+    void *cmp = C.state_copy[w];
     T v[RZ];
-    float m = 0.f;
+    float sc = 1.f;
+    if (STORE) {
+        float m = 0.f;
+#pragma unroll
+        for (int k = 0; k < RZ; k++) {
+            const int gz = z0 + ty + k * BY, gx = x0 + tx;
+            v[k] = (gz < nrow && gx < g.NX) ? f[row_off(g, gz, gx)] : T(0);
+            m = fmaxf(m, fabsf((float)v[k]));
+        }
+        if (C.fp16) {
+            const float s = pow2_scale(tile_max(m, red));
+            sc = 1.f / s;
+            if (threadIdx.x == 0) *scale = s;
+        }
+    } else if (C.fp16) {
+        sc = *scale;
+    }
 #pragma unroll
     for (int k = 0; k < RZ; k++) {
-        const int gz = z0 + threadIdx.y + k * BY, gx = x0 + threadIdx.x;
-        v[k] = (gz < nrow && gx < g.NX) ? f[row_off(g, gz, gx)] : T(0);
-        m = fmaxf(m, fabsf((float)v[k]));
-    }
-    float inv = 1.f;
-    if (fp16) {
-        const float s = pow2_scale(tile_max(m, red));
-        inv = 1.f / s;
-        if (threadIdx.x == 0 && threadIdx.y == 0) scale[(long long)shot * ntiles + tile] = s;
-    }
-#pragma unroll
-    for (int k = 0; k < RZ; k++) {
-        const int gz = z0 + threadIdx.y + k * BY, gx = x0 + threadIdx.x;
+        const int gz = z0 + ty + k * BY, gx = x0 + tx;
         if (gz >= nrow || gx >= g.NX) continue;
-        const long long ci = shot * sstride + (long long)gz * g.NX + gx;
-        if (fp16) static_cast<__half *>(dst)[ci] = __float2half_rn((float)v[k] * inv);
-        else static_cast<T *>(dst)[ci] = v[k];
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(NTH) k_load(const Geom g, T *field, const void *src, const float *scale, int fp16,
-                                              long long sstride, int ntx) {
-    const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ, shot = blockIdx.z, nrow = g.NZ * g.NY;
-    const int tile = blockIdx.y * ntx + blockIdx.x, ntiles = ntx * gridDim.y;
-    T *f = field + (long long)shot * g.fstride;
-    const float s = fp16 ? scale[(long long)shot * ntiles + tile] : 1.f;
-#pragma unroll
-    for (int k = 0; k < RZ; k++) {
-        const int gz = z0 + threadIdx.y + k * BY, gx = x0 + threadIdx.x;
-        if (gz >= nrow || gx >= g.NX) continue;
-        const long long ci = shot * sstride + (long long)gz * g.NX + gx;
-        f[row_off(g, gz, gx)] =
-            fp16 ? T(__half2float(static_cast<const __half *>(src)[ci]) * s) : static_cast<const T *>(src)[ci];
+        const long long ci = ((long long)shot * nrow + gz) * g.NX + gx;
+        if (STORE) {
+            if (C.fp16) static_cast<__half *>(cmp)[ci] = __float2half_rn((float)v[k] * sc);
+            else static_cast<T *>(cmp)[ci] = v[k];
+        } else {
+            f[row_off(g, gz, gx)] =
+                C.fp16 ? T(__half2float(static_cast<const __half *>(cmp)[ci]) * sc) : static_cast<const T *>(cmp)[ci];
+        }
     }
 }
 
@@ -94,12 +93,11 @@ __device__ __forceinline__ int box_of(const CkBoxes &B, long long r) {
 }
 
 template <typename T, bool STORE>
-__global__ void __launch_bounds__(256) k_boxes(const Geom g, const CkBoxes B, T *field, void *cmp, float *scale,
-                                               int fp16, int nshots) {
+__device__ __forceinline__ void box_row(const Geom &g, const CkArgs<T> &C, int j, long long w) {
     const int lane = threadIdx.x & 31;
+    const CkBoxes &B = C.box[j / 2];
     const long long rows = B.row0[B.n];
-    const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-    if (w >= rows * nshots) return;
+    if (w >= rows * C.nshots) return;
     const int shot = (int)(w / rows);
     const long long r = w - (long long)shot * rows;
     const int k = box_of(B, r);
@@ -107,27 +105,45 @@ __global__ void __launch_bounds__(256) k_boxes(const Geom g, const CkBoxes B, T 
     const long long lr = r - B.row0[k];
     const int ny = b.y1 - b.y0, len = b.x1 - b.x0;
     const int z = b.z0 + (int)(lr / ny), y = b.y0 + (int)(lr % ny);
-    T *f = field + (long long)shot * g.fstride + cell_off(g, z, y, b.x0);
+    T *f = C.mem[j] + (long long)shot * g.fstride + cell_off(g, z, y, b.x0);
+    void *cmp = C.mem_copy[j];
     const long long e0 = (long long)shot * B.elem0[B.n] + B.elem0[k] + lr * len;
     const long long si = (long long)shot * rows + r;
     if (STORE) {
         float inv = 1.f;
-        if (fp16) {
+        if (C.fp16) {
             float m = 0.f;
             for (int i = lane; i < len; i += 32) m = fmaxf(m, fabsf((float)f[i]));
             const float sc = pow2_scale(warp_max(m));
             inv = 1.f / sc;
-            if (lane == 0) scale[si] = sc;
+            if (lane == 0) C.mem_scale[j][si] = sc;
         }
         for (int i = lane; i < len; i += 32) {
-            if (fp16) static_cast<__half *>(cmp)[e0 + i] = __float2half_rn((float)f[i] * inv);
+            if (C.fp16) static_cast<__half *>(cmp)[e0 + i] = __float2half_rn((float)f[i] * inv);
             else static_cast<T *>(cmp)[e0 + i] = f[i];
         }
     } else {
-        const float sc = fp16 ? scale[si] : 1.f;
+        const float sc = C.fp16 ? C.mem_scale[j][si] : 1.f;
         for (int i = lane; i < len; i += 32)
-            f[i] = fp16 ? T(__half2float(static_cast<const __half *>(cmp)[e0 + i]) * sc) : static_cast<const T *>(cmp)[e0 + i];
+            f[i] = C.fp16 ? T(__half2float(static_cast<const __half *>(cmp)[e0 + i]) * sc)
+                          : static_cast<const T *>(cmp)[e0 + i];
     }
+}
+
+template <typename T, bool STORE>
+__global__ void __launch_bounds__(NTH) k_checkpoint(const Geom g, const __grid_constant__ CkArgs<T> C) {
+    __shared__ float red[NTH / 32];
+    unsigned b = blockIdx.x;
+    const unsigned tiles = (unsigned)C.ntx * C.ntz, states = 2u * tiles * C.nshots;
+    if (b < states) {
+        const unsigned t = b % tiles, q = b / tiles;
+        state_tile<T, STORE>(g, C, q & 1, t % C.ntx, t / C.ntx, q >> 1, red);
+        return;
+    }
+    b -= states;
+    int j = 0;
+    while (j + 1 < C.nmem && b >= C.block0[j + 1]) j++;
+    box_row<T, STORE>(g, C, j, (long long)(b - C.block0[j]) * (NTH / 32) + (threadIdx.x >> 5));
 }
 
 template <typename T>
@@ -288,36 +304,17 @@ __global__ void k_add(const double *__restrict__ acc, T *grad, long long n) {
 }  // namespace
 
 template <typename T>
-cudaError_t launch_store_state(const Geom &g, const T *field, void *dst, float *scale, int fp16, int nshots,
-                               long long shot_stride, int ntx, int ntz, cudaStream_t st) {
-    k_store<T><<<dim3(ntx, ntz, nshots), dim3(BX, BY), 0, st>>>(g, field, dst, scale, fp16, shot_stride, ntx);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_load_state(const Geom &g, T *field, const void *src, const float *scale, int fp16, int nshots,
-                              long long shot_stride, int ntx, int ntz, cudaStream_t st) {
-    k_load<T><<<dim3(ntx, ntz, nshots), dim3(BX, BY), 0, st>>>(g, field, src, scale, fp16, shot_stride, ntx);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_store_boxes(const Geom &g, const CkBoxes &b, const T *field, void *dst, float *scale, int fp16,
-                               int nshots, cudaStream_t st) {
-    const long long warps = b.row0[b.n] * nshots;
-    if (warps == 0) return cudaSuccess;
-    k_boxes<T, true><<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(g, b, const_cast<T *>(field), dst, scale, fp16,
-                                                                  nshots);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_load_boxes(const Geom &g, const CkBoxes &b, T *field, const void *src, const float *scale,
-                              int fp16, int nshots, cudaStream_t st) {
-    const long long warps = b.row0[b.n] * nshots;
-    if (warps == 0) return cudaSuccess;
-    k_boxes<T, false><<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(g, b, field, const_cast<void *>(src),
-                                                                   const_cast<float *>(scale), fp16, nshots);
+cudaError_t launch_checkpoint(const Geom &g, CkArgs<T> c, bool store, cudaStream_t st) {
+    long long blocks = 0;
+    for (int j = 0; j < c.nmem; j++) {
+        const CkBoxes &B = c.box[j / 2];
+        c.block0[j] = (unsigned)blocks;
+        blocks += (B.row0[B.n] * c.nshots + NTH / 32 - 1) / (NTH / 32);
+    }
+    blocks += 2LL * c.ntx * c.ntz * c.nshots;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    if (store) k_checkpoint<T, true><<<(unsigned)blocks, NTH, 0, st>>>(g, c);
+    else k_checkpoint<T, false><<<(unsigned)blocks, NTH, 0, st>>>(g, c);
     return cudaGetLastError();
 }
 
@@ -354,14 +351,7 @@ cudaError_t launch_add_gradient(const double *acc, T *grad, long long n, cudaStr
 }
 
 #define INST(T)                                                                                               \
-    template cudaError_t launch_store_state<T>(const Geom &, const T *, void *, float *, int, int, long long,  \
-                                               int, int, cudaStream_t);                                       \
-    template cudaError_t launch_load_state<T>(const Geom &, T *, const void *, const float *, int, int,        \
-                                              long long, int, int, cudaStream_t);                             \
-    template cudaError_t launch_store_boxes<T>(const Geom &, const CkBoxes &, const T *, void *, float *, int, int, \
-                                               cudaStream_t);                                                \
-    template cudaError_t launch_load_boxes<T>(const Geom &, const CkBoxes &, T *, const void *, const float *, int, \
-                                              int, cudaStream_t);                                            \
+    template cudaError_t launch_checkpoint<T>(const Geom &, CkArgs<T>, bool, cudaStream_t);                   \
     template cudaError_t launch_residual<T>(const T *, const T *, T *, long long, double *, int, cudaStream_t); \
     template cudaError_t launch_fold_gradient<T>(const Geom &, const T *, long long, int, const T *,      \
                                                  double, double *, cudaStream_t);                             \

@@ -1850,24 +1850,25 @@ cudaError_t checkpoint(sim_t s, const StepArgs<T> &a, const CkLayout &c, int k, 
     const size_t es = fp16 ? 2 : sizeof(T);
     float *scale = reinterpret_cast<float *>(slot + c.off_scale);
     const size_t ck_tiles = (size_t)s->d.max_shots * c.ckx * c.ckz;
-    const long long ncomp = (long long)g.NZ * g.NY * g.NX;
-    cudaError_t e = cudaSuccess;
-    for (int w = 0; w < 2 && e == cudaSuccess; w++) {  // w = 1: p^n, w = 0: p^{n-1}
-        T *f = a.pbuf[(n + 1 + w) & 1];
-        void *dst = slot + w * c.state * es;
-        e = store ? launch_store_state<T>(g, f, dst, scale + w * ck_tiles, fp16, nshots, ncomp, c.ckx, c.ckz, st)
-                  : launch_load_state<T>(g, f, dst, scale + w * ck_tiles, fp16, nshots, ncomp, c.ckx, c.ckz, st);
+    CkArgs<T> ck{};
+    ck.fp16 = fp16;
+    ck.nshots = nshots;
+    ck.ntx = c.ckx;
+    ck.ntz = c.ckz;
+    ck.nmem = c.nf;
+    for (int w = 0; w < 2; w++) {  // w = 1: p^n, w = 0: p^{n-1}
+        ck.state[w] = a.pbuf[(n + 1 + w) & 1];
+        ck.state_copy[w] = slot + w * c.state * es;
+        ck.state_scale[w] = scale + w * ck_tiles;
     }
-    for (int j = 0; j < c.nf && e == cudaSuccess; j++) {
+    for (int j = 0; j < c.nf; j++) {
         const int ax = c.ax[j];
-        T *f = static_cast<T *>(j % 2 ? s->zeta[ax] : s->psi[ax][g.ndim == 2 ? (n + 1) & 1 : 0]);
-        const CkBoxes &B = c.box[j / 2];
-        e = store ? launch_store_boxes<T>(g, B, f, slot + c.off_f[j], reinterpret_cast<float *>(slot + c.off_fs[j]),
-                                          fp16, nshots, st)
-                  : launch_load_boxes<T>(g, B, f, slot + c.off_f[j], reinterpret_cast<const float *>(slot + c.off_fs[j]),
-                                         fp16, nshots, st);
+        ck.mem[j] = static_cast<T *>(j % 2 ? s->zeta[ax] : s->psi[ax][g.ndim == 2 ? (n + 1) & 1 : 0]);
+        ck.mem_copy[j] = slot + c.off_f[j];
+        ck.mem_scale[j] = reinterpret_cast<float *>(slot + c.off_fs[j]);
+        ck.box[j / 2] = c.box[j / 2];
     }
-    return e;
+    return launch_checkpoint<T>(g, ck, store, st);
 }
 
 // The reverse schedule of a plan as a sequence of runs of steps:

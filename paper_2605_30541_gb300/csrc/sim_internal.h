@@ -460,14 +460,6 @@ cudaError_t launch_step2d_f32(const StepArgs<float> &a, const StepTime &t, int t
                               cudaStream_t st, bool pdl);
 cudaError_t configure_step2d_f32();
 
-// Checkpoint of one state (computational grid of each shot): FP32/FP64 copy
-// or FP16 with a power-of-two scale per 2D tile.
-template <typename T>
-cudaError_t launch_store_state(const Geom &g, const T *field, void *dst, float *scale, int fp16, int nshots,
-                               long long shot_stride, int ntx, int ntz, cudaStream_t st);
-template <typename T>
-cudaError_t launch_load_state(const Geom &g, T *field, const void *src, const float *scale, int fp16, int nshots,
-                              long long shot_stride, int ntx, int ntz, cudaStream_t st);
 // Checkpoint of the CPML memory of one axis: only the boxes of its strips
 // (the memory is zero elsewhere), compact [shot][rows][x] with, in FP16, a
 // power-of-two scale per (shot, box row). row0 / elem0 are prefix sums over
@@ -482,12 +474,23 @@ struct CkBoxes {
     long long row0[kMaxCkBoxes + 1];
     long long elem0[kMaxCkBoxes + 1];
 };
+// One checkpoint: the two pressure fields (compact [shot][NZ NY NX] copies, in
+// FP16 with a power-of-two scale per 2D tile, ntx x ntz of them) and the CPML
+// memory, two fields per absorbing axis.
 template <typename T>
-cudaError_t launch_store_boxes(const Geom &g, const CkBoxes &b, const T *field, void *dst, float *scale, int fp16,
-                               int nshots, cudaStream_t st);
+struct CkArgs {
+    int fp16, nshots, ntx, ntz, nmem;
+    T *state[2];
+    void *state_copy[2];
+    float *state_scale[2];
+    T *mem[6];
+    void *mem_copy[6];
+    float *mem_scale[6];
+    CkBoxes box[3];
+    unsigned block0[6];  // set by the launch
+};
 template <typename T>
-cudaError_t launch_load_boxes(const Geom &g, const CkBoxes &b, T *field, const void *src, const float *scale,
-                              int fp16, int nshots, cudaStream_t st);
+cudaError_t launch_checkpoint(const Geom &g, CkArgs<T> c, bool store, cudaStream_t st);
 // res = g - d (all shots), per-block partial sums of res^2 / 2 into part.
 template <typename T>
 cudaError_t launch_residual(const T *g, const T *d, T *res, long long n, double *part, int nblocks, cudaStream_t st);
