@@ -63,6 +63,7 @@
 // of the previous step, which a schedule without a grid barrier lacks.
 #include <algorithm>
 #include <cfloat>
+#include <type_traits>
 
 #include "f32_tile.cuh"
 #include "sim_internal.h"
@@ -144,7 +145,7 @@ __device__ __forceinline__ void d2x_pairs(const float4 &L, const float4 &C, cons
     db = d2c2(hi2(C), v56, v78, lo2(C), lo2(R), v34, v910, hi2(L), hi2(R));
 }
 
-template <int RZ, int MODE>
+template <int RZ, int MODE, bool QH>
 __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ StepArgs<float> A,
                                                        const __grid_constant__ ResidentArgs R) {
     constexpr int WZ = NWR * RZ;
@@ -428,22 +429,19 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ S
         char *const qs = R.q + slot * R.qstride;
         // FP16 slots: a warp's scale lies in the shot's top ghost rows, which hold nothing else
         float *const qsc = reinterpret_cast<float *>(reinterpret_cast<__half *>(qs) + sh) + tile * NWR + w;
-        float4 qv[RZ];
+        std::conditional_t<ADJ && QH, uint2, float4> qv[RZ];
         float qs1 = 1.f;
         if (MODE == kResAdjoint) {
-            qs1 = A.q_fp16 ? *qsc : 1.f;
+            if constexpr (QH) qs1 = *qsc;
 #pragma unroll
             for (int j = 0; j < RZ; j++) {
-                qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                qv[j] = {};
                 if (j >= rpw || w * rpw + j >= rows) continue;
                 const long long o = sh + org + lo + j * P;
-                if (A.q_fp16) {
-                    const uint2 u = *reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(qs) + o);
-                    qv[j].x = __uint_as_float(u.x);
-                    qv[j].y = __uint_as_float(u.y);
-                } else {
+                if constexpr (ADJ && QH)
+                    qv[j] = *reinterpret_cast<const uint2 *>(reinterpret_cast<const __half *>(qs) + o);
+                else
                     qv[j] = ld4(reinterpret_cast<const float *>(qs) + o);
-                }
             }
         }
 
@@ -711,30 +709,31 @@ const float4 y4 = ld4(KA + lz * TX + 4 * lane);
                 if (hasW && 4 * lane < H) put4(ob + XWST + lz * HM + 4 * lane, r4, tag + 1);
                 if (hasE && 4 * lane >= TX - H) put4(ob + XEST + lz * HM + 4 * lane - (TX - H), r4, tag + 1);
             }
-            if (MODE == kResRecord) {
+            if constexpr (MODE == kResRecord) {
                 qv[j] = make_float4(qk[0], qk[1], qk[2], qk[3]);
-                if (A.q_fp16)
+                if (QH)
                     tmax = fmaxf(tmax, fmaxf(fmaxf(fabsf(qk[0]), fabsf(qk[1])), fmaxf(fabsf(qk[2]), fabsf(qk[3]))));
                 else
                     st4(reinterpret_cast<float *>(qs) + sh + org + lo + j * P, qv[j]);
             }
-            if (ADJ) {
+            if constexpr (ADJ) {
                 float *gp = GG + lz * TX + 4 * lane;
-                float4 gv = ld4(gp);
-                if (A.q_fp16) {
-                    const unsigned u0 = __float_as_uint(qv[j].x), u1 = __float_as_uint(qv[j].y);
-                    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&u0)),
-                                 b = __half22float2(*reinterpret_cast<const __half2 *>(&u1));
-                    qv[j] = make_float4(a.x * qs1, a.y * qs1, b.x * qs1, b.y * qs1);
+                float4 gv = ld4(gp), q;
+                if constexpr (QH) {
+                    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&qv[j].x)),
+                                 b = __half22float2(*reinterpret_cast<const __half2 *>(&qv[j].y));
+                    q = make_float4(a.x * qs1, a.y * qs1, b.x * qs1, b.y * qs1);
+                } else {
+                    q = qv[j];
                 }
-                gv.x += res[0] * qv[j].x;
-                gv.y += res[1] * qv[j].y;
-                gv.z += res[2] * qv[j].z;
-                gv.w += res[3] * qv[j].w;
+                gv.x += res[0] * q.x;
+                gv.y += res[1] * q.y;
+                gv.z += res[2] * q.z;
+                gv.w += res[3] * q.w;
                 st4(gp, gv);
             }
         }
-        if (MODE == kResRecord && A.q_fp16) {  // one power-of-two scale per warp and step
+        if constexpr (MODE == kResRecord && QH) {  // one power-of-two scale per warp and step
             const float s = pow2_scale(warp_max(tmax)), inv = 1.f / s;
             if (lane == 0) *qsc = s;
 #pragma unroll
@@ -836,7 +835,7 @@ const float4 y4 = ld4(KA + lz * TX + 4 * lane);
     }
 }
 
-template <int RZ, int MODE>
+template <int RZ, int MODE, bool QH>
 cudaError_t launch_rz(const StepArgs<float> &a, const ResidentArgs &r, int nshots, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(r.ntiles * nshots);
@@ -848,20 +847,23 @@ cudaError_t launch_rz(const StepArgs<float> &a, const ResidentArgs &r, int nshot
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_resident2d<RZ, MODE>, a, r);
+    return cudaLaunchKernelEx(&cfg, k_resident2d<RZ, MODE, QH>, a, r);
 }
 
 template <int RZ>
 cudaError_t launch_mode(const StepArgs<float> &a, const ResidentArgs &r, int mode, int nshots, cudaStream_t st) {
-    if (mode == kResRecord) return launch_rz<RZ, kResRecord>(a, r, nshots, st);
-    if (mode == kResAdjoint) return launch_rz<RZ, kResAdjoint>(a, r, nshots, st);
-    return launch_rz<RZ, kResForward>(a, r, nshots, st);
+    const bool qh = a.q_fp16 != 0;
+    if (mode == kResForward) return launch_rz<RZ, kResForward, false>(a, r, nshots, st);
+    if (mode == kResRecord)
+        return qh ? launch_rz<RZ, kResRecord, true>(a, r, nshots, st) : launch_rz<RZ, kResRecord, false>(a, r, nshots, st);
+    return qh ? launch_rz<RZ, kResAdjoint, true>(a, r, nshots, st) : launch_rz<RZ, kResAdjoint, false>(a, r, nshots, st);
 }
 
 template <int RZ>
 cudaError_t configure_rz() {
     cudaError_t e = cudaSuccess;
-    for (auto k : {k_resident2d<RZ, kResForward>, k_resident2d<RZ, kResRecord>, k_resident2d<RZ, kResAdjoint>})
+    for (auto k : {k_resident2d<RZ, kResForward, false>, k_resident2d<RZ, kResRecord, false>, k_resident2d<RZ, kResRecord, true>,
+                   k_resident2d<RZ, kResAdjoint, false>, k_resident2d<RZ, kResAdjoint, true>})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentMaxSmem - 64);
     return e;
