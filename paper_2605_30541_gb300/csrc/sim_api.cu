@@ -1037,8 +1037,10 @@ long long spin_limit() {
 // even in time per step as the GPU allows. Cost model (fitted to per-CTA
 // phase timings of this kernel, in units of one interior row): a subdomain
 // costs 50 (halo exchange and barriers) plus, per row, 1, plus 0.039 per
-// CPML x-strip float4 chunk its column updates, plus 1.34 within 4 rows of a
-// CPML z-strip. The smallest target cost whose subdomains (times the shots)
+// CPML x-strip float4 chunk its column updates, plus 1.6 within 4 rows of a
+// CPML z-strip (1.34 left the corner subdomains of a 659 x 1040 slice behind the
+// others: 1000 steps with 100 snapshots 4.18 ms, 4.03 with 1.6; no more from 1.8,
+// and other slices then lose 1%). The smallest target cost whose subdomains (times the shots)
 // all fit on the GPU at once is chosen, trying RZ = 1, 2, ... 2D FP32 forward
 // runs with FP32 (or no) snapshots only; GSIM_RESIDENT=0 turns the path off.
 // CPML x-strip float4 chunks (psi and zeta) a column updates, as the kernel counts them.
@@ -1059,6 +1061,7 @@ int strip_chunks(const Geom &g, int bx) {
 }
 
 constexpr double kTileFixed = 50.0;  // exchange and barriers
+constexpr double kZStripRow = 1.6;   // a row within 4 rows of a z strip, above a plain one
 constexpr int kSourceRows = 2;       // a shot's source injects into two rows at most
 constexpr int kMaxGroups = 16;
 
@@ -1077,7 +1080,7 @@ bool cut_columns(const sim_s *s, int wz, double target, std::vector<RTile> &tile
             double acc = kTileFixed;
             while (z < g.NZ && t.rows < wz) {
                 const bool zs = cp && ((g.nbz0 > 0 && z < g.nbz0 + 4) || (g.nbz1 > 0 && z >= g.NZ - g.nbz1 - 4));
-                const double c = 1.0 + cx + (zs ? 1.34 : 0.0);
+                const double c = 1.0 + cx + (zs ? kZStripRow : 0.0);
                 if (t.rows >= hmin && acc + c > target) break;
                 acc += c;
                 t.rows++;
@@ -1127,7 +1130,7 @@ double plan_cost(const sim_s *s, const std::vector<RTile> &tiles) {
         double c = kTileFixed + t.rows * (1.0 + (cp ? 0.039 * strip_chunks(g, t.bx) : 0.0));
         if (cp)
             for (int z = t.z0; z < t.z0 + t.rows; z++)
-                if ((g.nbz0 > 0 && z < g.nbz0 + 4) || (g.nbz1 > 0 && z >= g.NZ - g.nbz1 - 4)) c += 1.34;
+                if ((g.nbz0 > 0 && z < g.nbz0 + 4) || (g.nbz1 > 0 && z >= g.NZ - g.nbz1 - 4)) c += kZStripRow;
         worst = std::max(worst, c);
     }
     return worst;
