@@ -703,7 +703,7 @@ const float4 y4 = ld4(KA + lz * TX + 4 * lane);
             const float4 r4 = make_float4(res[0], res[1], res[2], res[3]);
             if (top && lz >= 1 && lz <= H) st4(nxt + (HM - lz) * SW + c0, neg4(r4));  // odd mirror above the free surface
             st4(nxt + (rb + j) * SW + c0, r4);
-            if (n + 1 < R.n1) {
+            if (RZ < 3 && n + 1 < R.n1) {
                 if (hasN && lz < H) put4(ob + XN + lz * TX + 4 * lane, r4, tag + 1);
                 if (hasS && lz >= rows - H) put4(ob + XS + (lz - rows + H) * TX + 4 * lane, r4, tag + 1);
                 if (hasW && 4 * lane < H) put4(ob + XWST + lz * HM + 4 * lane, r4, tag + 1);
@@ -732,6 +732,28 @@ const float4 y4 = ld4(KA + lz * TX + 4 * lane);
                 gv.w += res[3] * q.w;
                 st4(gp, gv);
             }
+        }
+        // Borders of tall subdomains, from the rows just written: few instances of
+        // the sending code for the instruction cache, and the side columns of all
+        // rows at once (with 4 rows per warp a gradient of 16 shots 22.35 -> 21.76
+        // ms, with 3 a slice 4.03 -> 4.01; with 1 or 2 rows, where a send per row
+        // in place starts earlier, 2.84 -> 2.90 and 6.13 -> 6.17)
+        if (RZ >= 3 && n + 1 < R.n1) {
+            __syncwarp();
+            const int w0 = w * rpw, w1 = min(w0 + rpw, rows);
+            if (hasN)
+#pragma unroll 1
+                for (int lz = w0; lz < min(w1, H); lz++)
+                    put4(ob + XN + lz * TX + 4 * lane, ld4(nxt + (HM + lz) * SW + c0), tag + 1);
+            if (hasS)
+#pragma unroll 1
+                for (int lz = max(w0, rows - H); lz < w1; lz++)
+                    put4(ob + XS + (lz - rows + H) * TX + 4 * lane, ld4(nxt + (HM + lz) * SW + c0), tag + 1);
+            // lane: (row, side, float4)
+            const int b = cpml ? 2 : 1, lz = w0 + (lane >> b), east = (lane >> (b - 1)) & 1, q = cpml ? lane & 1 : 0;
+            if (lz < w1 && (east ? hasE : hasW))
+                put4(ob + (east ? XEST : XWST) + lz * HM + 4 * q, ld4(nxt + (HM + lz) * SW + HM + (east ? TX - H : 0) + 4 * q),
+                     tag + 1);
         }
         if constexpr (MODE == kResRecord && QH) {  // one power-of-two scale per warp and step
             const float s = pow2_scale(warp_max(tmax)), inv = 1.f / s;
