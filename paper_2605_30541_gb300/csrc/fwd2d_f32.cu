@@ -77,8 +77,11 @@ constexpr size_t smem_floats(bool cpml) {
 // One tile of one step: the whole CTA updates the 128 x TZ tile (bx, bz) of
 // `shot`. Shared by the per-step kernel (one tile per CTA) and the persistent
 // batch kernel (a work list of tiles). With PDL the fields of the previous
-// step are touched only after cudaGridDependencySynchronize().
-template <int TZ, int MODE, bool PDL>
+// step are touched only after cudaGridDependencySynchronize(). CP: the CPML code is
+// there; launches without CPML run an instance that it costs neither registers
+// nor instruction fetch (one 679 x 1120 sponge shot, 701 steps with FP16
+// snapshots: 4.58 ms with one instance for both, 4.13 now).
+template <int TZ, int MODE, bool PDL, bool CP>
 __device__ __forceinline__ void tile_step(const StepArgs<float> &A, const StepTime &t, const int bx, const int bz,
                                           const int shot, float *S, float *red) {
     constexpr int RZ = TZ / NW;
@@ -97,7 +100,7 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &A, const StepTi
     float *pnb = A.pbuf[(t.n + 1) & 1] + sh + org;          // p^{n-1} in, p^{n+1} out
     const float *chb = A.ch + org;
 
-    const bool cpml = A.bc == SIM_BC_CPML;
+    const bool cpml = CP && A.bc == SIM_BC_CPML;
     const bool cpx = cpml && A.ca[2] &&
                      ((g.nbx0 > 0 && x0 - 4 < g.nbx0) || (g.nbx1 > 0 && x0 + TX + 4 > g.NX - g.nbx1));
     const bool cpz = cpml && A.ca[0] &&
@@ -105,6 +108,11 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &A, const StepTi
     const bool spg = A.bc == SIM_BC_SPONGE &&
                      ((g.nbx0 > 0 && x0 < g.nbx0) || (g.nbx1 > 0 && x0 + TX > g.NX - g.nbx1) ||
                       (g.nbz0 > 0 && z0 < g.nbz0) || (g.nbz1 > 0 && z0 + TZ > g.NZ - g.nbz1));
+    // rows in a z strip widened by r: elsewhere psi_z and zeta_z are and stay zero, and
+    // the addend with them (4 shots of 279 x 364 cells, 691 steps: 5.54 ms with every
+    // row of a z-strip tile in full, 4.92 now; the same test along x, lane by lane, gave
+    // no more)
+    auto meets_z = [&](int z, int r) { return (g.nbz0 > 0 && z < g.nbz0 + r) || (g.nbz1 > 0 && z >= g.NZ - g.nbz1 - r); };
     const bool xedge = x0 + TX > g.NX;          // last tile column: mask cells beyond NX
     const bool zedge = z0 + TZ > g.NZ;          // last tile row: skip rows beyond NZ
     const bool top = g.fs && z0 == 0;           // free-surface tile
@@ -220,6 +228,7 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &A, const StepTi
 #pragma unroll
         for (int j = 0; j < RZ + 1; j++) {
             const int lzz = -4 + w + NW * j, gz = z0 + lzz;
+            if (!meets_z(gz, 0)) continue;
             const float *col = S + (HM + lzz) * SW + c0;
             float4 q[9];
 #pragma unroll
@@ -274,7 +283,7 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &A, const StepTi
                 }
                 st4(zp, make_float4(zo[0], zo[1], zo[2], zo[3]));
             }
-            if (cpz) {
+            if (cpz && meets_z(gz, 4)) {
                 const float *col = S + (rb + j) * SW + c0;
                 const float *pzc = PZ + (lz + 4) * TX + 4 * lane;
                 const float az = __ldg(A.ca[0] + gz), bz = __ldg(A.cb[0] + gz);
@@ -459,11 +468,11 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &A, const StepTi
     }
 }
 
-template <int TZ, int MODE>
+template <int TZ, int MODE, bool CP>
 __global__ void __launch_bounds__(NTH, 2) k_step2d_f32(const StepArgs<float> A, const StepTime t) {
     extern __shared__ float4 smem4[];
     __shared__ float red[NW];
-    tile_step<TZ, MODE, true>(A, t, blockIdx.x, blockIdx.y, blockIdx.z, reinterpret_cast<float *>(smem4), red);
+    tile_step<TZ, MODE, true, CP>(A, t, blockIdx.x, blockIdx.y, blockIdx.z, reinterpret_cast<float *>(smem4), red);
 }
 
 // ---------------------------------------------------------------- batch
@@ -551,7 +560,7 @@ __global__ void __launch_bounds__(NTH, 2) k_batch2d(const BatchArgs B) {
         t.n = n;
         t.snap_k = t.max_k = -1;
         t.inj_row = n;
-        tile_step<TZ, kModeForward, false>(sA, t, bx, bz, M.shot, reinterpret_cast<float *>(smem4), red);
+        tile_step<TZ, kModeForward, false, true>(sA, t, bx, bz, M.shot, reinterpret_cast<float *>(smem4), red);
         __syncthreads();
         if (tid == 0) {
             __threadfence();
@@ -596,7 +605,7 @@ __global__ void __launch_bounds__(NTH, 2) k_multi2d(const BatchArgs B, const int
     t.n = n;
     t.snap_k = t.max_k = -1;
     t.inj_row = n;
-    tile_step<TZ, kModeForward, true>(sA, t, bx, bz, M.shot, reinterpret_cast<float *>(smem4), red);
+    tile_step<TZ, kModeForward, true, true>(sA, t, bx, bz, M.shot, reinterpret_cast<float *>(smem4), red);
 }
 
 template <int TZ, int MODE>
@@ -612,13 +621,18 @@ cudaError_t launch_mode(const StepArgs<float> &a, const StepTime &t, int nshots,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_step2d_f32<TZ, MODE>, a, t);
+    return cp ? cudaLaunchKernelEx(&cfg, k_step2d_f32<TZ, MODE, true>, a, t)
+              : cudaLaunchKernelEx(&cfg, k_step2d_f32<TZ, MODE, false>, a, t);
 }
 
 template <int TZ, int MODE>
 cudaError_t configure_one() {
-    return cudaFuncSetAttribute(k_step2d_f32<TZ, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(smem_floats<TZ>(true) * sizeof(float)));
+    cudaError_t e = cudaFuncSetAttribute(k_step2d_f32<TZ, MODE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(smem_floats<TZ>(true) * sizeof(float)));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_step2d_f32<TZ, MODE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(smem_floats<TZ>(false) * sizeof(float)));
+    return e;
 }
 
 template <int TZ>
