@@ -52,8 +52,8 @@
 // kernel raises kFlagTimeout and every CTA returns.
 //
 // Measured (gradients, per-step kernels and this): 16 shots of 241 x 241 cells,
-// 1000 steps, CPML, FP16 checkpoints 58.3 and 24.5 ms; 4 shots of 231 x 381,
-// 600 steps, sponge, with the forward of the loss 13.0 and 6.3 ms.
+// 1000 steps, CPML, FP16 checkpoints 58.2 and 21.5 ms; 4 shots of 231 x 381,
+// 600 steps, sponge, with the forward of the loss 13.0 and 6.1 ms.
 //
 // The scheme is the leapfrog update with the centred sponge term or the CPML
 // memory terms (Sec. 2, App. E.3-E.4), free surface as an odd mirror with
