@@ -208,6 +208,14 @@ struct TileMap {
     std::vector<int> z0;    // [tile]
 };
 
+// What a captured time loop depends on beyond the handle's buffers: its kind,
+// then that kind's values, compared one by one. (Values packed into one word by
+// shifts met when a shot count and a group size had overlapping bits: on 201 x
+// 201 cells with 20 CPML cells a gradient of 30 shots replayed the launches of
+// one of 14.)
+using GraphKey = std::vector<long long>;
+enum { kGraphForward, kGraphMarch, kGraphForward3D, kGraphGradient, kGraphResidentGradient, kGraphGradient3D };
+
 // Resident-path decomposition of one shot count (see plan_resident).
 struct ResidentPlan {
     int rz = 0;                // 0: the run does not fit on chip
@@ -262,11 +270,11 @@ struct sim_s {
     void *inj_ent = nullptr;  // InjEntryT<T>
     size_t cap_rec = 0, cap_grp = 0, cap_start = 0;
     unsigned *flags_host = nullptr;  // pinned copy of the device flags
-    // time loops are captured once per (kind, nshots) and replayed as CUDA graphs
+    // time loops are captured once per key and replayed as CUDA graphs
     // on a handle-owned stream, ordered with the caller's stream by events
     cudaStream_t cst = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-    std::vector<std::pair<long long, cudaGraphExec_t>> graphs;
+    std::vector<std::pair<GraphKey, cudaGraphExec_t>> graphs;
     bool use_graphs = true;
     int tuned_nshots = 0;  // shot count the tile shape was tuned for (0: not yet)
     bool use_march = false; // the autotuner's choice: row march rather than the tiled step kernel
@@ -687,7 +695,7 @@ cudaError_t launch_step<double>(sim_t s, const StepArgs<double> &a, int n, int n
 // (captured on first use, replayed afterwards), ordered after everything
 // already queued on the handle's stream and before anything queued later.
 template <typename F>
-sim_status run_graph(sim_t s, long long key, F body) {
+sim_status run_graph(sim_t s, const GraphKey &key, F body) {
     if (!s->use_graphs) {
         cudaError_t e = body(s->st);
         return s->cuda(e, "time loop");
@@ -1010,8 +1018,7 @@ sim_status forward3d(sim_t s, int nshots, const void *wav, const double *src_pos
     a.sample = nrec > 0 && gdev != nullptr;
     const bool has_src = !src.empty(), has_snap = io.snaps != nullptr;
     const Pt3 *s3 = s->src3, *r3 = s->rec3;
-    const long long key = ((long long)nrec << 32) | ((long long)nshots << 8) | (a.sample << 7) | (has_src << 6) |
-                          (has_snap << 5) | (3 << 2) | 2;
+    const GraphKey key = {kGraphForward3D, nshots, nrec, a.sample, has_src, has_snap};
     return run_graph(s, key, [&](cudaStream_t st) {
         cudaError_t e = cudaSuccess;
         for (int n = 0; n < d.nt && e == cudaSuccess; n++) {
@@ -1288,10 +1295,6 @@ sim_status run_resident<float>(sim_t s, const StepArgs<float> &a, const Resident
     return s->cuda(launch_resident2d(a, r, plan.rz, kResForward, nshots, s->st), "resident launch");
 }
 
-// What a captured gradient depends on beyond the handle's buffers.
-long long resident_key(const ResidentPlan &plan) {
-    return (((long long)plan.group << 20) ^ (plan.lay[kResAdjoint].injr << 8) ^ 1) << 24 ^ spin_limit() * 0x9e3779b97f4aLL;
-}
 // Lists follow the resident subdomains while this lasts.
 struct MapScope {
     sim_t s;
@@ -1423,8 +1426,7 @@ sim_status run_march<float>(sim_t s, const StepArgs<float> &a, int nshots) {
     MarchArgs m{};
     if (sim_status r = march_prepare(s, a, nshots, m)) return r;
     const bool cpml = s->d.bc == SIM_BC_CPML;
-    return run_graph(s, ((long long)nshots << 16) | ((long long)march_item_rows() << 8) | ((long long)s->tile_z << 2) | 3,
-                     [&](cudaStream_t st) {
+    return run_graph(s, {kGraphMarch, nshots, march_item_rows(), s->tile_z}, [&](cudaStream_t st) {
         cudaError_t e0 = cudaMemsetAsync(m.ctr, 0, 2 * sizeof(unsigned), st);
         if (e0 != cudaSuccess) return e0;
         for (int n = 0; n < s->d.nt; n++) {
@@ -1525,14 +1527,13 @@ sim_status forward_t(sim_t s, int nshots, const void *wavelet, const double *src
         if (sim_status r = run_resident(s, a, *plan, nshots)) return r;
     } else if (march) {
         if (sim_status r = run_march(s, a, nshots)) return r;
-    } else if (sim_status r = run_graph(s, ((long long)nshots << 8) | ((long long)s->tile_z << 2) | 1,
-                                        [&](cudaStream_t st) {
-                                            for (int n = 0; n < d.nt; n++) {
-                                                cudaError_t e = launch_step<T>(s, a, n, nshots, kModeForward, st);
-                                                if (e != cudaSuccess) return e;
-                                            }
-                                            return cudaSuccess;
-                                        })) {
+    } else if (sim_status r = run_graph(s, {kGraphForward, nshots, s->tile_z}, [&](cudaStream_t st) {
+                   for (int n = 0; n < d.nt; n++) {
+                       cudaError_t e = launch_step<T>(s, a, n, nshots, kModeForward, st);
+                       if (e != cudaSuccess) return e;
+                   }
+                   return cudaSuccess;
+               })) {
         return r;
     }
     }
@@ -2102,8 +2103,7 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
     const int nrg = (int)rg.size();
     const bool fused = cpml && cpml3d_adjoint_fits(a);
     const Pt3 *r3 = s->rec3, *s3 = s->src3;
-    const long long gkey = ((long long)nshots << 40) ^ ((long long)nrec << 16) ^ ((long long)ckpt_fp16 << 3) ^
-                           ((long long)o.vjp << 5) ^ 6;
+    const GraphKey gkey = {kGraphGradient3D, nshots, nrec, ckpt_fp16, o.vjp};
     if (sim_status r = run_graph(s, gkey, [&](cudaStream_t st) {
             cudaError_t e = reset_state_on(s, nshots, st);
             if (e != cudaSuccess) return e;
@@ -2269,9 +2269,11 @@ sim_status adjoint_t(sim_t s, int nshots, const void *wavelet, const double *src
         adj.cext = static_cast<const T *>(s->cext);
     }
     const size_t qstride = q_slot_bytes(s, ckpt_fp16);
-    // graph key: everything the captured launches depend on beyond handle buffers
-    const long long gkey = ((long long)nshots << 40) ^ ((long long)nrec << 12) ^ ((long long)s->tile_z << 4) ^
-                           ((long long)ckpt_fp16 << 3) ^ ((long long)o.vjp << 9) ^ (plan ? resident_key(*plan) : 0) ^ 5;
+    GraphKey gkey = {plan ? kGraphResidentGradient : kGraphGradient, nshots, nrec, ckpt_fp16, o.vjp};
+    if (plan)  // its subdomains and shared-memory layouts follow from these
+        gkey.insert(gkey.end(), {plan->rz, plan->group, (long long)plan->tiles.size(), plan->lay[kResAdjoint].injr, spin_limit()});
+    else
+        gkey.push_back(s->tile_z);
     if (sim_status r = run_graph(s, gkey, [&](cudaStream_t st) {
             cudaError_t e = reset_state_on(s, nshots, st);
             if (e != cudaSuccess) return e;
