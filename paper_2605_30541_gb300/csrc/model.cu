@@ -27,9 +27,11 @@ constexpr int kMaxBeds = 128;
 // angles pi x_k / 4 lie 45 degrees apart: with a = pi fr / 4 and b = pi / 4 - a
 // their sines are sin b, cos a, cos b, sin a, -sin b, -cos a, -cos b, -sin a
 // for k = 0 .. 7. Two sine-cosine pairs and eight reciprocals in place of
-// sixteen sines and sixteen quotients.
+// sixteen sines and sixteen quotients. A hair above a sample, where 1 / fr^2
+// would overflow (fr below 5.4e-20) and every other weight is below 2^-40, the
+// sample itself is taken.
 __device__ __forceinline__ void tap_weights(float fr, float *w) {
-    if (!(fr > 0.f && fr < 1.f)) {  // on a sample (fr rounds to 1 just below the next one)
+    if (fr <= 0x1p-40f || fr >= 1.f) {  // on a sample (fr rounds to 1 just below the next one); not for NaN
 #pragma unroll
         for (int k = 0; k < kTaps; k++) w[k] = k == (fr < 1.f ? 3 : 4) ? 1.f : 0.f;
         return;
