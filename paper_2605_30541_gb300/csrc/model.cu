@@ -51,12 +51,16 @@ __device__ __forceinline__ void tap_weights(float fr, float *w) {
 #pragma unroll
     for (int k = 0; k < kTaps; k++) w[k] *= inv;
 }
-// first tap index and weights of the 8 taps around s
-__device__ __forceinline__ int taps(double s, float *w) {
+// First tap index and weights of the 8 taps around s. The index is held to
+// [-far, far] - 3 so that the sums formed with it do not overflow for positions
+// of any size; one that is no number reads some cell of the grid.
+__device__ __forceinline__ int taps(double s, int far, float *w) {
     const double f = floor(s);
     tap_weights((float)(s - f), w);
-    return (int)f - 3;
+    return max(-far, min(far, (int)f)) - 3;
 }
+constexpr int kFarPoint = 0x7fffffff - kTaps;  // positions
+constexpr int kFarShift = 1 << 30;             // displacements and offsets of depths below 2^30
 
 __device__ __forceinline__ int clampi(int i, int n) { return i < 0 ? 0 : (i >= n ? n - 1 : i); }
 
@@ -80,7 +84,7 @@ __global__ void k_squish(int nz, int ny, int nx, const float *__restrict__ v, co
     const long long col = (long long)y * nx + x, plane = (long long)ny * nx;
     const float d = dz[col];
     float w[kTaps];
-    const int s0 = taps((double)d, w);  // taps of row z: z + s0 .. z + s0 + 7
+    const int s0 = taps((double)d, kFarShift, w);  // taps of row z: z + s0 .. z + s0 + 7
     // the pulled depth z + d = (z + di) + fr with di = floor(d), fr in [0, 1)
     // exact in FP32, so the fill test and the nearest row are integer logic
     const int di = s0 + 3;
@@ -233,7 +237,7 @@ __device__ __forceinline__ void fault_voxel(int nz, int ny, int nx, const float 
         return;
     }
     float wzt[kTaps], wxt[kTaps];
-    const int iz0 = taps(sz, wzt), ix0 = taps(sx, wxt);
+    const int iz0 = taps(sz, kFarPoint, wzt), ix0 = taps(sx, kFarPoint, wxt);
     int xs[kTaps];
 #pragma unroll
     for (int c = 0; c < kTaps; c++) xs[c] = clampi(ix0 + c, nx);
@@ -249,7 +253,7 @@ __device__ __forceinline__ void fault_voxel(int nz, int ny, int nx, const float 
         }
     } else {
         float wyt[kTaps];
-        const int iy0 = taps(sy, wyt);
+        const int iy0 = taps(sy, kFarPoint, wyt);
         for (int a = 0; a < kTaps; a++) {
             const long long pz = (long long)clampi(iz0 + a, nz) * ny;
             float pa = 0.f;
@@ -491,7 +495,7 @@ extern "C" sim_status sim_model_deposit(int nz, int ny, int nx, const float *v_i
     double sum = 0.0;
     for (int b = 0; b < p->nbeds; b++) {
         K.vbed[b] = vbed[b];
-        K.off[b] = offsets[b];
+        K.off[b] = std::max(-kFarShift, std::min(kFarShift, offsets[b]));  // z - start + offset does not overflow
         sum += vbed[b];
     }
     K.vbar = (float)(sum / p->nbeds);
