@@ -42,7 +42,7 @@
 //     store, barrier, release, poll, barrier, fetch, barrier - the exchange
 //     alone took 2.55 us: 1000 steps of 241 x 241 cells 3.87 ms, of 669 x 1100
 //     with 100 snapshots 6.35 ms; 2.86 and 4.25 ms with the words.) The
-//     stencil is a cross, so corner neighbours are never needed.
+//     stencil is a cross, so it needs no corner neighbours; receivers may.
 //     Two outbox halves alternate by step parity: a CTA that writes p^{n+1}
 //     over p^{n-1} has read p^n from every neighbour that reads it, and each of
 //     them sent p^n only after a barrier behind all its reads of p^{n-1}. Tags
@@ -145,11 +145,14 @@ __device__ __forceinline__ void d2x_pairs(const float4 &L, const float4 &C, cons
     db = d2c2(hi2(C), v56, v78, lo2(C), lo2(R), v34, v910, hi2(L), hi2(R));
 }
 
-template <int RZ, int MODE, bool QH>
+// OPT: record and adjoint, FP16 imaging terms; forward, the corners are
+// exchanged (an instance of its own: one for both took 2.79 ms instead of 2.74
+// for 1000 steps of 241 x 241 cells).
+template <int RZ, int MODE, bool OPT>
 __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ StepArgs<float> A,
                                                        const __grid_constant__ ResidentArgs R) {
     constexpr int WZ = NWR * RZ;
-    constexpr bool ADJ = MODE == kResAdjoint;
+    constexpr bool ADJ = MODE == kResAdjoint, QH = OPT && MODE != kResForward, CORNERS = OPT && MODE == kResForward;
     extern __shared__ float4 smem4[];
     __shared__ unsigned s_mask[2];  // rows with injected cells
     const RLayout &Y = R.lay;
@@ -355,6 +358,10 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ S
     // rows of the subdomain above, rows >= rows from the top rows of the one
     // below (a last one of fewer than H rows has no more: zeros), columns left
     // and right from the subdomains of the adjacent columns that hold the row.
+    // The stencil needs no corner; a receiver between the last row and column
+    // and the next ones reads the south-east one (CORNERS). Its subdomain may
+    // share no row or column with this one, so it waits in turn for this one's
+    // corner: neither then overwrites a word that the other has yet to read.
     int xsrc[2] = {-1, -1}, xdst[2] = {0, 0}, xmir[2] = {-1, -1};  // xmir: the float4's place above the free surface
     {
         const int hq = H / 4, nN = hasN ? 32 * H : 0;
@@ -402,8 +409,21 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ S
                 if (top && r >= 1 && r <= H) xmir[v] = xdst[v] - 2 * r * SW;
             }
         }
+        // the corners, by threads whose second float4 is free: the subdomain that
+        // holds one is a neighbour of the one below (south-east) or above (north-west)
+        if (CORNERS && tid >= NTR - 2) {
+            const bool se = tid == NTR - 1;
+            const int via = se ? down : up, z = se ? z0 + rows : z0 - 1;
+            for (int k = 0; via >= 0 && k < R.tiles[via].nnbr; k++) {
+                const int j = R.tiles[via].nbr[k];
+                const RTile &u = R.tiles[j];
+                if (u.bx != (se ? bx + 1 : bx - 1) || z < u.z0 || z >= u.z0 + u.rows) continue;
+                xsrc[1] = (lshot * ntiles + j) * kResidentOutbox + (se ? XWST : XEST + H - 4) + (z - u.z0) * HM;
+                xdst[1] = se ? (HM + rows) * SW + HM + TX : (HM - 1) * SW + HM - 4;
+            }
+        }
     }
-    static_assert(2 * HM * 32 + 2 * 64 * (HM / 4) <= 2 * NTR, "two halo float4s per thread at most");
+    static_assert(2 * HM * 32 + 2 * 64 * (HM / 4) + 2 <= 2 * NTR, "two halo float4s per thread at most");
     const float *const wav = static_cast<const float *>(io->wavelet);
     float *const gout = static_cast<float *>(io->gather);
     float *const snaps = MODE == kResForward ? static_cast<float *>(io->snaps) : nullptr;
@@ -857,7 +877,7 @@ const float4 y4 = ld4(KA + lz * TX + 4 * lane);
     }
 }
 
-template <int RZ, int MODE, bool QH>
+template <int RZ, int MODE, bool OPT>
 cudaError_t launch_rz(const StepArgs<float> &a, const ResidentArgs &r, int nshots, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(r.ntiles * nshots);
@@ -869,13 +889,14 @@ cudaError_t launch_rz(const StepArgs<float> &a, const ResidentArgs &r, int nshot
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_resident2d<RZ, MODE, QH>, a, r);
+    return cudaLaunchKernelEx(&cfg, k_resident2d<RZ, MODE, OPT>, a, r);
 }
 
 template <int RZ>
 cudaError_t launch_mode(const StepArgs<float> &a, const ResidentArgs &r, int mode, int nshots, cudaStream_t st) {
     const bool qh = a.q_fp16 != 0;
-    if (mode == kResForward) return launch_rz<RZ, kResForward, false>(a, r, nshots, st);
+    if (mode == kResForward)
+        return r.corners ? launch_rz<RZ, kResForward, true>(a, r, nshots, st) : launch_rz<RZ, kResForward, false>(a, r, nshots, st);
     if (mode == kResRecord)
         return qh ? launch_rz<RZ, kResRecord, true>(a, r, nshots, st) : launch_rz<RZ, kResRecord, false>(a, r, nshots, st);
     return qh ? launch_rz<RZ, kResAdjoint, true>(a, r, nshots, st) : launch_rz<RZ, kResAdjoint, false>(a, r, nshots, st);
@@ -884,8 +905,8 @@ cudaError_t launch_mode(const StepArgs<float> &a, const ResidentArgs &r, int mod
 template <int RZ>
 cudaError_t configure_rz() {
     cudaError_t e = cudaSuccess;
-    for (auto k : {k_resident2d<RZ, kResForward, false>, k_resident2d<RZ, kResRecord, false>, k_resident2d<RZ, kResRecord, true>,
-                   k_resident2d<RZ, kResAdjoint, false>, k_resident2d<RZ, kResAdjoint, true>})
+    for (auto k : {k_resident2d<RZ, kResForward, false>, k_resident2d<RZ, kResForward, true>, k_resident2d<RZ, kResRecord, false>,
+                   k_resident2d<RZ, kResRecord, true>, k_resident2d<RZ, kResAdjoint, false>, k_resident2d<RZ, kResAdjoint, true>})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentMaxSmem - 64);
     return e;

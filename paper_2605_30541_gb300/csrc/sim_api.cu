@@ -1263,12 +1263,22 @@ const ResidentPlan *plan_resident_gradient(sim_t s, int nshots, int nrec, const 
     return best.rz ? &best : nullptr;
 }
 
+// A receiver of the lists (built on the plan's subdomains) takes a share of the
+// cell past the last row and the last column of its subdomain.
+template <typename T>
+bool corner_receivers(const ResidentPlan &plan, const std::vector<int> &start, const std::vector<RecEntryT<T>> &ent) {
+    for (size_t t = 0; t < plan.tiles.size(); t++)
+        for (int e = start[t]; e < start[t + 1]; e++)
+            if (ent[e].lz == plan.tiles[t].rows - 1 && ent[e].lx == kTileXF - 1 && ent[e].w[3] != T(0)) return true;
+    return false;
+}
+
 // One cooperative launch for the whole time loop, after zeroing the border
 // words; ordered on the handle's stream like any other work.
 template <typename T>
-sim_status run_resident(sim_t s, const StepArgs<T> &a, const ResidentPlan &plan, int nshots);
+sim_status run_resident(sim_t s, const StepArgs<T> &a, const ResidentPlan &plan, int nshots, bool corners);
 template <>
-sim_status run_resident<double>(sim_t s, const StepArgs<double> &, const ResidentPlan &, int) {
+sim_status run_resident<double>(sim_t s, const StepArgs<double> &, const ResidentPlan &, int, bool) {
     return s->fail(SIM_ERR_UNSUPPORTED, "the resident path is FP32 only");
 }
 // no word of an earlier run may carry a tag of this one
@@ -1285,11 +1295,12 @@ ResidentArgs resident_args(sim_t s, const ResidentPlan &plan, int mode) {
     return r;
 }
 template <>
-sim_status run_resident<float>(sim_t s, const StepArgs<float> &a, const ResidentPlan &plan, int nshots) {
+sim_status run_resident<float>(sim_t s, const StepArgs<float> &a, const ResidentPlan &plan, int nshots, bool corners) {
     if (sim_status r = upload(s, s->rtiles, plan.tiles, (size_t)max_tiles(s), "subdomains")) return r;
     ResidentArgs r = resident_args(s, plan, kResForward);
     if (sim_status e = s->cuda(clear_outbox(s, r.ntiles * nshots, s->st), "border words")) return e;
     r.n1 = a.nt;
+    r.corners = corners;
     if (s->d.bc == SIM_BC_CPML)
         for (int k = 0; k < 2; k++) r.m2[k] = a.zeta[k ? 0 : 2];
     return s->cuda(launch_resident2d(a, r, plan.rz, kResForward, nshots, s->st), "resident launch");
@@ -1305,13 +1316,14 @@ struct MapScope {
 // (recording into q when given), or adjoint sweep steps; a launch per group of
 // shots. tag: the next unused tag of this call.
 cudaError_t gradient_run(sim_t s, const StepArgs<float> &a, const ResidentPlan &plan, int mode, int n0, int n1, int nshots,
-                         size_t qstride, unsigned &tag, cudaStream_t st) {
+                         size_t qstride, bool corners, unsigned &tag, cudaStream_t st) {
     ResidentArgs r = resident_args(s, plan, mode);
     r.n0 = n0;
     r.n1 = n1;
     r.load = 1;
     r.store_mem = mode != kResRecord;  // a recorded segment is followed by a restored state
     r.exact_sponge = 1;
+    r.corners = corners && mode == kResForward && a.sample;
     r.q = static_cast<char *>(s->qbuf);
     r.qstride = (long long)qstride;
     if (s->d.bc == SIM_BC_CPML)
@@ -1524,7 +1536,7 @@ sim_status forward_t(sim_t s, int nshots, const void *wavelet, const double *src
     if (rz)
         for (const RTile &t : plan->tiles) s->last_rows = std::max(s->last_rows, t.rows);
     if (rz) {
-        if (sim_status r = run_resident(s, a, *plan, nshots)) return r;
+        if (sim_status r = run_resident(s, a, *plan, nshots, corner_receivers(*plan, rstart, rent))) return r;
     } else if (march) {
         if (sim_status r = run_march(s, a, nshots)) return r;
     } else if (sim_status r = run_graph(s, {kGraphForward, nshots, s->tile_z}, [&](cudaStream_t st) {
@@ -2270,8 +2282,10 @@ sim_status adjoint_t(sim_t s, int nshots, const void *wavelet, const double *src
     }
     const size_t qstride = q_slot_bytes(s, ckpt_fp16);
     GraphKey gkey = {plan ? kGraphResidentGradient : kGraphGradient, nshots, nrec, ckpt_fp16, o.vjp};
+    const bool corners = plan && corner_receivers(*plan, rstart, rent);
     if (plan)  // its subdomains and shared-memory layouts follow from these
-        gkey.insert(gkey.end(), {plan->rz, plan->group, (long long)plan->tiles.size(), plan->lay[kResAdjoint].injr, spin_limit()});
+        gkey.insert(gkey.end(), {plan->rz, plan->group, (long long)plan->tiles.size(), plan->lay[kResAdjoint].injr, corners,
+                                 spin_limit()});
     else
         gkey.push_back(s->tile_z);
     if (sim_status r = run_graph(s, gkey, [&](cudaStream_t st) {
@@ -2285,7 +2299,7 @@ sim_status adjoint_t(sim_t s, int nshots, const void *wavelet, const double *src
                 if (plan) {
                     unsigned tag = 0;
                     auto run = [&](const StepArgs<float> &x, int mode, int n0, int n1) {
-                        return gradient_run(s, x, *plan, mode, n0, n1, nshots, qstride, tag, st);
+                        return gradient_run(s, x, *plan, mode, n0, n1, nshots, qstride, corners, tag, st);
                     };
                     e = clear_outbox(s, (int)plan->tiles.size() * plan->group, st);
                     if (e == cudaSuccess)

@@ -439,6 +439,7 @@ struct ResidentArgs {
     // slots keep a scale per (subdomain, warp) in the top ghost rows of each shot's field
     char *q;
     long long qstride;
+    int corners;  // a receiver reads the cell past a subdomain's last row and column: exchange it
 };
 cudaError_t configure_resident2d();
 bool resident2d_layout(const Geom &g, int bc, int rz, int mode, bool exact_sponge, const std::vector<RTile> &tiles, int injr,
