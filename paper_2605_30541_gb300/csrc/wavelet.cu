@@ -19,8 +19,19 @@
 // dropped at the end. The recursion runs in FP64 as a scan over chunks of
 // the record (k_bandpass_ricker); the result is written in the requested
 // precision.
+//
+// A section's state. In transposed direct form, y = v + z1, z1' = z2 - a1 y,
+// z2' = -v - a2 y, the poles lie within theta = 2 pi f dt of z = 1, z1 and z2
+// nearly cancel, and every rounding grows by 1 / theta^2. With the sum e = z1 +
+// z2, which is small, in place of z2 the same recursion is
+//     y = v + z1,  z1' = k y + (e + v),  e' = e - d y,  k = -(1 + a1),  d = 1 + a1 + a2,
+// whose roundings do not grow (k and d are exact for a1 < -1/2). Sections with
+// a1 > 0, whose poles lie nearer z = -1, take e = z2 - z1 likewise: t is the
+// sign, 1 or -1, in z1' = k y + (e + t v), e' = t e - d y, k = -(t + a1),
+// d = 1 + t a1 + a2.
 #include <cooperative_groups.h>
 
+#include <climits>
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -88,11 +99,17 @@ constexpr int kMaxSections = 16;
 // lower triangular (section i depends on sections j <= i only), block (i, j)
 // at i (i + 1) / 2 + j, its four values row by row.
 //
-// The poles lie close to z = 1, so an error in the map of one chunk is
-// amplified by the powers: formed in FP64 they put 1.5e-11 of the peak into
-// the wavelet (the serial recursion has 1e-13). They are therefore formed in
-// pairs of doubles (an unevaluated sum hi + lo, Dekker's and Knuth's error-free
-// sum and product) and rounded once: 7e-14 .. 1e-13, the serial recursion's.
+// The powers are formed in pairs of doubles (an unevaluated sum hi + lo,
+// Dekker's and Knuth's error-free sum and product) and rounded once: in FP64
+// alone their own errors are several times those of the recursion. Error of the
+// two passes against 113-bit arithmetic with the same coefficients, of the peak
+// (a host model; direct form is the transposed one above):
+//   order, band, dt, samples       | serial, direct | scan, direct | scan, this
+//   4, 3-6 Hz, 1 ms, 8001          | 6e-14          | 2.9e-13      | 5e-16
+//   4, 3-25 Hz, 1 ms, 8001         | 2e-14          | 1.6e-13      | 4e-16
+//   4, 3-6 Hz, 0.1 ms, 40001       | 2.0e-12        | 2.2e-11      | 1.4e-15
+//   12, 3-25 Hz, 1 ms, 8001        | 2.0e-11        | 7.4e-11      | 1.3e-13
+//   16, 3-25 Hz, 1 ms, 8001        | 3.2e-10        | 4.2e-9       | 4e-12
 struct Dd {
     double hi, lo;
 };
@@ -138,11 +155,12 @@ struct Scan {
     static_assert(T == 1 << LEV, "levels of the scan");
     int nsec, C;
     double g;
-    double a1[MAXS], a2[MAXS];
+    double k[MAXS], d[MAXS], t[MAXS];  // a section's k, d and t
+    int flip[MAXS];                    // sign bit of t in the high word
     double P[LEV][MAXS * (MAXS + 1) / 2 * 4];
 };
 
-// map of one sample: v = 0; per section y = v + z1, z1' = z2 - a1 y, z2' = -v - a2 y, v = y
+// map of one sample: the recursion from v = 0; state values (z1, e)
 template <int NS>
 void plan_scan(Scan<NS> &F, int C) {
     const int N = F.nsec;
@@ -153,11 +171,11 @@ void plan_scan(Scan<NS> &F, int C) {
         for (int q = 0; q < 2; q++) {  // column of state value q of section j
             Dd v{0.0, 0.0};
             for (int i = j; i < N; i++) {
-                const Dd z1{i == j && q == 0 ? 1.0 : 0.0, 0.0}, z2{i == j && q == 1 ? 1.0 : 0.0, 0.0};
-                const Dd y = dd_fma({1.0, 0.0}, v, z1);
+                const Dd z1{i == j && q == 0 ? 1.0 : 0.0, 0.0}, e{i == j && q == 1 ? 1.0 : 0.0, 0.0};
+                const Dd y = dd_fma({1.0, 0.0}, v, z1), t{F.t[i], 0.0};
                 Block &b = one[i * (i + 1) / 2 + j];
-                b.v[q] = dd_fma({-F.a1[i], 0.0}, y, z2);
-                b.v[2 + q] = dd_fma({-F.a2[i], 0.0}, y, {-v.hi, -v.lo});
+                b.v[q] = dd_fma({F.k[i], 0.0}, y, dd_fma(t, v, e));
+                b.v[2 + q] = dd_fma({-F.d[i], 0.0}, y, dd_fma(t, e, {0.0, 0.0}));
                 v = y;
             }
         }
@@ -190,8 +208,9 @@ __device__ double ricker_at(double f0, double t) {
 // a sample never leaves its thread until it is written out. What is left is
 // the latency of the FP64 chains (about C samples four times over, 30 chunk
 // maps, C exponentials), which the four warps of each SM overlap: with one
-// warp per SM (256 chunks) the kernel took 167 us, with four 105 us. 8001
-// samples, launch and host plan included: 22.4 ms before, 0.13 ms after.
+// warp per SM (256 chunks) the kernel took 167 us, with four 105 us (both in
+// direct form). 8001 samples, launch and host plan included: 22.4 ms before,
+// 127 us in direct form, 130 us in the form with the sum e.
 template <int NS>
 __global__ void __launch_bounds__(32 * Scan<NS>::WPC) k_bandpass_ricker(const __grid_constant__ Scan<NS> F, int nt,
                                                                             double dt, double f0, int pad, double scale,
@@ -222,12 +241,14 @@ __global__ void __launch_bounds__(32 * Scan<NS>::WPC) k_bandpass_ricker(const __
 
     for (int dir = 1; dir >= -1; dir -= 2) {
         const bool first = m > 0 && (dir > 0 ? t == 0 : j0 + C >= n);
-        double z1[S::MAXS], z2[S::MAXS], s1[S::MAXS], s2[S::MAXS];
+        double z1[S::MAXS], z2[S::MAXS], s1[S::MAXS], s2[S::MAXS];  // z2: the state value e
         auto start = [&]() {  // the first chunk: the steady state of its first sample
 #pragma unroll
             for (int k = 0; k < S::MAXS; k++) {
                 if (NS == 0 && k >= N) break;
-                z1[k] = z2[k] = k == 0 && first ? -F.g * x[(long long)(dir > 0 ? 0 : m - 1) * ld] : 0.0;
+                const double v = k == 0 && first ? F.g * x[(long long)(dir > 0 ? 0 : m - 1) * ld] : 0.0;
+                z1[k] = -v;
+                z2[k] = -v - F.t[k] * v;
             }
         };
         auto run = [&](bool store) {
@@ -237,9 +258,9 @@ __global__ void __launch_bounds__(32 * Scan<NS>::WPC) k_bandpass_ricker(const __
 #pragma unroll
                 for (int k = 0; k < S::MAXS; k++) {
                     if (NS == 0 && k >= N) break;
-                    const double y = v + z1[k];
-                    z1[k] = fma(-F.a1[k], y, z2[k]);
-                    z2[k] = fma(-F.a2[k], y, -v);
+                    const double y = v + z1[k], e = z2[k];
+                    z1[k] = fma(F.k[k], y, fma(F.t[k], v, e));
+                    z2[k] = fma(-F.d[k], y, __hiloint2double(__double2hiint(e) ^ F.flip[k], __double2loint(e)));  // t e
                     v = y;
                 }
                 if (store) *p = v;
@@ -361,8 +382,10 @@ cudaError_t launch_bandpass(const std::vector<Sos> &s, int nt, double dt, double
     F.nsec = (int)s.size();
     F.g = s[0].b0;
     for (int k = 0; k < F.nsec; k++) {
-        F.a1[k] = s[k].a1;
-        F.a2[k] = s[k].a2;
+        F.t[k] = s[k].a1 <= 0.0 ? 1.0 : -1.0;
+        F.flip[k] = s[k].a1 <= 0.0 ? 0 : INT_MIN;
+        F.k[k] = -(F.t[k] + s[k].a1);
+        F.d[k] = (1.0 + F.t[k] * s[k].a1) + s[k].a2;
     }
     const long long n = nt + 2LL * pad;
     plan_scan<NS>(F, (int)((n + S::T - 1) / S::T));
