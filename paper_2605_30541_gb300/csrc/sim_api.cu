@@ -1226,7 +1226,7 @@ bool resident_gradient_faster(const sim_s *s, int nshots, const ResidentPlan &p)
 // The gradient's plan: shots in as few launches (groups) per run of steps as
 // are fastest by the cost model.
 const ResidentPlan *plan_resident_gradient(sim_t s, int nshots, int nrec, const double *rec_pos, bool q_fp16) {
-    if (!resident_enabled(s) || s->plan.L < 2) return nullptr;  // the adjoint's in-place fields: sim_internal.h
+    if (!resident_enabled(s) || s->plan.L < 2) return nullptr;  // runs of two steps and more: gradient_run
     const Geom &g = s->g;
     // rows of a column that receivers inject into, at most
     std::vector<char> seen((size_t)((g.NX + kTileXF - 1) / kTileXF) * g.NZ, 0);
@@ -1314,9 +1314,15 @@ struct MapScope {
 
 // A run of steps of the gradient: forward from the state in the global fields
 // (recording into q when given), or adjoint sweep steps; a launch per group of
-// shots. tag: the next unused tag of this call.
+// shots. tag: the next unused tag of this call. The adjoint's mu is loaded with
+// a ring of the neighbours' cells and stored in place (as u is): in a run of two
+// steps and more a subdomain stores after a wait for words that each neighbour
+// sends after its loads. Nothing orders the two in a run of one step, which is
+// therefore taken only first in the sweep, where u, nu and mu are zero before
+// and after.
 cudaError_t gradient_run(sim_t s, const StepArgs<float> &a, const ResidentPlan &plan, int mode, int n0, int n1, int nshots,
                          size_t qstride, bool corners, unsigned &tag, cudaStream_t st) {
+    if (mode == kResAdjoint && n1 - n0 < 2 && n0 != 0) return cudaErrorInvalidValue;
     ResidentArgs r = resident_args(s, plan, mode);
     r.n0 = n0;
     r.n1 = n1;
