@@ -125,7 +125,9 @@ typedef struct {
     int adj_inner;            /* m: innermost segments per top segment (1 with one level) */
     int adj_top;              /* top-level checkpoints, every m L steps */
     int adj_sub;              /* second-level checkpoint slots */
-    int pad1;
+    int adj_path;             /* how the last sim_adjoint ran its steps: 0 none yet, 1 launches per step,
+                                 2 resident: runs of steps between checkpoints in one launch each
+                                 (2D FP32 shots that fit on the GPU), 3 the 3D path */
     size_t adj_bytes;         /* device memory of the gradient's buffers */
     int z_variant;            /* 3D: staging of the z-march (1 per-thread cp.async copies, 6 TMA copies) */
     int z_chunk;              /* 3D: planes per CTA of the z-march */

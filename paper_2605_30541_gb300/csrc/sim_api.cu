@@ -294,7 +294,7 @@ struct sim_s {
     long long march_key = -1;              // (shot count, item rows, tile height) of the plan on the device
     int march_nwarps = 0, march_nitems = 0;
     unsigned *mctr = nullptr;              // row march: per-step item counters
-    int last_path = 0, last_rows = 0;      // see sim_info
+    int last_path = 0, last_rows = 0, adj_path = 0;  // see sim_info
     ZShape zshape;                         // z-march variant, tile and chunk, see autotune3d
     int batch_sched = 0, batch_tile = 0;   // schedule and tile of the last batch forward (as sim_info)
     void *pbuf3 = nullptr;                 // two-step row march: third and fourth pressure fields (max_shots shots each)
@@ -2056,6 +2056,7 @@ sim_status adjoint3d(sim_t s, int nshots, const void *wavelet, const double *src
     const sim_desc &d = s->d;
     const Geom &g = s->g;
     if (sim_status r = ensure_adjoint(s, ckpt_fp16)) return r;
+    s->adj_path = 3;
     const size_t nt = d.nt;
     const int ms = d.max_shots;
     const long long nint = (long long)g.nz * g.ny * g.nx;
@@ -2191,6 +2192,7 @@ sim_status adjoint_t(sim_t s, int nshots, const void *wavelet, const double *src
         std::is_same<T, float>::value ? plan_resident_gradient(s, nshots, nrec, rec_pos, ckpt_fp16 != 0) : nullptr;
     if (!plan)
         if (sim_status r = autotune(s, nshots)) return r;
+    s->adj_path = plan ? 2 : 1;
     MapScope map_scope{s};
     s->tmap = plan ? &plan->map : nullptr;
     const size_t nt = d.nt;
@@ -3220,6 +3222,7 @@ sim_status sim_get_info(sim_t s, sim_info *out) {
     out->tile_z = s->tile_z;
     out->last_path = s->last_path;
     out->last_rows = s->last_rows;
+    out->adj_path = s->adj_path;
     out->vmin = s->vmin;
     out->vmax = s->vmax;
     out->courant = s->vmax * s->d.dt / s->d.h;
