@@ -9,28 +9,46 @@
 // low-pass to band-pass map around w0 = sqrt(w_lo w_hi) with bandwidth
 // w_hi - w_lo (edges prewarped, w = 2 fs tan(pi f / fs)), then the bilinear
 // map z = (2 fs + s) / (2 fs - s), grouped into second-order sections (each
-// a conjugate pole pair with two zeros; gain on the first section).
+// a conjugate pole pair with two zeros; gain on the first section). The half of
+// the pairs with the lower frequencies takes the zeros at z = 1, two each, the
+// other half those at z = -1 (an odd order's middle pair one of each), low ones
+// first: high-passes, then low-passes.
 // Forward-backward filtering follows the usual zero-phase recipe: the signal
 // is extended at both ends by its odd reflection about the end samples
 // (3 (2 S + 1) samples for S sections; the record must be longer than that),
 // each pass starts every section in the steady state of a constant input
-// equal to the first sample it sees (a band-pass section passes no constant,
-// so only the first section has a state to start from), and the extension is
+// equal to the first sample it sees (the first section passes no constant, so
+// only it has a state to start from), and the extension is
 // dropped at the end. The recursion runs in FP64 as a scan over chunks of
 // the record (k_bandpass_ricker); the result is written in the requested
 // precision.
 //
-// A section's state. In transposed direct form, y = v + z1, z1' = z2 - a1 y,
-// z2' = -v - a2 y, the poles lie within theta = 2 pi f dt of z = 1, z1 and z2
-// nearly cancel, and every rounding grows by 1 / theta^2. With the sum e = z1 +
-// z2, which is small, in place of z2 the same recursion is
-//     y = v + z1,  z1' = k y + (e + v),  e' = e - d y,  k = -(1 + a1),  d = 1 + a1 + a2,
-// whose roundings do not grow (k and d are exact for a1 < -1/2). Sections with
-// a1 > 0, whose poles lie nearer z = -1, take e = z2 - z1 likewise: t is the
-// sign, 1 or -1, in z1' = k y + (e + t v), e' = t e - d y, k = -(t + a1),
-// d = 1 + t a1 + a2.
+// What keeps the rounding small. With a zero at 1 and one at -1 in every section
+// the low ones answer a step, such as the start of a chunk, by 1 / theta each
+// (theta = 2 pi f dt), which a wide band's other sections do not undo: the
+// chunks' shares of a state then cancel to a small part of themselves. As
+// high-passes and low-passes they answer by no more than they pass. And a
+// section in transposed direct form, y = v + z1, z1' = z2 + b1 v - a1 y,
+// z2' = b2 v - a2 y, whose poles lie within theta of z = 1, has z1 and z2 that
+// nearly cancel: every rounding grows by 1 / theta^2. With e = z2 + t z1 in place
+// of z2, t = 1 (a1 <= 0) or -1 (poles nearer z = -1), the same recursion is
+//     y = v + z1,  z1' = k y + (p v + e),  e' = q v + t e - d y,
+//     k = -(t + a1),  d = 1 + t a1 + a2,  p = t + b1,  q = 1 + t b1 + b2
+// (p = -1, 1, 3 or -3; q = 0 or 4; k and d exact for |a1| > 1/2), whose
+// roundings do not grow. Error of the two passes against 113-bit arithmetic with
+// the same coefficients, of the peak (a host model; the first two columns in
+// direct form with zeros at 1 and -1 in every section):
+//   order, band, dt, samples      | serial  | scan    | scan, this form
+//   4, 3-6 Hz, 1 ms, 8001         | 6e-14   | 2.9e-13 | 5e-15
+//   4, 3-25 Hz, 1 ms, 8001        | 2e-14   | 1.6e-13 | 1e-15
+//   4, 3-6 Hz, 0.1 ms, 40001      | 2.0e-12 | 2.2e-11 | 1.9e-14
+//   4, 2-1500 Hz, 0.25 ms, 4777   | 8e-13   | 1.6e-11 | 1.5e-15
+//   8, 2-1500 Hz, 0.25 ms, 4777   | 5e-10   | 3.5e-6  | 2e-15
+//   16, 3-25 Hz, 1 ms, 8001       | 3.2e-10 | 4.2e-9  | 3e-15
+//   16, 5-400 Hz, 1 ms, 4000      | 2.8e-5  | > 1     | 1.5e-15
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <complex>
@@ -44,7 +62,7 @@ namespace {
 using cd = std::complex<double>;
 
 struct Sos {
-    double b0, b1, b2, a1, a2;  // a0 = 1
+    double b0, b1, b2, a1, a2;  // b0 (1 + b1 z^-1 + b2 z^-2) / (1 + a1 z^-1 + a2 z^-2)
 };
 
 // Digital Butterworth band-pass of order N (2N poles) at [f_lo, f_hi], fs = 1/dt.
@@ -67,26 +85,27 @@ std::vector<Sos> butter_bandpass(int N, double f_lo, double f_hi, double fs) {
         gain /= (2.0 * fs - p);
     }
     gain *= std::pow(2.0 * fs, N);  // prod over the N finite zeros (s = 0) of (2 fs - 0)
-    // zeros: N at z = 1 (from s = 0), N at z = -1 (from s = infinity)
-    // sections: conjugate pairs of poles (upper half plane ones), zeros (1, -1) each
+    // zeros: N at z = 1 (from s = 0), N at z = -1 (from s = infinity);
+    // sections: conjugate pairs of poles (upper half plane ones)
     std::vector<cd> up;
     for (const cd &z : zp)
         if (z.imag() > 0) up.push_back(z);
+    std::sort(up.begin(), up.end(), [](const cd &a, const cd &b) { return std::arg(a) < std::arg(b); });
+    const int n = (int)up.size(), half = n / 2;
+    // within a kind the sharpest first (of the orders tried the smallest error)
+    auto sharp = [](const cd &a, const cd &b) { return std::norm(a) > std::norm(b); };
+    std::sort(up.begin(), up.begin() + half, sharp);
+    std::sort(up.end() - half, up.end(), sharp);
     std::vector<Sos> s;
-    for (size_t i = 0; i < up.size(); i++) {
+    for (int i = 0; i < n; i++) {
         Sos q{};
-        q.b0 = 1.0;
-        q.b1 = 0.0;  // (z - 1)(z + 1) = z^2 - 1
-        q.b2 = -1.0;
+        q.b0 = i == 0 ? gain.real() : 1.0;
+        q.b1 = i < half ? -2.0 : (i >= n - half ? 2.0 : 0.0);
+        q.b2 = i < half || i >= n - half ? 1.0 : -1.0;
         q.a1 = -2.0 * up[i].real();
         q.a2 = std::norm(up[i]);
         s.push_back(q);
     }
-    if (s.empty()) return s;
-    const double g = gain.real();
-    s[0].b0 *= g;
-    s[0].b1 *= g;
-    s[0].b2 *= g;
     return s;
 }
 
@@ -98,31 +117,8 @@ constexpr int kMaxSections = 16;
 // section) linearly; P[l] is that map over 2^l chunks of C samples, block
 // lower triangular (section i depends on sections j <= i only), block (i, j)
 // at i (i + 1) / 2 + j, its four values row by row.
-//
-// The powers are formed in pairs of doubles (an unevaluated sum hi + lo,
-// Dekker's and Knuth's error-free sum and product) and rounded once: in FP64
-// alone their own errors are several times those of the recursion. Error of the
-// two passes against 113-bit arithmetic with the same coefficients, of the peak
-// (a host model; direct form is the transposed one above):
-//   order, band, dt, samples       | serial, direct | scan, direct | scan, this
-//   4, 3-6 Hz, 1 ms, 8001          | 6e-14          | 2.9e-13      | 5e-16
-//   4, 3-25 Hz, 1 ms, 8001         | 2e-14          | 1.6e-13      | 4e-16
-//   4, 3-6 Hz, 0.1 ms, 40001       | 2.0e-12        | 2.2e-11      | 1.4e-15
-//   12, 3-25 Hz, 1 ms, 8001        | 2.0e-11        | 7.4e-11      | 1.3e-13
-//   16, 3-25 Hz, 1 ms, 8001        | 3.2e-10        | 4.2e-9       | 4e-12
-struct Dd {
-    double hi, lo;
-};
-Dd dd_fma(const Dd &a, const Dd &b, const Dd &c) {  // a b + c
-    const volatile double prod = a.hi * b.hi;  // volatile: the compiler may not fuse it into the sum below
-    const double p = prod, pe = std::fma(a.hi, b.hi, -p) + (a.hi * b.lo + a.lo * b.hi);
-    const double s = p + c.hi, t = s - p;
-    const double se = ((p - (s - t)) + (c.hi - t)) + (pe + c.lo);
-    const double h = s + se;
-    return {h, se - (h - s)};
-}
 struct Block {
-    Dd v[4];
+    double v[4];
 };
 using Tri = std::vector<Block>;  // N (N + 1) / 2 blocks
 
@@ -135,7 +131,7 @@ Tri tri_mul(const Tri &a, const Tri &b, int N) {
                 const Block &x = a[i * (i + 1) / 2 + k], &y = b[k * (k + 1) / 2 + j];
                 for (int p = 0; p < 2; p++)
                     for (int q = 0; q < 2; q++)
-                        o.v[2 * p + q] = dd_fma(x.v[2 * p + 1], y.v[2 + q], dd_fma(x.v[2 * p], y.v[q], o.v[2 * p + q]));
+                        o.v[2 * p + q] = std::fma(x.v[2 * p + 1], y.v[2 + q], std::fma(x.v[2 * p], y.v[q], o.v[2 * p + q]));
             }
             r[i * (i + 1) / 2 + j] = o;
         }
@@ -155,8 +151,9 @@ struct Scan {
     static_assert(T == 1 << LEV, "levels of the scan");
     int nsec, C;
     double g;
-    double k[MAXS], d[MAXS], t[MAXS];  // a section's k, d and t
-    int flip[MAXS];                    // sign bit of t in the high word
+    double k[MAXS], d[MAXS], p[MAXS], q[MAXS];  // a section's constants
+    int flip[MAXS];                             // sign bit of its t in the high word
+    double e0;                                  // first section's e at rest under a unit input
     double P[LEV][MAXS * (MAXS + 1) / 2 * 4];
 };
 
@@ -166,16 +163,15 @@ void plan_scan(Scan<NS> &F, int C) {
     const int N = F.nsec;
     F.C = C;
     Tri one((size_t)N * (N + 1) / 2), m = one;
-    for (int k = 0; k < N; k++) m[k * (k + 1) / 2 + k].v[0].hi = m[k * (k + 1) / 2 + k].v[3].hi = 1.0;
+    for (int k = 0; k < N; k++) m[k * (k + 1) / 2 + k].v[0] = m[k * (k + 1) / 2 + k].v[3] = 1.0;
     for (int j = 0; j < N; j++)
-        for (int q = 0; q < 2; q++) {  // column of state value q of section j
-            Dd v{0.0, 0.0};
+        for (int c = 0; c < 2; c++) {  // column of state value c of section j
+            double v = 0.0;
             for (int i = j; i < N; i++) {
-                const Dd z1{i == j && q == 0 ? 1.0 : 0.0, 0.0}, e{i == j && q == 1 ? 1.0 : 0.0, 0.0};
-                const Dd y = dd_fma({1.0, 0.0}, v, z1), t{F.t[i], 0.0};
+                const double z1 = i == j && c == 0 ? 1.0 : 0.0, e = i == j && c == 1 ? 1.0 : 0.0, y = v + z1;
                 Block &b = one[i * (i + 1) / 2 + j];
-                b.v[q] = dd_fma({F.k[i], 0.0}, y, dd_fma(t, v, e));
-                b.v[2 + q] = dd_fma({-F.d[i], 0.0}, y, dd_fma(t, e, {0.0, 0.0}));
+                b.v[c] = std::fma(F.k[i], y, std::fma(F.p[i], v, e));
+                b.v[2 + c] = std::fma(-F.d[i], y, std::fma(F.q[i], v, F.flip[i] ? -e : e));
                 v = y;
             }
         }
@@ -185,7 +181,7 @@ void plan_scan(Scan<NS> &F, int C) {
     }
     for (int l = 0; l < Scan<NS>::LEV; l++) {
         for (size_t b = 0; b < m.size(); b++)
-            for (int q = 0; q < 4; q++) F.P[l][4 * b + q] = m[b].v[q].hi;
+            for (int q = 0; q < 4; q++) F.P[l][4 * b + q] = m[b].v[q];
         if (l + 1 < Scan<NS>::LEV) m = tri_mul(m, m, N);
     }
 }
@@ -210,7 +206,7 @@ __device__ double ricker_at(double f0, double t) {
 // maps, C exponentials), which the four warps of each SM overlap: with one
 // warp per SM (256 chunks) the kernel took 167 us, with four 105 us (both in
 // direct form). 8001 samples, launch and host plan included: 22.4 ms before,
-// 127 us in direct form, 130 us in the form with the sum e.
+// 128 us in direct form, 134 us in the present form.
 template <int NS>
 __global__ void __launch_bounds__(32 * Scan<NS>::WPC) k_bandpass_ricker(const __grid_constant__ Scan<NS> F, int nt,
                                                                             double dt, double f0, int pad, double scale,
@@ -248,7 +244,7 @@ __global__ void __launch_bounds__(32 * Scan<NS>::WPC) k_bandpass_ricker(const __
                 if (NS == 0 && k >= N) break;
                 const double v = k == 0 && first ? F.g * x[(long long)(dir > 0 ? 0 : m - 1) * ld] : 0.0;
                 z1[k] = -v;
-                z2[k] = -v - F.t[k] * v;
+                z2[k] = F.e0 * v;
             }
         };
         auto run = [&](bool store) {
@@ -259,8 +255,10 @@ __global__ void __launch_bounds__(32 * Scan<NS>::WPC) k_bandpass_ricker(const __
                 for (int k = 0; k < S::MAXS; k++) {
                     if (NS == 0 && k >= N) break;
                     const double y = v + z1[k], e = z2[k];
-                    z1[k] = fma(F.k[k], y, fma(F.t[k], v, e));
-                    z2[k] = fma(-F.d[k], y, __hiloint2double(__double2hiint(e) ^ F.flip[k], __double2loint(e)));  // t e
+                    z1[k] = fma(F.k[k], y, fma(F.p[k], v, e));
+                    double u = __hiloint2double(__double2hiint(e) ^ F.flip[k], __double2loint(e));  // t e
+                    if (F.q[k] != 0.0) u = fma(F.q[k], v, u);
+                    z2[k] = fma(-F.d[k], y, u);
                     v = y;
                 }
                 if (store) *p = v;
@@ -382,10 +380,13 @@ cudaError_t launch_bandpass(const std::vector<Sos> &s, int nt, double dt, double
     F.nsec = (int)s.size();
     F.g = s[0].b0;
     for (int k = 0; k < F.nsec; k++) {
-        F.t[k] = s[k].a1 <= 0.0 ? 1.0 : -1.0;
-        F.flip[k] = s[k].a1 <= 0.0 ? 0 : INT_MIN;
-        F.k[k] = -(F.t[k] + s[k].a1);
-        F.d[k] = (1.0 + F.t[k] * s[k].a1) + s[k].a2;
+        const double t = s[k].a1 <= 0.0 ? 1.0 : -1.0;
+        F.flip[k] = t > 0.0 ? 0 : INT_MIN;
+        F.k[k] = -(t + s[k].a1);
+        F.d[k] = (1.0 + t * s[k].a1) + s[k].a2;
+        F.p[k] = t + s[k].b1;
+        F.q[k] = 1.0 + t * s[k].b1 + s[k].b2;
+        if (k == 0) F.e0 = s[k].b2 - t;
     }
     const long long n = nt + 2LL * pad;
     plan_scan<NS>(F, (int)((n + S::T - 1) / S::T));

@@ -1,8 +1,11 @@
 """Rounding error of the FP64 band-passed wavelet (csrc/wavelet.cu): against the
 same definition in extended precision (numpy's long double) with the library's
 own FP64 coefficients, the scan is no further off than the plain FP64 recursion
-in transposed direct form, one sample after another. The coefficients come from
-the library's source, compiled here with a small wrapper."""
+in transposed direct form with a zero at 1 and one at -1 in every section, one
+sample after another: the production bands, finer time steps, other orders and
+bands over several octaves; and it stays within 1e-13 of the peak (a host model
+of it has at most 2.4e-14). The coefficients come from the library's source,
+compiled here with a small wrapper."""
 import ctypes
 import os
 import subprocess
@@ -73,7 +76,10 @@ def wavelet(T, order, lo, hi, f0, dt, nt, coef):
 
 @pytest.mark.parametrize("order,lo,hi,f0,dt,nt", [(4, *b, 1e-3, 8001) for b in W.BANDS] +
                          [(4, 3.0, 6.0, 4.5, 2.5e-4, 16001), (4, 3.0, 6.0, 4.5, 1e-4, 40001), (4, 5.0, 200.0, 80.0, 1e-3, 3001),
-                          (2, 3.0, 12.0, 7.5, 1e-3, 8001), (8, 3.0, 12.0, 7.5, 1e-3, 8001), (12, 3.0, 25.0, 14.0, 1e-3, 8001)])
+                          (2, 3.0, 12.0, 7.5, 1e-3, 8001), (8, 3.0, 12.0, 7.5, 1e-3, 8001), (12, 3.0, 25.0, 14.0, 1e-3, 8001),
+                          (16, 3.0, 25.0, 14.0, 1e-3, 8001), (4, 2.0, 1500.0, 10.0, 2.5e-4, 4777),
+                          (8, 2.0, 1500.0, 10.0, 2.5e-4, 4777), (16, 5.0, 400.0, 20.0, 1e-3, 4000), (3, 3.0, 15.0, 8.0, 2.5e-4, 3001),
+                          (5, 100.0, 180.0, 140.0, 1e-3, 2000), (1, 3.0, 12.0, 7.5, 1e-3, 1001)])
 def test_no_further_off_than_the_plain_recursion(pkg, design, order, lo, hi, f0, dt, nt):
     coef = design(order, lo, hi, 1.0 / dt)
     ref = wavelet(np.longdouble, order, lo, hi, f0, dt, nt, coef)
@@ -82,4 +88,4 @@ def test_no_further_off_than_the_plain_recursion(pkg, design, order, lo, hi, f0,
     peak = np.abs(ref).max()
     e, e0 = float(np.abs(g - ref).max() / peak), float(np.abs(plain - ref).max() / peak)
     print("order %d %g-%g Hz dt %g nt %d: plain %.1e scan %.1e" % (order, lo, hi, dt, nt, e0, e))
-    assert e <= e0
+    assert e <= min(e0, 1e-13)
