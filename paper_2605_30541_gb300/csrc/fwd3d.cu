@@ -1,12 +1,15 @@
 // 3D time step of the acoustic scheme (FP32).
 //
 // Main kernel: a z-march over (x, y) tiles (2.5D blocking). A CTA of 8 warps
-// owns a 128 x TY column of the grid (TY = 8 RY); each lane owns 4
-// consecutive x cells in RY y-rows and keeps the 9 planes z-4 .. z+4 of those
-// cells in a register queue, so p^n is read from memory once per cell for the
-// z-derivative. The planes with their radius-4 x/y halo are staged into a
-// shared-memory ring ahead of use: by per-thread cp.async copies (k_step3d)
-// or by tensor-memory-accelerator copies that one thread issues (k_step3d_tma). The update is the leapfrog step with the
+// owns a column of 1024 cells of the grid, 64 x 16 or 32 x 32 where the planes
+// are staged by tensor-memory-accelerator copies that one thread issues
+// (k_step3d_tma, the only form that runs unasked) and 128 x 8 where every
+// thread copies its share by cp.async (k_step3d, which GSIM_ZMARCH=async selects:
+// the form the tests compare the other with). Each thread owns 4 consecutive x
+// cells of a row and keeps the 9 planes z-4 .. z+4 of those cells in a register
+// queue, so p^n is read from memory once per cell for the z-derivative. The
+// planes with their radius-4 x/y halo are staged into a shared-memory ring
+// ahead of use. The update is the leapfrog step with the
 // centred sponge term (Eq. cerjan_pde), the free-surface plane z = 0 held at
 // zero with an odd mirror above it (Eq. free_surface), and no boundary
 // arithmetic outside absorbing tiles.

@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(NTR, 1) k_resident2d(const __grid_constant__ S
                 for (int k = 0; k < 4; k++) qk[k] = 0.f * (res[k] - lane_of(pp4, k)) - rhs[k];
             } else if (R.exact_sponge) {
                 const float ez = CAZ[lz + 8];
-const float4 y4 = ld4(KA + lz * TX + 4 * lane);
+                const float4 y4 = ld4(KA + lz * TX + 4 * lane);
                 const float2 one = splat2(1.f), two = splat2(2.f), ea = add2(splat2(ez), lo2(E4)), eb = add2(splat2(ez), hi2(E4));
                 const float2 ta = fma2(lo2(c4), ra, fma2(neg2(fma2(neg2(lo2(c4)), ea, one)), lo2(pp4), mul2(two, lo2(C))));
                 const float2 tb = fma2(hi2(c4), rbb, fma2(neg2(fma2(neg2(hi2(c4)), eb, one)), hi2(pp4), mul2(two, hi2(C))));
@@ -755,7 +755,7 @@ const float4 y4 = ld4(KA + lz * TX + 4 * lane);
         }
         // Borders of tall subdomains, from the rows just written: few instances of
         // the sending code for the instruction cache, and the side columns of all
-        // rows at once (with 4 rows per warp a gradient of 16 shots 22.35 -> 21.76
+        // rows at once (with 4 rows per warp a gradient of 16 shots 22.32 -> 21.49
         // ms, with 3 a slice 4.03 -> 4.01; with 1 or 2 rows, where a send per row
         // in place starts earlier, 2.84 -> 2.90 and 6.13 -> 6.17)
         if (RZ >= 3 && n + 1 < R.n1) {
